@@ -375,3 +375,65 @@ def test_tensor_core_layers_close_to_rounded_oracle(ctx, oracle, shape):
     net.close()
     assert np.max(np.abs(got - ref)) <= 2e-2 * np.max(np.abs(ref))
     assert np.corrcoef(got.ravel(), ref.ravel())[0, 1] > 0.999
+
+
+def _pass_through_params(channel):
+    """Parameters that hand input channel `channel` (positive) through the centre taps unchanged."""
+    p = np.zeros(32 * 2 * 9 + 32 + 2 * (32 * 32 * 9 + 32) + 32 * 9 + 1, dtype=np.float32)
+    at = 0
+    for layer, (ci, co) in enumerate(((2, 32), (32, 32), (32, 32), (32, 1))):
+        p[at + (channel if layer == 0 else 0) * 9 + 4] = 1.0
+        at += co * ci * 9 + co
+    return p
+
+
+@pytest.mark.parametrize("F,shape", [(1, (2, 5, 7)), (2, (1, 6, 258)), (3, (2, 9, 771)), (5, (1, 35, 45)),
+                                     (8, (2, 136, 72)), (16, (1, 48, 272)), (31, (1, 62, 93)), (32, (1, 64, 96))])
+@pytest.mark.parametrize("channel", [0, 1])
+def test_pooling_and_interpolation(ctx, F, shape, channel):
+    """Block means of log k and f, and the interpolation back, through a network
+    that passes one channel on.  Both sides round a mean to fp32 once (half an
+    ulp, 2^-24 each); everything else is fp64."""
+    from paper_2204_02064_gb300 import api
+    nimg, ny, nx = shape
+    n = nimg * ny * nx
+    k = np.exp(40.0 * inputs.uniform(61, n)).reshape(shape)   # logs 0..40: the exponents' sum carries the mean
+    f = 1.0 + inputs.uniform(62, n).reshape(shape)
+    net = api.WarmNet(ctx, storage=api.F32, dilations=DIL, seed=1, pool=F)
+    net.params = _pass_through_params(channel)
+    net.scale = 2.0
+    ref = _bilinear(_pool(np.log(k) if channel == 0 else f, F), F) * 2.0
+    # u at an odd offset too: rows that 16-byte stores cannot write
+    for off in (0, 1):
+        flat = torch.full((n + 1 + off,), -7.0, dtype=torch.float64, device="cuda")
+        u = flat[off:off + n].reshape(shape)
+        net.predict(_dev(k), _dev(f), u)
+        torch.cuda.synchronize()
+        assert np.max(np.abs(u.cpu().numpy() - ref)) <= 2.0 ** -22 * np.max(np.abs(ref))
+        assert bool((flat[off + n:] == -7.0).all()) and bool((flat[:off] == -7.0).all())
+
+
+@pytest.mark.parametrize("F", [1, 4])
+@pytest.mark.parametrize("value", [5e-324, 1e-310, 2.2250738585072014e-308, 1.7e308])
+def test_log_of_extreme_coefficients(ctx, F, value):
+    """A subnormal, the smallest normal and a huge coefficient: the mean log of their coarse cell, from a
+    network that subtracts ReLU(-x) from ReLU(x) (fp32 rounding of a mean, as above)."""
+    from paper_2204_02064_gb300 import api
+    ny, nx = 4 * F, 8 * F
+    k = np.full((1, ny, nx), np.e)
+    k[0, F, 3 * F - 1] = value
+    net = api.WarmNet(ctx, storage=api.F32, dilations=DIL, seed=1, pool=F)
+    p = _pass_through_params(0)
+    p[2 * 9 + 4] = -1.0
+    a1 = 32 * 2 * 9 + 32
+    p[a1 + (32 + 1) * 9 + 4] = 1.0
+    a2 = a1 + 32 * 32 * 9 + 32
+    p[a2 + (32 + 1) * 9 + 4] = 1.0
+    p[a2 + 32 * 32 * 9 + 32 + 9 + 4] = -1.0
+    net.params = p
+    net.scale = 1.0
+    u = torch.zeros((1, ny, nx), dtype=torch.float64, device="cuda")
+    net.predict(_dev(k), _dev(np.zeros_like(k)), u)
+    torch.cuda.synchronize()
+    ref = _bilinear(_pool(np.log(k), F), F)
+    assert np.max(np.abs(u.cpu().numpy() - ref)) <= 2.0 ** -22 * np.max(np.abs(ref))
