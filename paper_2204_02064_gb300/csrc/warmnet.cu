@@ -6,10 +6,10 @@
 // Layers: conv(2->C) ReLU, conv(C->C) ReLU, conv(C->C) ReLU, conv(C->1);
 // dilation per layer; zero padding.  Activations are stored in bf16 (or
 // fp32), every product is accumulated in fp32, master weights are fp32.
-// Backward through a layer: the input gradient is the same direct
-// convolution with the weights flipped and transposed, masked by the ReLU of
-// the forward activation; the weight gradient accumulates, per block, over a
-// strided set of pixel tiles in registers before one atomic add per weight.
+// Backward through a layer: the input gradient is a direct convolution with
+// the weights flipped and transposed, masked by the ReLU of the forward
+// activation; the weight gradient accumulates, per block, over a strided set
+// of pixel tiles in registers, and a last kernel adds the blocks' sums.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -32,120 +32,493 @@ template <typename S> __device__ __forceinline__ float ld_f(const S *p) { return
 template <> __device__ __forceinline__ float ld_f<float>(const float *p) { return *p; }
 template <typename S> __device__ __forceinline__ S st_f(float v) { return from_acc<S>(v); }
 template <> __device__ __forceinline__ float st_f<float>(float v) { return v; }
+// 16 bytes of a pixel's channels
+template <typename S> struct alignas(16) VecC {
+    static constexpr int N = 16 / sizeof(S);
+    S v[N];
+};
 
-// out[img][co][y][x] = bias[co] + sum_ci sum_tap W'[ci][tap][co] in[img][ci][y+dy][x+dx]
-// W' is gathered from the layer weights w[cout_l][cin_l][9]:
-//   TRANSPOSE = false: W'[ci][tap][co] = w[co][ci][tap]        (forward)
-//   TRANSPOSE = true : W'[ci][tap][co] = w[ci][co][8 - tap]    (input gradient)
-// Epilogue: RELU -> max(0, .); MASK -> multiply by (mask[img][co][p] > 0).
-template <typename SI, typename SO, int CIN, int COUT, bool TRANSPOSE, bool RELU, bool MASK, typename SM>
-__global__ void __launch_bounds__(kConvThreads) conv_kernel(const SI *__restrict__ in, const float *__restrict__ w,
-                                                          const float *__restrict__ bias, SO *__restrict__ out,
-                                                          const SM *__restrict__ mask, int H, int W, int dil,
-                                                          int tiles_x, int tiles_y) {
-    extern __shared__ __align__(16) float smem[];
-    const int halo = dil;
-    const int TW = kTile + 2 * halo;
-    float *s_w = smem;                           // CIN * 9 * COUT
-    float *s_in = smem + CIN * 9 * COUT;         // CIN * TW * TW
-    const int tile = blockIdx.x;
-    const int img = blockIdx.y;
-    const int tx0 = (tile % tiles_x) * kTile, ty0 = (tile / tiles_x) * kTile;
-    for (int e = threadIdx.x; e < CIN * 9 * COUT; e += blockDim.x) {
-        const int co = e % COUT, tap = (e / COUT) % 9, ci = e / (9 * COUT);
-        s_w[e] = TRANSPOSE ? w[(ci * COUT + co) * 9 + (8 - tap)] : w[(co * CIN + ci) * 9 + tap];
-    }
-    const long long plane = (long long)H * W;
-    const SI *inb = in + (long long)img * CIN * plane;
-    for (int e = threadIdx.x; e < CIN * TW * TW; e += blockDim.x) {
-        const int xx = e % TW, yy = (e / TW) % TW, ci = e / (TW * TW);
-        const int gx = tx0 + xx - halo, gy = ty0 + yy - halo;
-        s_in[e] = (gx >= 0 && gx < W && gy >= 0 && gy < H) ? ld_f(inb + ci * plane + (long long)gy * W + gx) : 0.f;
-    }
+// Activations of the hidden layers are NHWC ([img][y][x][32]), so a pixel's
+// channels are one 64- or 128-byte run; the two input channels and the output
+// are planes.
+
+// First layer, 2 -> 32 channels: one thread per pixel, all 32 outputs in
+// registers, weights [ci][tap][co] in shared memory (read by broadcast).
+// x1[p][co] = relu(bias[co] + sum_ci sum_tap w[co][ci][tap] x0[ci][p + off])
+template <typename S>
+__global__ void __launch_bounds__(256, 2) conv_first_kernel(const S *__restrict__ x0, const float *__restrict__ w,
+                                                         const float *__restrict__ bias, S *__restrict__ x1, int nimg,
+                                                         int H, int W, int dil) {
+    __shared__ __align__(16) float s_w[18 * kMaxC];
+    for (int e = threadIdx.x; e < 18 * kMaxC; e += blockDim.x) s_w[e] = w[(e % kMaxC) * 18 + e / kMaxC];
     __syncthreads();
-    const int lx = threadIdx.x % kTile, ly = threadIdx.x / kTile;
-    const int gx = tx0 + lx, gy = ty0 + ly;
-    float acc[COUT];
+    const long long plane = (long long)H * W, total = plane * nimg;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long img = i / plane;
+        const int p = (int)(i - img * plane), y = p / W, x = p % W;
+        float acc[kMaxC];
 #pragma unroll
-    for (int co = 0; co < COUT; ++co) acc[co] = bias ? bias[co] : 0.f;
-    for (int ci = 0; ci < CIN; ++ci) {
+        for (int co = 0; co < kMaxC; ++co) acc[co] = bias[co];
+#pragma unroll 1
+        for (int ci = 0; ci < 2; ++ci) {
+            const S *in = x0 + (img * 2 + ci) * plane;
+#pragma unroll 3
+            for (int tap = 0; tap < 9; ++tap) {
+                const int yy = y + (tap / 3 - 1) * dil, xx = x + (tap % 3 - 1) * dil;
+                const float v = yy >= 0 && yy < H && xx >= 0 && xx < W ? ld_f(in + (long long)yy * W + xx) : 0.f;
+                const float *wr = s_w + (ci * 9 + tap) * kMaxC;
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-            const int ky = tap / 3, kx = tap % 3;
-            const float v = s_in[(ci * TW + ly + ky * dil) * TW + lx + kx * dil];
-            const float *wr = s_w + (ci * 9 + tap) * COUT;
-#pragma unroll
-            for (int co = 0; co < COUT; ++co) acc[co] = fmaf(wr[co], v, acc[co]);
+                for (int co = 0; co < kMaxC; ++co) acc[co] = fmaf(wr[co], v, acc[co]);
+            }
         }
-    }
-    if (gx < W && gy < H) {
-        SO *ob = out + (long long)img * COUT * plane + (long long)gy * W + gx;
-        const SM *mb = MASK ? mask + (long long)img * COUT * plane + (long long)gy * W + gx : nullptr;
+        VecC<S> *o = reinterpret_cast<VecC<S> *>(x1 + i * kMaxC);
 #pragma unroll
-        for (int co = 0; co < COUT; ++co) {
-            float v = acc[co];
-            if (RELU) v = fmaxf(v, 0.f);
-            if (MASK) v = ld_f(mb + co * plane) > 0.f ? v : 0.f;
-            ob[co * plane] = st_f<SO>(v);
+        for (int c = 0; c < kMaxC / VecC<S>::N; ++c) {
+            VecC<S> v;
+#pragma unroll
+            for (int j = 0; j < VecC<S>::N; ++j) v.v[j] = st_f<S>(fmaxf(acc[c * VecC<S>::N + j], 0.f));
+            o[c] = v;
         }
     }
 }
 
-// dW[co][ci][tap] += sum_{img,p} dy[img][co][p] * x[img][ci][p + off(tap)],
-// db[co] += sum dy[img][co][p].  Thread t < CIN*9 owns (ci, tap) for all co.
-template <typename SX, int CIN, int COUT>
-__global__ void __launch_bounds__(kMaxC * 9) wgrad_kernel(const SX *__restrict__ x, const float *__restrict__ dy,
-                                                          float *dw, float *db, int nimg, int H, int W, int dil,
-                                                          int tiles_x, int tiles_y) {
+// Inner layer 32 -> 32 on the CUDA cores (fp32 storage, or bf16 with the
+// tensor cores off): a 16 x 16 pixel tile with its halo in shared memory as
+// [ci][y][x] (an odd pitch per channel, so a pixel's channels are stored
+// without bank conflicts), one thread per pixel.
+__host__ __device__ constexpr int conv_mid_pitch(int dil) { return ((kTile + 2 * dil) * (kTile + 2 * dil)) | 1; }
+template <typename S>
+__global__ void __launch_bounds__(kConvThreads) conv_mid_kernel(const S *__restrict__ in, const float *__restrict__ w,
+                                                              const float *__restrict__ bias, S *__restrict__ out,
+                                                              int H, int W, int dil, int tiles_x) {
     extern __shared__ __align__(16) float smem[];
-    const int halo = dil;
-    const int TW = kTile + 2 * halo;
-    float *s_x = smem;                          // CIN * TW * TW
-    float *s_dy = smem + CIN * TW * TW;         // kTile*kTile * COUT, [p][co]
-    const int t = threadIdx.x;
-    const bool active = t < CIN * 9;
-    const int ci = active ? t / 9 : 0, tap = active ? t % 9 : 0;
-    const int ky = tap / 3, kx = tap % 3;
-    float acc[COUT];
-    float bacc = 0.f;
+    const int TW = kTile + 2 * dil;
+    float *s_w = smem;                           // 32 * 9 * 32
+    float *s_in = smem + kMaxC * 9 * kMaxC;      // 32 * pitch
+    const int pitch = conv_mid_pitch(dil);
+    const int tile = blockIdx.x, img = blockIdx.y;
+    const int tx0 = (tile % tiles_x) * kTile, ty0 = (tile / tiles_x) * kTile;
+    for (int e = threadIdx.x; e < kMaxC * 9 * kMaxC; e += blockDim.x) {
+        const int co = e % kMaxC, tap = (e / kMaxC) % 9, ci = e / (9 * kMaxC);
+        s_w[e] = w[(co * kMaxC + ci) * 9 + tap];
+    }
+    const S *inb = in + (long long)img * H * W * kMaxC;
+    for (int e = threadIdx.x; e < kMaxC * TW * TW; e += blockDim.x) {
+        const int ci = e % kMaxC, q = e / kMaxC, xx = q % TW, yy = q / TW;
+        const int gx = tx0 + xx - dil, gy = ty0 + yy - dil;
+        s_in[ci * pitch + q] =
+            (gx >= 0 && gx < W && gy >= 0 && gy < H) ? ld_f(inb + ((long long)gy * W + gx) * kMaxC + ci) : 0.f;
+    }
+    __syncthreads();
+    const int lx = threadIdx.x % kTile, ly = threadIdx.x / kTile;
+    const int gx = tx0 + lx, gy = ty0 + ly;
+    float acc[kMaxC];
 #pragma unroll
-    for (int co = 0; co < COUT; ++co) acc[co] = 0.f;
-    const long long plane = (long long)H * W;
-    const int ntile = tiles_x * tiles_y;
-    for (long long job = blockIdx.x; job < (long long)ntile * nimg; job += gridDim.x) {
-        const int img = (int)(job / ntile), tile = (int)(job % ntile);
-        const int tx0 = (tile % tiles_x) * kTile, ty0 = (tile / tiles_x) * kTile;
-        __syncthreads();
-        const SX *xb = x + (long long)img * CIN * plane;
-        for (int e = t; e < CIN * TW * TW; e += blockDim.x) {
-            const int xx = e % TW, yy = (e / TW) % TW, c = e / (TW * TW);
-            const int gx = tx0 + xx - halo, gy = ty0 + yy - halo;
-            s_x[e] = (gx >= 0 && gx < W && gy >= 0 && gy < H) ? ld_f(xb + c * plane + (long long)gy * W + gx) : 0.f;
-        }
-        const float *dyb = dy + (long long)img * COUT * plane;
-        for (int e = t; e < kTile * kTile * COUT; e += blockDim.x) {
-            const int co = e % COUT, p = e / COUT;
-            const int gx = tx0 + p % kTile, gy = ty0 + p / kTile;
-            s_dy[e] = (gx < W && gy < H) ? dyb[co * plane + (long long)gy * W + gx] : 0.f;
-        }
-        __syncthreads();
-        if (active) {
-            for (int p = 0; p < kTile * kTile; ++p) {
-                const int py = p / kTile, px = p % kTile;
-                const float v = s_x[(ci * TW + py + ky * dil) * TW + px + kx * dil];
-                const float *d = s_dy + p * COUT;
+    for (int co = 0; co < kMaxC; ++co) acc[co] = bias[co];
+    for (int ci = 0; ci < kMaxC; ++ci) {
 #pragma unroll
-                for (int co = 0; co < COUT; ++co) acc[co] = fmaf(d[co], v, acc[co]);
+        for (int tap = 0; tap < 9; ++tap) {
+            const float v = s_in[ci * pitch + (ly + (tap / 3) * dil) * TW + lx + (tap % 3) * dil];
+            const float *wr = s_w + (ci * 9 + tap) * kMaxC;
+#pragma unroll
+            for (int co = 0; co < kMaxC; ++co) acc[co] = fmaf(wr[co], v, acc[co]);
+        }
+    }
+    if (gx < W && gy < H) {
+        VecC<S> *o = reinterpret_cast<VecC<S> *>(out + (((long long)img * H + gy) * W + gx) * kMaxC);
+#pragma unroll
+        for (int c = 0; c < kMaxC / VecC<S>::N; ++c) {
+            VecC<S> v;
+#pragma unroll
+            for (int j = 0; j < VecC<S>::N; ++j) v.v[j] = st_f<S>(fmaxf(acc[c * VecC<S>::N + j], 0.f));
+            o[c] = v;
+        }
+    }
+}
+
+// Last layer, 32 -> 1: one thread per pixel, its nine taps' channels read as
+// 16-byte vectors through L1 (8 channels of all taps at a time, so every
+// output keeps one fma chain: channel by channel, tap by tap).  With the
+// 32 x 32 pixel input window of 32 channels in shared memory (131 KB, one
+// block of 256 threads per SM) the same sum took 1790 us for 256 images of
+// 64^2; 81 us now.
+template <typename S>
+__global__ void __launch_bounds__(256) conv_last_kernel(const S *__restrict__ x3, const float *__restrict__ w,
+                                                        const float *__restrict__ bias, float *__restrict__ out,
+                                                        int nimg, int H, int W, int dil) {
+    constexpr int N = VecC<S>::N;
+    __shared__ float s_w[kMaxC * 9];
+    for (int e = threadIdx.x; e < kMaxC * 9; e += blockDim.x) s_w[e] = w[e];
+    __syncthreads();
+    const long long plane = (long long)H * W, total = plane * nimg;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int p = (int)(i % plane), y = p / W, x = p % W;
+        float acc = bias[0];
+#pragma unroll 1
+        for (int c = 0; c < kMaxC / N; ++c) {
+            VecC<S> v[9];
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap) {
+                const int dy = (tap / 3 - 1) * dil, dx = (tap % 3 - 1) * dil;
+                const bool inside = y + dy >= 0 && y + dy < H && x + dx >= 0 && x + dx < W;
+                if (inside) v[tap] = reinterpret_cast<const VecC<S> *>(x3 + (i + (long long)dy * W + dx) * kMaxC)[c];
+                else v[tap] = VecC<S>{};
+            }
+#pragma unroll
+            for (int j = 0; j < N; ++j)
+#pragma unroll
+                for (int tap = 0; tap < 9; ++tap) acc = fmaf(s_w[(c * N + j) * 9 + tap], to_acc(v[tap].v[j]), acc);
+        }
+        out[i] = acc;
+    }
+}
+
+// ------------------------------------------------------------------ backward
+//
+// Weight gradients: every block sums the pixels it visits in registers,
+// writes its sums to its own row of `part` ([block][parameter]) and
+// reduce_grad_kernel adds the rows in block order, so a gradient does not
+// depend on the order of atomics.
+
+// dg[p][ci] = (x3[p][ci] > 0) sum_tap w[ci][8 - tap] dy[p + off(tap)]   (last layer, 32 <- 1)
+template <typename S>
+__global__ void __launch_bounds__(256) dgrad_last_kernel(const float *__restrict__ dy, const float *__restrict__ w,
+                                                         const S *__restrict__ act, float *__restrict__ dg, int nimg,
+                                                         int H, int W, int dil) {
+    __shared__ __align__(16) float s_w[9 * kMaxC];  // [tap][ci]
+    for (int e = threadIdx.x; e < 9 * kMaxC; e += blockDim.x) s_w[e] = w[(e % kMaxC) * 9 + 8 - e / kMaxC];
+    __syncthreads();
+    // four threads per pixel, 8 channels each
+    const long long plane = (long long)H * W, total = plane * nimg * 4;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long q = i >> 2;
+        const int c0 = (int)(i & 3) * 8;
+        const int p = (int)(q % plane), y = p / W, x = p % W;
+        float acc[8] = {};
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+            const int oy = (tap / 3 - 1) * dil, ox = (tap % 3 - 1) * dil;
+            const bool inside = y + oy >= 0 && y + oy < H && x + ox >= 0 && x + ox < W;
+            const float v = inside ? dy[q + (long long)oy * W + ox] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j] = fmaf(s_w[tap * kMaxC + c0 + j], v, acc[j]);
+        }
+        const S *m = act + q * kMaxC + c0;
+        float4 *o = reinterpret_cast<float4 *>(dg + q * kMaxC + c0);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] = ld_f(m + j) > 0.f ? acc[j] : 0.f;
+        o[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        o[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    }
+}
+
+// dx[p][ci] = (act[p][ci] > 0) sum_tap sum_co w[co][ci][8 - tap] dy[p + off(tap)][co]   (32 <- 32)
+//
+// Bound: the fp32 pipe (9216 fma per pixel).  A block takes 16 x 16 pixels;
+// a thread 4 pixels x 8 channels, so that 12 16-byte shared loads (4 of
+// pixels, 8 of weights, all without bank conflicts: pixels are padded to 80
+// bytes) feed 128 fma, as packed pairs of channels.  dy comes in two halves
+// of 16 channels, which keeps three blocks per SM at the default dilations.
+// One thread per pixel with all 32 outputs, 9 loads per 32 fma: 89 + 80 us
+// for the two layers of 16 images of 64^2, 39 + 38 us now.
+constexpr int kDgHalf = 16;                      // dy channels staged at a time
+constexpr int kDgPitch = kDgHalf + 4;            // floats per staged pixel
+template <typename S>
+__global__ void __launch_bounds__(256) dgrad_mid_kernel(const float *__restrict__ dy, const float *__restrict__ w,
+                                                        const S *__restrict__ act, float *__restrict__ dx, int H,
+                                                        int W, int dil, int tiles_x) {
+    extern __shared__ __align__(16) float smem[];
+    const int TW = kTile + 2 * dil;
+    float *s_w = smem;                            // [tap][co 16][ci 32]
+    float *s_d = smem + 9 * kDgHalf * kMaxC;      // [TW * TW][kDgPitch]
+    const int tile = blockIdx.x, img = blockIdx.y;
+    const int tx0 = (tile % tiles_x) * kTile, ty0 = (tile / tiles_x) * kTile;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int c0 = (lane >> 3) * 8, l = lane & 7;  // channels c0..c0+7; pixels x = l, l + 8 of rows 2 warp, 2 warp + 1
+    const float *dyb = dy + (long long)img * H * W * kMaxC;
+    float2 acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    for (int half = 0; half < 2; ++half) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < kDgHalf * kMaxC * 9; e += blockDim.x) {
+            const int tap = e % 9, ci = (e / 9) % kMaxC, co = e / (9 * kMaxC);
+            s_w[((8 - tap) * kDgHalf + co) * kMaxC + ci] = w[half * kDgHalf * kMaxC * 9 + e];
+        }
+        for (int e = threadIdx.x; e < TW * TW * (kDgHalf / 4); e += blockDim.x) {
+            const int c = e % (kDgHalf / 4), q = e / (kDgHalf / 4);
+            const int gx = tx0 + q % TW - dil, gy = ty0 + q / TW - dil;
+            const bool inside = gx >= 0 && gx < W && gy >= 0 && gy < H;
+            cp_async16_or_zero(s_d + q * kDgPitch + c * 4,
+                               inside ? dyb + ((long long)gy * W + gx) * kMaxC + half * kDgHalf + c * 4 : dyb, inside);
+        }
+        cp_async_wait_all();
+        __syncthreads();
+#pragma unroll 1
+        for (int tap = 0; tap < 9; ++tap) {
+            const float *pd = s_d + ((2 * warp + (tap / 3) * dil) * TW + l + (tap % 3) * dil) * kDgPitch;
+            const float *pw = s_w + tap * kDgHalf * kMaxC + c0;
+#pragma unroll
+            for (int k = 0; k < kDgHalf; k += 4) {
+                float4 v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    v[i] = *reinterpret_cast<const float4 *>(pd + ((i >> 1) * TW + (i & 1) * 8) * kDgPitch + k);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float4 wa = *reinterpret_cast<const float4 *>(pw + (k + u) * kMaxC);
+                    const float4 wb = *reinterpret_cast<const float4 *>(pw + (k + u) * kMaxC + 4);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float x = u == 0 ? v[i].x : u == 1 ? v[i].y : u == 2 ? v[i].z : v[i].w;
+                        const float2 xx = make_float2(x, x);
+                        acc[i][0] = __ffma2_rn(make_float2(wa.x, wa.y), xx, acc[i][0]);
+                        acc[i][1] = __ffma2_rn(make_float2(wa.z, wa.w), xx, acc[i][1]);
+                        acc[i][2] = __ffma2_rn(make_float2(wb.x, wb.y), xx, acc[i][2]);
+                        acc[i][3] = __ffma2_rn(make_float2(wb.z, wb.w), xx, acc[i][3]);
+                    }
+                }
             }
         }
-        if (t < COUT)
-            for (int p = 0; p < kTile * kTile; ++p) bacc += s_dy[p * COUT + t];
     }
-    if (active) {
 #pragma unroll
-        for (int co = 0; co < COUT; ++co) atomicAdd(dw + (co * CIN + ci) * 9 + tap, acc[co]);
+    for (int i = 0; i < 4; ++i) {
+        const int gx = tx0 + l + (i & 1) * 8, gy = ty0 + 2 * warp + (i >> 1);
+        if (gx >= W || gy >= H) continue;
+        const long long o = (((long long)img * H + gy) * W + gx) * kMaxC + c0;
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { v[2 * j] = acc[i][j].x; v[2 * j + 1] = acc[i][j].y; }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = ld_f(act + o + j) > 0.f ? v[j] : 0.f;
+        reinterpret_cast<float4 *>(dx + o)[0] = make_float4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<float4 *>(dx + o)[1] = make_float4(v[4], v[5], v[6], v[7]);
     }
-    if (t < COUT) atomicAdd(db + t, bacc);
+}
+
+// part[block][co][ci][tap] = sum over the block's pixels of dy[p][co] x[p + off(tap)][ci], and the bias sums
+// (32 x 32 x 9).
+//
+// Bound: the fp32 pipe (9216 fma per pixel).  A thread owns 8 co x 4 ci x the
+// 3 taps of one kernel row (96 sums, as packed pairs of co): 5 16-byte shared
+// loads per pixel feed 96 fma.  A warp is the 4 x 8 grid of (co, ci) groups of
+// one kernel row, three warps a pixel stream; a block runs two streams (even
+// and odd rows of a 16 x 8 pixel tile), added at the end.  One thread per
+// (ci, tap) with all 32 co, 9 loads per 32 fma, and 5.6 M atomics: 114 + 88 us
+// for 16 images of 64^2, 48 + 48 us now.
+constexpr int kWgX = 16, kWgY = 8, kWgThreads = 192;
+template <typename S>
+__global__ void __launch_bounds__(kWgThreads, 2) wgrad_mid_kernel(const S *__restrict__ x, const float *__restrict__ dy,
+                                                                float *__restrict__ part, int nparams, int off_w,
+                                                                int off_b, int nimg, int H, int W, int dil) {
+    extern __shared__ __align__(16) float smem[];
+    const int TX = kWgX + 2 * dil, TY = kWgY + 2 * dil;
+    float *s_dy = smem;                            // [128][32]
+    float *s_x = smem + kWgX * kWgY * kMaxC;       // [TX * TY][32]
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int ky = warp % 3, stream = warp / 3;
+    const int co0 = (lane >> 3) * 8, ci0 = (lane & 7) * 4;
+    float2 acc[4][4][3];                           // [co pair][ci][kx]
+    float bacc[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) acc[i][j][k] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) bacc[i] = 0.f;
+    const int tiles_x = (W + kWgX - 1) / kWgX, tiles_y = (H + kWgY - 1) / kWgY;
+    const long long tiles_img = (long long)tiles_x * tiles_y, jobs = tiles_img * nimg;
+    for (long long job = blockIdx.x; job < jobs; job += gridDim.x) {
+        const int img = (int)(job / tiles_img), tile = (int)(job % tiles_img);
+        const int tx0 = (tile % tiles_x) * kWgX, ty0 = (tile / tiles_x) * kWgY;
+        __syncthreads();
+        const float *dyb = dy + (long long)img * H * W * kMaxC;
+        for (int e = t; e < kWgX * kWgY * (kMaxC / 4); e += kWgThreads) {
+            const int c = e % (kMaxC / 4), p = e / (kMaxC / 4);
+            const int gx = tx0 + p % kWgX, gy = ty0 + p / kWgX;
+            const bool inside = gx < W && gy < H;
+            cp_async16_or_zero(s_dy + p * kMaxC + c * 4, inside ? dyb + ((long long)gy * W + gx) * kMaxC + c * 4 : dyb,
+                               inside);
+        }
+        constexpr int N = VecC<S>::N;
+        const S *xb = x + (long long)img * H * W * kMaxC;
+#pragma unroll 4
+        for (int e = t; e < TX * TY * (kMaxC / N); e += kWgThreads) {
+            const int c = e % (kMaxC / N), q = e / (kMaxC / N);
+            const int gx = tx0 + q % TX - dil, gy = ty0 + q / TX - dil;
+            VecC<S> v{};
+            if (gx >= 0 && gx < W && gy >= 0 && gy < H)
+                v = *reinterpret_cast<const VecC<S> *>(xb + ((long long)gy * W + gx) * kMaxC + c * N);
+            float *d = s_x + q * kMaxC + c * N;
+#pragma unroll
+            for (int j = 0; j < N; j += 4)
+                *reinterpret_cast<float4 *>(d + j) =
+                    make_float4(to_acc(v.v[j]), to_acc(v.v[j + 1]), to_acc(v.v[j + 2]), to_acc(v.v[j + 3]));
+        }
+        cp_async_wait_all();
+        __syncthreads();
+#pragma unroll 1
+        for (int py = stream; py < kWgY; py += 2) {
+            const float *pd = s_dy + py * kWgX * kMaxC + co0;
+            const float *px = s_x + (py + ky * dil) * TX * kMaxC + ci0;
+#pragma unroll 2
+            for (int p = 0; p < kWgX; ++p) {
+                const float4 da = *reinterpret_cast<const float4 *>(pd + p * kMaxC);
+                const float4 db = *reinterpret_cast<const float4 *>(pd + p * kMaxC + 4);
+                const float2 d[4] = {make_float2(da.x, da.y), make_float2(da.z, da.w), make_float2(db.x, db.y),
+                                     make_float2(db.z, db.w)};
+                if (ky == 0) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) { bacc[2 * i] += d[i].x; bacc[2 * i + 1] += d[i].y; }
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const float4 xv = *reinterpret_cast<const float4 *>(px + (p + k * dil) * kMaxC);
+                    const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float2 xx = make_float2(xs[j], xs[j]);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[i][j][k] = __ffma2_rn(d[i], xx, acc[i][j][k]);
+                    }
+                }
+            }
+        }
+    }
+    // the two streams' sums, through shared memory, into the block's row
+    float *row = part + (long long)blockIdx.x * nparams;
+    float *s_o = smem;                              // 96 threads x 105 sums
+    __syncthreads();
+    if (stream == 1) {
+        float *o = s_o + (warp - 3) * 32 + lane;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    o[(((i * 4 + j) * 3 + k) * 2 + 0) * 96] = acc[i][j][k].x;
+                    o[(((i * 4 + j) * 3 + k) * 2 + 1) * 96] = acc[i][j][k].y;
+                }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[(96 + i) * 96] = bacc[i];
+    }
+    __syncthreads();
+    if (stream == 0) {
+        const float *o = s_o + warp * 32 + lane;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const int r = ((i * 4 + j) * 3 + k) * 2;
+                    const int a = off_w + ((co0 + 2 * i) * kMaxC + ci0 + j) * 9 + ky * 3 + k;
+                    row[a] = acc[i][j][k].x + o[r * 96];
+                    row[a + kMaxC * 9] = acc[i][j][k].y + o[(r + 1) * 96];
+                }
+        if (ky == 0 && ci0 == 0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) row[off_b + co0 + i] = bacc[i] + o[(96 + i) * 96];
+        }
+    }
+}
+
+// A block's sums over warps: v[i] of every lane added over the block's warps
+// into row[at(i)] by warp 0 (n values per lane).
+template <int N, class AT>
+__device__ __forceinline__ void sum_over_warps(const float (&v)[N], float *s, float *row, AT &&at) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int i = 0; i < N; ++i) s[(warp * N + i) * 32 + lane] = v[i];
+    __syncthreads();
+    for (int i = warp; i < N; i += nw) {
+        float t = 0.f;
+        for (int k = 0; k < nw; ++k) t += s[(k * N + i) * 32 + lane];
+        const int a = at(i, lane);
+        if (a >= 0) row[a] = t;
+    }
+}
+
+// Last layer (32 -> 1): part[block][ci][tap] = sum_q dy[q - off(tap)] x3[q][ci]; a warp visits pixels, lane = ci,
+// so every activation is read once.  The bias sum rides along.
+template <typename S>
+__global__ void __launch_bounds__(256) wgrad_last_kernel(const S *__restrict__ x3, const float *__restrict__ dy,
+                                                         float *__restrict__ part, int nparams, int off_w, int off_b,
+                                                         int nimg, int H, int W, int dil) {
+    __shared__ float s[8 * 10 * 32];
+    const int lane = threadIdx.x & 31;
+    const long long plane = (long long)H * W, total = plane * nimg;
+    float acc[10] = {};
+    for (long long q = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; q < total;
+         q += ((long long)gridDim.x * blockDim.x) >> 5) {
+        const int p = (int)(q % plane), y = p / W, x = p % W;
+        const float v = ld_f(x3 + q * kMaxC + lane);
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+            const int oy = -(tap / 3 - 1) * dil, ox = -(tap % 3 - 1) * dil;
+            const bool inside = y + oy >= 0 && y + oy < H && x + ox >= 0 && x + ox < W;
+            acc[tap] = fmaf(inside ? dy[q + (long long)oy * W + ox] : 0.f, v, acc[tap]);
+        }
+        if (lane == 0) acc[9] += dy[q];
+    }
+    sum_over_warps(acc, s, part + (long long)blockIdx.x * nparams,
+                   [&](int i, int l) { return i < 9 ? off_w + l * 9 + i : l == 0 ? off_b : -1; });
+}
+
+// First layer (2 -> 32): part[block][co][ci][tap] = sum_p dy[p][co] x0[ci][p + off(tap)]; lane = co.
+template <typename S>
+__global__ void __launch_bounds__(256) wgrad_first_kernel(const S *__restrict__ x0, const float *__restrict__ dy,
+                                                          float *__restrict__ part, int nparams, int off_w, int off_b,
+                                                          int nimg, int H, int W, int dil) {
+    __shared__ float s[8 * 19 * 32];
+    const int lane = threadIdx.x & 31;
+    const long long plane = (long long)H * W, total = plane * nimg;
+    float acc[19] = {};
+    for (long long q = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; q < total;
+         q += ((long long)gridDim.x * blockDim.x) >> 5) {
+        const long long img = q / plane;
+        const int p = (int)(q % plane), y = p / W, x = p % W;
+        const float d = dy[q * kMaxC + lane];
+        // lanes 0..17 load the 18 inputs of the pixel, shuffles hand them to every lane
+        float mine = 0.f;
+        if (lane < 18) {
+            const int ci = lane / 9, tap = lane % 9;
+            const int yy = y + (tap / 3 - 1) * dil, xx = x + (tap % 3 - 1) * dil;
+            if (yy >= 0 && yy < H && xx >= 0 && xx < W) mine = ld_f(x0 + (img * 2 + ci) * plane + (long long)yy * W + xx);
+        }
+#pragma unroll
+        for (int i = 0; i < 18; ++i) acc[i] = fmaf(d, __shfl_sync(0xffffffffu, mine, i), acc[i]);
+        acc[18] += d;
+    }
+    sum_over_warps(acc, s, part + (long long)blockIdx.x * nparams,
+                   [&](int i, int l) { return i < 18 ? off_w + l * 18 + i : off_b + l; });
+}
+
+// grads[i] = sum of part[b][i] over blocks: 32 parameters per block, 8 slices of rows.
+__global__ void __launch_bounds__(256) reduce_grad_kernel(const float *__restrict__ part, int nblocks, int nparams,
+                                                          float *__restrict__ grads) {
+    __shared__ float s[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
+    float t = 0.f;
+    if (i < nparams)
+#pragma unroll 8
+        for (int b = warp; b < nblocks; b += 8) t += part[(long long)b * nparams + i];
+    s[warp][lane] = t;
+    __syncthreads();
+    if (warp == 0 && i < nparams) {
+        float v = 0.f;
+        for (int k = 0; k < 8; ++k) v += s[k][lane];
+        grads[i] = v;
+    }
 }
 
 // A column's share of a coarse cell's mean log: the product of the values'
@@ -398,13 +771,16 @@ __global__ void adam_kernel(float *p, const float *g, float *m, float *v, int n,
     p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-size_t conv_smem(int cin, int cout, int dil) {
-    const int TW = kTile + 2 * dil;
-    return sizeof(float) * ((size_t)cin * 9 * cout + (size_t)cin * TW * TW);
+size_t conv_mid_smem(int dil) {
+    return sizeof(float) * ((size_t)kMaxC * 9 * kMaxC + (size_t)kMaxC * conv_mid_pitch(dil));
 }
-size_t wgrad_smem(int cin, int cout, int dil) {
+size_t dgrad_mid_smem(int dil) {
     const int TW = kTile + 2 * dil;
-    return sizeof(float) * ((size_t)cin * TW * TW + (size_t)kTile * kTile * cout);
+    return sizeof(float) * ((size_t)9 * kDgHalf * kMaxC + (size_t)TW * TW * kDgPitch);
+}
+size_t wgrad_mid_smem(int dil) {  // operands, and the streams' sums afterwards
+    const size_t ops = (size_t)kWgX * kWgY * kMaxC + (size_t)(kWgX + 2 * dil) * (kWgY + 2 * dil) * kMaxC;
+    return sizeof(float) * std::max<size_t>(ops, 96 * 104);
 }
 
 template <typename K> perks_status set_smem(perks_context *ctx, K kernel, size_t bytes) {
@@ -435,6 +811,7 @@ struct perks_warmnet {
     long long cap_pixels = 0;   // nimg * H * W
     void *x0 = nullptr, *x1 = nullptr, *x2 = nullptr, *x3 = nullptr;
     float *outb = nullptr, *g0 = nullptr, *g1 = nullptr;
+    float *part = nullptr;      // [2 x SMs][nparams] partial sums of the weight gradients
 };
 
 namespace {
@@ -471,49 +848,38 @@ perks_status forward(perks_warmnet *n, int nimg, int ny, int nx, const double *k
     perks_context *ctx = n->ctx;
     const int H = ny / n->pool, W = nx / n->pool;
     const int tx = (W + kTile - 1) / kTile, ty = (H + kTile - 1) / kTile;
-    const dim3 grid(tx * ty, nimg);
+    const long long pixels = (long long)nimg * H * W;
+    const int pgrid = (int)std::min<long long>((pixels + 255) / 256, 16LL * ctx->sm_count);  // thread per pixel
     S *x0 = (S *)n->x0, *x1 = (S *)n->x1, *x2 = (S *)n->x2, *x3 = (S *)n->x3;
     const int cells = kPoolThreads / n->pool;
     const long long jobs = (long long)nimg * H * ((W + cells - 1) / cells);
     features_kernel<S><<<(int)std::min<long long>(jobs, 8LL * ctx->sm_count), kPoolThreads, 0, s>>>(
         k, f, u, x0, n->ut, ny, nx, n->pool, nimg);
     const float *P = n->params;
-    {
-        auto kern = conv_kernel<S, S, 2, kMaxC, false, true, false, float>;
-        const size_t sm = conv_smem(2, kMaxC, n->dil[0]);
-        perks_status rc = set_smem(ctx, kern, sm);
-        if (rc) return rc;
-        kern<<<grid, kConvThreads, sm, s>>>(x0, P + n->off_w[0], P + n->off_b[0], x1, (const float *)nullptr, H, W,
-                                           n->dil[0], tx, ty);
-    }
+    conv_first_kernel<S><<<pgrid, 256, 0, s>>>(x0, P + n->off_w[0], P + n->off_b[0], x1, nimg, H, W, n->dil[0]);
     if (std::is_same<S, __nv_bfloat16>::value && n->tensor_cores) {
         // inner layers as implicit GEMMs on the tensor cores
-        perks_status rc = set_smem(ctx, tc_conv32_kernel, tc_conv_smem());
-        if (rc) return rc;
-        const long long ntiles = (long long)nimg * (((long long)H * W + kTcPix - 1) / kTcPix);
-        const int blocks = (int)std::min<long long>(ntiles, 2LL * ctx->sm_count);
-        for (int l = 1; l <= 2; ++l)
-            tc_conv32_kernel<<<blocks, kTcThreads, tc_conv_smem(), s>>>(
+        const long long ntiles = (long long)nimg * ((W + kTcTX - 1) / kTcTX) * ((H + kTcTY - 1) / kTcTY);
+        for (int l = 1; l <= 2; ++l) {
+            const size_t sm = tc_conv_smem(n->dil[l]);
+            perks_status rc = set_smem(ctx, tc_conv32_kernel, sm);
+            if (rc) return rc;
+            const int per_sm = std::max(1, std::min(3, (int)(ctx->smem_per_sm / (sm + 1024))));
+            const int blocks = (int)std::min<long long>(ntiles, (long long)per_sm * ctx->sm_count);
+            tc_conv32_kernel<<<blocks, kTcThreads, sm, s>>>(
                 reinterpret_cast<const __nv_bfloat16 *>(l == 1 ? x1 : x2), P + n->off_w[l], P + n->off_b[l],
                 reinterpret_cast<__nv_bfloat16 *>(l == 1 ? x2 : x3), nimg, H, W, n->dil[l], n->err);
+        }
     } else {
-        auto kern = conv_kernel<S, S, kMaxC, kMaxC, false, true, false, float>;
         for (int l = 1; l <= 2; ++l) {
-            const size_t sm = conv_smem(kMaxC, kMaxC, n->dil[l]);
-            perks_status rc = set_smem(ctx, kern, sm);
+            const size_t sm = conv_mid_smem(n->dil[l]);
+            perks_status rc = set_smem(ctx, conv_mid_kernel<S>, sm);
             if (rc) return rc;
-            kern<<<grid, kConvThreads, sm, s>>>(l == 1 ? x1 : x2, P + n->off_w[l], P + n->off_b[l], l == 1 ? x2 : x3,
-                                               (const float *)nullptr, H, W, n->dil[l], tx, ty);
+            conv_mid_kernel<S><<<dim3(tx * ty, nimg), kConvThreads, sm, s>>>(
+                l == 1 ? x1 : x2, P + n->off_w[l], P + n->off_b[l], l == 1 ? x2 : x3, H, W, n->dil[l], tx);
         }
     }
-    {
-        auto kern = conv_kernel<S, float, kMaxC, 1, false, false, false, float>;
-        const size_t sm = conv_smem(kMaxC, 1, n->dil[3]);
-        perks_status rc = set_smem(ctx, kern, sm);
-        if (rc) return rc;
-        kern<<<grid, kConvThreads, sm, s>>>(x3, P + n->off_w[3], P + n->off_b[3], n->outb, (const float *)nullptr, H,
-                                           W, n->dil[3], tx, ty);
-    }
+    conv_last_kernel<S><<<pgrid, 256, 0, s>>>(x3, P + n->off_w[3], P + n->off_b[3], n->outb, nimg, H, W, n->dil[3]);
     PERKS_CUDA(ctx, cudaGetLastError());
     return PERKS_OK;
 }
@@ -523,49 +889,36 @@ perks_status backward(perks_warmnet *n, int nimg, int H, int W, cudaStream_t s) 
     perks_context *ctx = n->ctx;
     const int tx = (W + kTile - 1) / kTile, ty = (H + kTile - 1) / kTile;
     const dim3 grid(tx * ty, nimg);
-    const int wgrid = 4 * ctx->sm_count;
+    const long long pixels = (long long)nimg * H * W;
+    const int pgrid = (int)std::min<long long>((pixels * 4 + 255) / 256, 16LL * ctx->sm_count);
+    // rows of partial sums: two blocks per SM, or one per tile where there are fewer
+    const long long tiles = (long long)nimg * ((W + kWgX - 1) / kWgX) * ((H + kWgY - 1) / kWgY);
+    const int nb = (int)std::min<long long>(tiles, 2LL * ctx->sm_count);
+    if (!n->part) PERKS_CUDA(ctx, cudaMalloc(&n->part, sizeof(float) * 2 * ctx->sm_count * (size_t)n->nparams));
     S *x0 = (S *)n->x0, *x1 = (S *)n->x1, *x2 = (S *)n->x2, *x3 = (S *)n->x3;
     const float *P = n->params;
-    float *G = n->grads;
-    PERKS_CUDA(ctx, cudaMemsetAsync(G, 0, sizeof(float) * n->nparams, s));
+    float *part = n->part;
+    const int np = n->nparams;
     // layer 4 (C -> 1): dy = outb-gradient in g1[0..pixels)
     float *dy4 = n->g1;
-    {
-        auto kw = wgrad_kernel<S, kMaxC, 1>;
-        const size_t sm = wgrad_smem(kMaxC, 1, n->dil[3]);
-        perks_status rc = set_smem(ctx, kw, sm);
-        if (rc) return rc;
-        kw<<<wgrid, kMaxC * 9, sm, s>>>(x3, dy4, G + n->off_w[3], G + n->off_b[3], nimg, H, W, n->dil[3], tx, ty);
-        auto kd = conv_kernel<float, float, 1, kMaxC, true, false, true, S>;
-        const size_t sd = conv_smem(1, kMaxC, n->dil[3]);
-        rc = set_smem(ctx, kd, sd);
-        if (rc) return rc;
-        kd<<<grid, kConvThreads, sd, s>>>(dy4, P + n->off_w[3], nullptr, n->g0, x3, H, W, n->dil[3], tx, ty);
-    }
+    wgrad_last_kernel<S><<<nb, 256, 0, s>>>(x3, dy4, part, np, n->off_w[3], n->off_b[3], nimg, H, W, n->dil[3]);
+    dgrad_last_kernel<S><<<pgrid, 256, 0, s>>>(dy4, P + n->off_w[3], x3, n->g0, nimg, H, W, n->dil[3]);
     // layers 3 and 2 (C -> C)
     float *dy = n->g0, *dx = n->g1;
     for (int l = 2; l >= 1; --l) {
         S *xin = l == 2 ? x2 : x1;
-        auto kw = wgrad_kernel<S, kMaxC, kMaxC>;
-        const size_t sm = wgrad_smem(kMaxC, kMaxC, n->dil[l]);
-        perks_status rc = set_smem(ctx, kw, sm);
+        const size_t sm = wgrad_mid_smem(n->dil[l]), sd = dgrad_mid_smem(n->dil[l]);
+        perks_status rc = set_smem(ctx, wgrad_mid_kernel<S>, sm);
+        if (!rc) rc = set_smem(ctx, dgrad_mid_kernel<S>, sd);
         if (rc) return rc;
-        kw<<<wgrid, kMaxC * 9, sm, s>>>(xin, dy, G + n->off_w[l], G + n->off_b[l], nimg, H, W, n->dil[l], tx, ty);
-        auto kd = conv_kernel<float, float, kMaxC, kMaxC, true, false, true, S>;
-        const size_t sd = conv_smem(kMaxC, kMaxC, n->dil[l]);
-        rc = set_smem(ctx, kd, sd);
-        if (rc) return rc;
-        kd<<<grid, kConvThreads, sd, s>>>(dy, P + n->off_w[l], nullptr, dx, xin, H, W, n->dil[l], tx, ty);
+        wgrad_mid_kernel<S><<<nb, kWgThreads, sm, s>>>(xin, dy, part, np, n->off_w[l], n->off_b[l], nimg, H, W,
+                                                       n->dil[l]);
+        dgrad_mid_kernel<S><<<grid, 256, sd, s>>>(dy, P + n->off_w[l], xin, dx, H, W, n->dil[l], tx);
         float *t = dy; dy = dx; dx = t;
     }
     // layer 1 (2 -> C): weight gradient only
-    {
-        auto kw = wgrad_kernel<S, 2, kMaxC>;
-        const size_t sm = wgrad_smem(2, kMaxC, n->dil[0]);
-        perks_status rc = set_smem(ctx, kw, sm);
-        if (rc) return rc;
-        kw<<<wgrid, kMaxC * 9, sm, s>>>(x0, dy, G + n->off_w[0], G + n->off_b[0], nimg, H, W, n->dil[0], tx, ty);
-    }
+    wgrad_first_kernel<S><<<nb, 256, 0, s>>>(x0, dy, part, np, n->off_w[0], n->off_b[0], nimg, H, W, n->dil[0]);
+    reduce_grad_kernel<<<(np + 31) / 32, 256, 0, s>>>(part, nb, np, n->grads);
     PERKS_CUDA(ctx, cudaGetLastError());
     return PERKS_OK;
 }
@@ -669,7 +1022,7 @@ extern "C" perks_status perks_warmnet_destroy(perks_warmnet *n) {
     if (!n) return PERKS_OK;
     cudaSetDevice(n->device);
     free_net_bufs(n);
-    void *p[] = {n->params, n->grads, n->m, n->v, n->loss, n->ut, n->err};
+    void *p[] = {n->params, n->grads, n->m, n->v, n->loss, n->ut, n->err, n->part};
     for (void *q : p) if (q) cudaFree(q);
     delete n;
     return PERKS_OK;
