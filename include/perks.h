@@ -155,10 +155,13 @@ typedef struct {
     int32_t reserved[4];                /* reserved[0] = 1: one-cell-per-thread kernel instead of
                                            the 16-byte-vector kernel; reserved[1] = planes per
                                            block barrier of the vector kernel (2 or 4, 0 =
-                                           automatic); reserved[2] = kernel body
-                                           (PERKS_KERNEL_AUTO / _RESIDENT / _STREAMING; AUTO in a
-                                           plan means STREAMING, AUTO with no plan picks the
-                                           resident tile when every tile fits in shared memory);
+                                           automatic); STRIP: time steps per sweep (1, 2 or 4
+                                           where compiled, 0 = automatic), tiles_z the runs of
+                                           rows (0 = automatic); reserved[2] = kernel body
+                                           (PERKS_KERNEL_AUTO / _RESIDENT / _STREAMING / _STRIP;
+                                           AUTO in a plan means STREAMING, AUTO with no plan
+                                           picks the resident tile when every tile fits in shared
+                                           memory, the column strips for other 2-D domains);
                                            reserved[3] = threads per block (0 = automatic):
                                            256 or 512 for the resident tile kernel; 256 picks the
                                            plane-streaming kernel's two-blocks-per-SM
@@ -188,7 +191,7 @@ typedef struct {
     int64_t halo_cells_per_step;        /* halo cells written + read per step (H) */
     double algorithmic_bytes;           /* S (2 N D_uncache + 2 D_cache) + S N H for the whole run */
     int32_t kernel;                     /* PERKS_KERNEL_*: which kernel body runs */
-    int32_t planes_per_sync;            /* resident tile: planes a thread computes between two block
+    int32_t planes_per_sync;            /* column strips: time steps per sweep; resident tile: planes a thread computes between two block
                                            barriers; plane streaming: planes per block barrier */
 } perks_run_stats;
 
@@ -200,7 +203,10 @@ enum {
     PERKS_KERNEL_STREAMING = 2,  /* plane streaming: a block walks its tile plane by plane through a
                                     shared-memory ring, caching some planes in registers / shared
                                     memory */
-    PERKS_KERNEL_PER_STEP = 3    /* one launch per step (PERKS_PER_STEP) */
+    PERKS_KERNEL_PER_STEP = 3,   /* one launch per step (PERKS_PER_STEP) */
+    PERKS_KERNEL_STRIP = 4       /* column strips (2-D: 2d5pt, 2ds9pt, 2d9pt, 2d25pt): every warp streams a strip of
+                                    rows through register windows, several time steps per sweep; a sweep, not a
+                                    step, ends at the grid barrier.  Not used while a step trace is on */
 };
 
 /* Creates a stencil over a device-resident domain described by *desc (the
@@ -226,7 +232,8 @@ perks_status perks_stencil_get_trace(perks_stencil *st, uint64_t *host, int64_t 
  * stencil's current field -- each as the difference between runs of
  * `probe_steps` (>= 2) and 3 `probe_steps` steps, so that the per-run launch,
  * prologue and epilogue cancel -- the resident-tile kernel with 256 and 512
- * threads and 1 and 2 rows per thread where the domain fits, and the model's
+ * threads and 1 and 2 rows per thread where the domain fits, the column strips
+ * with each compiled number of steps per sweep (2-D), and the model's
  * own tiling and up to six tilings ranked by tz * (1 + halo fraction), each
  * with registers + shared memory, shared memory only, no cache, or no cache
  * in balanced shares (perks_stencil_plan.balanced), and with 2 or 4 planes

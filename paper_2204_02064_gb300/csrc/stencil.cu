@@ -11,6 +11,7 @@
 
 #include "internal.h"
 #include "stencil_registry.h"
+#include "stencil_strip.cuh"
 #include "stencil_tile.cuh"
 
 using namespace perks;
@@ -128,6 +129,17 @@ std::vector<TileKernelEntry> &tile_registry() {
     return table;
 }
 
+std::vector<StripKEntry> &strip_registry() {
+    static std::vector<StripKEntry> table = [] {
+        std::vector<StripKEntry> t;
+        register_strip_f64(t);
+        register_strip_f32(t);
+        register_strip_bf16(t);
+        return t;
+    }();
+    return table;
+}
+
 // Planes per block barrier preferred by default where both variants exist.
 constexpr int kDefaultPlanesPerBarrier = 2;
 
@@ -168,6 +180,8 @@ struct Plan {
     TileKernelEntry *tk = nullptr;
     int tx = 0, PP = 0, XGS = 0, groups = 0, chunks = 0, per_plane = 0;
     long long FS = 0;
+    // column-strip kernel (2-D): ntx strips across x, ntz runs of rows
+    StripKEntry *sk = nullptr;
 };
 
 }  // namespace
@@ -320,7 +334,63 @@ perks_status make_tile_plan(perks_stencil *st, Plan &pl) {
     return PERKS_OK;
 }
 
-perks_status make_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
+// Plan of the column-strip kernel (2-D domains): steps per sweep and runs of
+// rows from a model of a sweep in cycles of one SM quarter (SMSP), which
+// issues one warp instruction a cycle, or one fp64 one every 64 (measured: a
+// lone fp64 warp per SM runs at a quarter of the SM's rate).  An item of h
+// rows costs TS h + R TS (TS - 1) row-stages and, by itself, some 160 cycles
+// of latency per iteration on top of its instructions; a quarter works through
+// its warps' row-stages, the chip streams the field in and out, and a sweep
+// adds the grid barrier.  Measured against all runs from 8 to 256 at sides of
+// 256 to 4096, the plan it picks is within 10 % of the fastest.
+perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts, int want_nch) {
+    perks_context *ctx = st->ctx;
+    const int dt = st->desc.dtype, X = st->X, Z = st->Z, SM = ctx->sm_count;
+    double best = 1e300;
+    Plan bp;
+    if (st->desc.ndim == 2 && (dt != PERKS_BF16 || X % 8 == 0))
+        for (StripKEntry &e : strip_registry()) {
+            if (e.dtype != dt || e.shape != st->shape_id || e.aligned != (X % e.v == 0)) continue;
+            if (want_ts > 0 && e.ts != want_ts) continue;
+            const ShapeInfo &sh = shape_by_id(st->shape_id);
+            const int outw = (32 - 2 * e.hl) * e.v;
+            const int nsx = ceil_div(X, outw);
+            const double points = (double)e.v * sh.npts, R = sh.radius;
+            const double stage = dt == PERKS_F64 ? 64.0 * points : 0.75 * points + 4.0 * R + (dt == PERKS_BF16 ? 28 : 20);
+            // bytes per cycle the chip streams: from L2 while both fields fit there, else from HBM
+            const double rate = 2.0 * (double)st->cells * st->es < 1.0e8 ? 3600.0 : 2900.0;
+            const int most = 2 * e.nt / 32;  // warps per SM
+            for (int wps = 1; wps <= most; ++wps) {
+                int nch = std::max(1, std::min(Z, (int)((long long)wps * SM / nsx)));
+                if (want_nch > 0) nch = std::min(Z, want_nch);
+                const long long items = (long long)nsx * nch;
+                const double h = std::ceil((double)Z / nch);
+                const double rs = e.ts * h + R * e.ts * (e.ts - 1);
+                const double iters = h + (2.0 * R + 1.0) * e.ts;
+                const double quarter = std::ceil((double)items / (4.0 * SM));
+                const double rounds = std::ceil((double)items / ((double)most * SM));
+                const double bytes = ((double)items * iters * 32 * e.v + (double)st->cells) * st->es;
+                const double cyc =
+                    std::max({quarter * rs * stage, rounds * (rs * stage + 160.0 * iters), bytes / rate}) + 3500.0;
+                if (cyc / e.ts < best) {
+                    best = cyc / e.ts;
+                    bp.sk = &e;
+                    bp.ntx = nsx; bp.nty = 1; bp.ntz = nch;
+                    bp.txmax = outw; bp.tymax = 1; bp.tzmax = ceil_div(Z, nch);
+                    bp.blocks = items <= (long long)SM * e.nt / 32 ? SM : 2 * SM;
+                }
+            }
+        }
+    if (!bp.sk)
+        return fail(ctx, PERKS_ERR_UNSUPPORTED, "column-strip kernel: 2-D stencils 2d5pt, 2ds9pt, 2d9pt, 2d25pt only");
+    // halo cells: the overlap each item reads beyond its own cells, per step
+    bp.halo_cells = ((long long)bp.ntx * bp.ntz * 32 * bp.sk->v * (2LL * bp.sk->ts * shape_by_id(st->shape_id).radius) +
+                     (long long)bp.ntx * 2 * bp.sk->hl * bp.sk->v * Z) / bp.sk->ts;
+    pl = bp;
+    return PERKS_OK;
+}
+
+perks_status make_base_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
     perks_context *ctx = st->ctx;
     // The resident-tile kernel when it is asked for, or by default (no plan)
     // when every tile of the domain fits in shared memory.
@@ -500,7 +570,7 @@ perks_status make_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
         st->plan.reg_cache = 0;
         st->plan.smem_cache_planes = 0;
         Plan cf;
-        const perks_status r2 = make_plan(st, cf, false);
+        const perks_status r2 = make_base_plan(st, cf, false);
         st->has_plan = false;
         st->plan = saved_plan;
         if (r2 == PERKS_OK) {
@@ -513,6 +583,34 @@ perks_status make_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
     return PERKS_OK;
 }
 
+// 2d5pt domains that fit on chip whole.  fp32 / bf16: the strips are faster at
+// every size (1.43 us per step against 2.66 at 256^2 fp32, 2.2 against 5.0 at
+// 1000^2).  fp64, both on the fp64 pipe: 5.9 against 8.5 us at 700 x 500, 12.1
+// against 13.9 at 1000^2; up to 64 K cells, where it is 3.1 against 3.9, the
+// domain stays resident (small domains are held on chip by default).
+bool strip_beats_resident(const perks_stencil *st) { return st->desc.dtype != PERKS_F64 || st->cells > 65536; }
+
+// The plan a run uses.  A 2-D domain without a plan takes the column-strip
+// kernel where the other kernels could host the domain at all (so the domains
+// that are refused stay the same) and it is the faster one; a traced run keeps
+// the kernels that mark every step.
+perks_status make_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
+    const bool asked = !per_step && st->has_plan && st->plan.reserved[2] == PERKS_KERNEL_STRIP;
+    const bool open = !per_step && !st->has_plan && !st->no_resident && !st->trace && st->desc.ndim == 2;
+    if (!asked && !open) return make_base_plan(st, pl, per_step);
+    st->has_plan = false;
+    perks_status rc = make_base_plan(st, pl, false);
+    st->has_plan = asked;
+    if (rc) return rc;
+    if (asked) return make_strip_plan(st, pl, st->plan.reserved[1], st->plan.tiles_z);
+    if (pl.resident && !strip_beats_resident(st)) return PERKS_OK;
+    const std::string saved_msg = st->ctx->last_error;
+    Plan sp;
+    if (make_strip_plan(st, sp, 0, 0) == PERKS_OK) pl = sp;
+    else st->ctx->last_error = saved_msg;
+    return PERKS_OK;
+}
+
 void fill_stats(const perks_stencil *st, const Plan *pl, long long steps, int variant,
                 perks_run_stats *o) {
     std::memset(o, 0, sizeof(*o));
@@ -520,7 +618,17 @@ void fill_stats(const perks_stencil *st, const Plan *pl, long long steps, int va
     o->variant = variant;
     o->cells = st->cells;
     const double S = st->es;
-    if (variant == PERKS_PERSISTENT && pl && pl->resident) {
+    if (variant == PERKS_PERSISTENT && pl && pl->sk) {
+        o->kernel = PERKS_KERNEL_STRIP;
+        o->grid_blocks = pl->blocks;
+        o->threads_per_block = pl->sk->nt;
+        o->tiles_x = pl->ntx; o->tiles_y = pl->nty; o->tiles_z = pl->ntz;
+        o->planes_per_sync = pl->sk->ts;  // steps per sweep
+        o->halo_cells_per_step = pl->halo_cells;
+        // the field is read and written once per sweep of ts steps
+        const double sweeps = (double)((steps + pl->sk->ts - 1) / pl->sk->ts);
+        o->algorithmic_bytes = S * (2.0 * sweeps * (double)st->cells + (double)steps * pl->halo_cells);
+    } else if (variant == PERKS_PERSISTENT && pl && pl->resident) {
         o->kernel = PERKS_KERNEL_RESIDENT;
         o->grid_blocks = pl->blocks;
         o->threads_per_block = pl->tk->nt;
@@ -617,6 +725,34 @@ perks_status run_resident(perks_stencil *st, long long steps, cudaStream_t s, co
     return PERKS_OK;
 }
 
+// One cooperative launch of the column-strip kernel, sk->ts steps per sweep.
+perks_status run_strip(perks_stencil *st, long long steps, cudaStream_t s, const Plan &pl) {
+    perks_context *ctx = st->ctx;
+    if (!st->bar) PERKS_CUDA(ctx, cudaMalloc(&st->bar, sizeof(unsigned long long)));
+    if (!st->err) PERKS_CUDA(ctx, cudaMalloc(&st->err, sizeof(DevError)));
+    StripKArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.X = st->X; a.Z = st->Z;
+    a.nsx = pl.ntx; a.nch = pl.ntz;
+    a.sms = ctx->sm_count;
+    a.steps = steps;
+    a.boundary = st->desc.boundary;
+    a.boundary_f = (float)st->desc.boundary;
+    for (int i = 0; i < 25; ++i) { a.w[i] = st->kw[i]; a.wf[i] = (float)st->kw[i]; }
+    a.field[0] = st->field[st->cur];
+    a.field[1] = st->field[st->cur ^ 1];
+    a.bar = st->bar;
+    a.err = st->err;
+    a.timeout_ns = ctx->timeout_ns;
+    PERKS_CUDA(ctx, cudaMemsetAsync(st->bar, 0, sizeof(unsigned long long), s));
+    PERKS_CUDA(ctx, cudaMemsetAsync(st->err, 0, sizeof(DevError), s));
+    void *args[] = {&a};
+    PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)pl.sk->fn, dim3(pl.blocks), dim3(pl.sk->nt), args,
+                                                0, s));
+    if (((steps + pl.sk->ts - 1) / pl.sk->ts) & 1) st->cur ^= 1;
+    return PERKS_OK;
+}
+
 perks_status ensure_persistent_buffers(perks_stencil *st, const Plan &pl) {
     perks_context *ctx = st->ctx;
     const int RX = shape_by_id(st->shape_id).radius;
@@ -680,6 +816,7 @@ perks_status run_persistent(perks_stencil *st, long long steps, cudaStream_t s, 
     perks_status rc = make_plan(st, pl);
     if (rc) return rc;
     if (pl.resident) return run_resident(st, steps, s, pl);
+    if (pl.sk) return run_strip(st, steps, s, pl);
     rc = ensure_persistent_buffers(st, pl);
     if (rc) return rc;
     int per_sm = 0;
@@ -866,10 +1003,12 @@ extern "C" perks_status perks_stencil_set_plan(perks_stencil *st, const perks_st
     if (!plan) { st->has_plan = false; return PERKS_OK; }
     if (plan->tiles_x < 0 || plan->tiles_y < 0 || plan->tiles_z < 0 || plan->smem_cache_planes < -1)
         return fail(st->ctx, PERKS_ERR_INVALID_ARG, "stencil_set_plan: negative field");
-    if (plan->reserved[1] != 0 && plan->reserved[1] != 2 && plan->reserved[1] != 4)
+    if (plan->reserved[1] != 0 && plan->reserved[1] != 2 && plan->reserved[1] != 4 &&
+        !(plan->reserved[2] == PERKS_KERNEL_STRIP && plan->reserved[1] == 1))
         return fail(st->ctx, PERKS_ERR_INVALID_ARG, "stencil_set_plan: planes per barrier must be 0, 2 or 4");
-    if (plan->reserved[2] < PERKS_KERNEL_AUTO || plan->reserved[2] > PERKS_KERNEL_STREAMING)
-        return fail(st->ctx, PERKS_ERR_INVALID_ARG, "stencil_set_plan: kernel must be AUTO, RESIDENT or STREAMING");
+    if (plan->reserved[2] < PERKS_KERNEL_AUTO || (plan->reserved[2] > PERKS_KERNEL_STREAMING && plan->reserved[2] != PERKS_KERNEL_STRIP))
+        return fail(st->ctx, PERKS_ERR_INVALID_ARG,
+                    "stencil_set_plan: kernel must be AUTO, RESIDENT, STREAMING or STRIP");
     if (plan->reserved[3] != 0 && plan->reserved[3] != 256 && plan->reserved[3] != 512 && plan->reserved[3] != 1024)
         return fail(st->ctx, PERKS_ERR_INVALID_ARG, "stencil_set_plan: threads must be 0, 256, 512 or 1024");
     st->plan = *plan;
@@ -1050,6 +1189,22 @@ extern "C" perks_status perks_stencil_autotune(perks_stencil *st, int32_t varian
             p.reg_cache = 1 + (cand & 1);  // rows per thread
             p.reserved[2] = PERKS_KERNEL_RESIDENT;
             p.reserved[3] = cand < 2 ? 256 : 512;
+            st->plan = p;
+            st->has_plan = true;
+            Plan probe;
+            const std::string saved_msg = ctx->last_error;
+            if (make_plan(st, probe, false) == PERKS_OK) {
+                p.tiles_x = probe.ntx; p.tiles_y = probe.nty; p.tiles_z = probe.ntz;
+                plans.push_back(p);
+            }
+            ctx->last_error = saved_msg;
+        }
+    // column-strip kernel: the model's runs of rows for each compiled number of steps per sweep
+    if (!per_step && !st->no_resident && st->desc.ndim == 2)
+        for (int ts : {1, 2, 4}) {
+            perks_stencil_plan p{};
+            p.reserved[1] = ts;
+            p.reserved[2] = PERKS_KERNEL_STRIP;
             st->plan = p;
             st->has_plan = true;
             Plan probe;

@@ -48,6 +48,11 @@ void register_vec_f32_poisson(std::vector<KernelEntry> &out);
 void register_vec_bf16_poisson(std::vector<KernelEntry> &out);
 void register_vec_star2d_hi(std::vector<KernelEntry> &out);
 
+struct StripKEntry;  // stencil_strip.cuh
+void register_strip_f64(std::vector<StripKEntry> &out);
+void register_strip_f32(std::vector<StripKEntry> &out);
+void register_strip_bf16(std::vector<StripKEntry> &out);
+
 struct TileKernelEntry;  // stencil_tile.cuh
 void register_tile_kernels(std::vector<TileKernelEntry> &out);
 

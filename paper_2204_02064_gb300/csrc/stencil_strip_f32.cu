@@ -1,0 +1,15 @@
+// Instantiations of the column-strip stencil kernel, f32 storage.
+#include "stencil_registry.h"
+#include "stencil_strip.cuh"
+
+namespace perks {
+
+void register_strip_f32(std::vector<StripKEntry> &out) {
+    strip_entries<float, S2d5, 4>(out, PERKS_F32, SH_2D5);
+    strip_entries<float, S2d9, 4>(out, PERKS_F32, SH_2D9);
+    strip_entries<float, S2ds9, 2>(out, PERKS_F32, SH_2DS9);
+    strip_entries<float, S2ds9, 4, 192>(out, PERKS_F32, SH_2DS9);
+    strip_entries<float, S2d25, 2, 192>(out, PERKS_F32, SH_2D25);
+}
+
+}  // namespace perks
