@@ -306,6 +306,8 @@ struct perks_op {
     double *b = nullptr, *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr;
     float *r32 = nullptr, *p32 = nullptr, *q32 = nullptr, *d32 = nullptr;
     double *part = nullptr;
+    int max_nnz2 = 0, max_row = 0;                      // nonzeros of the largest block (of G2), of the longest row
+    int dyn3 = 0;                                       // kind 3: dynamic shared memory a block may take
     double *trace = nullptr;
     int trace_cap = 0;
     CgResult *res = nullptr;
@@ -338,6 +340,14 @@ void free_op(perks_op *op) {
     if (op->ms_done_host) cudaFreeHost(op->ms_done_host);
 }
 
+// Shared memory of kind 3 with a block's nonzeros on chip: 12 bytes per
+// nonzero (8 in fp32) and 4 per row.
+size_t slice_smem(const perks_op *op, int mode) {
+    const size_t nnz = ((size_t)op->max_nnz2 + 3) & ~size_t(3);
+    return kCgRowvecSmem + ((nnz * (mode == CGK_FP32_IR ? 4 : 8) + 15) & ~size_t(15)) + nnz * 4 +
+           ((size_t)op->max_rows2 + 4) * 4;
+}
+
 CgArgs make_args(perks_op *op, double rtol, int max_iter, int mode, double inner_rtol) {
     CgArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -367,6 +377,12 @@ CgArgs make_args(perks_op *op, double rtol, int max_iter, int mode, double inner
     a.spmv_kind = op->spmv_kind;
     a.vcache = rv && op->vcache_ok && mode != CGK_SPMV ? op->vcache_level : 0;
     a.vcache_rows = op->max_rows2;
+    if (rv && a.vcache == 0) {
+        a.slice_rows = op->max_rows2;
+        a.slice_nnz = (op->max_nnz2 + 3) & ~3;
+        a.slice = mode != CGK_SPMV && slice_smem(op, mode) <= (size_t)op->dyn3;
+    }
+    a.short_rows = rv && op->max_row <= kShortRow;  // at every vector cache level: the same sums
     a.seg.nseg = op->nseg;
     a.seg.val = op->sval;
     a.seg.val32 = op->sval32;
@@ -425,6 +441,16 @@ perks_status configure(perks_op *op) {
                                                                   kCgThreads, seg_smem_bytes()));
     if (per_sm3 < 1 || per_sm3 * ctx->sm_count < op->G)
         return fail(ctx, PERKS_ERR_LAUNCH_TOO_LARGE, "CG kernel of %d blocks is not co-resident", op->G);
+    // kind 3, two blocks per SM: each takes half of the SM's shared memory at most
+    cudaFuncAttributes fa3;
+    PERKS_CUDA(ctx, cudaFuncGetAttributes(&fa3, (const void *)perks_cg_kernel<3>));
+    const int dyn3 = std::min(ctx->smem_optin, ctx->smem_per_sm / 2 - 1024) - (int)fa3.sharedSizeBytes;
+    PERKS_CUDA(ctx, cudaFuncSetAttribute((const void *)perks_cg_kernel<3>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, dyn3));
+    int per_sm4 = 0;
+    PERKS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm4, (const void *)perks_cg_kernel<3>,
+                                                                  kCgThreads, dyn3));
+    op->dyn3 = per_sm4 * ctx->sm_count >= op->G2 ? dyn3 : 0;
     op->configured = true;
     return PERKS_OK;
 }
@@ -441,7 +467,12 @@ perks_status launch_persistent(perks_op *op, const CgArgs &a, cudaStream_t s) {
     PERKS_CUDA(ctx, cudaMemsetAsync(op->bar, 0, sizeof(unsigned long long), s));
     PERKS_CUDA(ctx, cudaMemsetAsync(op->err, 0, sizeof(DevError), s));
     void *args[] = {(void *)&a};
-    if (op->spmv_kind == PERKS_SPMV_ROWVEC)
+    // Kind 3 wherever the blocks' nonzeros fit on chip or the rows are short; long rows that stream from memory
+    // keep kind 0, whose L1 is not cut by shared memory.
+    if (op->spmv_kind == PERKS_SPMV_ROWVEC && a.vcache == 0 && (a.slice || a.short_rows))
+        PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)perks_cg_kernel<3>, dim3(op->G2), dim3(kCgThreads),
+                                                    args, a.slice ? slice_smem(op, a.mode) : kCgRowvecSmem, s));
+    else if (op->spmv_kind == PERKS_SPMV_ROWVEC)
         PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)perks_cg_kernel<0>, dim3(op->G2),
                                                     dim3(kCgThreads), args, rowvec_smem(op, a.vcache), s));
     else if (op->spmv_kind == PERKS_SPMV_SEG)
@@ -710,7 +741,11 @@ extern "C" perks_status perks_csr_create(perks_context *ctx, int32_t n, int64_t 
     {
         std::vector<int> pr((size_t)G2 + 1);
         OPCUDA(cudaMemcpy(pr.data(), op->part_row2, sizeof(int) * ((size_t)G2 + 1), cudaMemcpyDeviceToHost));
-        for (int g = 0; g < G2; ++g) op->max_rows2 = std::max(op->max_rows2, pr[g + 1] - pr[g]);
+        for (int g = 0; g < G2; ++g) {
+            op->max_rows2 = std::max(op->max_rows2, pr[g + 1] - pr[g]);
+            op->max_nnz2 = std::max(op->max_nnz2, rp[pr[g + 1]] - rp[pr[g]]);
+        }
+        for (int i = 0; i < n; ++i) op->max_row = std::max(op->max_row, rp[i + 1] - rp[i]);
     }
     int ov = 0;
     OPCUDA(cudaMemcpy(&ov, overflow, sizeof(int), cudaMemcpyDeviceToHost));

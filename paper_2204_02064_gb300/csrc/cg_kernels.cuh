@@ -34,6 +34,8 @@
 namespace perks {
 
 constexpr int kCgThreads = 512;
+// vector entries of a thread whose loads are in flight together (within 64 registers)
+constexpr int kCgRows64 = 1, kCgRows32 = 1;
 constexpr int kCgIpt = 4;
 constexpr int kCgTile = kCgThreads * kCgIpt;  // merge-path items per tile
 constexpr int kCgMaxTiles = 2048;              // tiles per block
@@ -76,6 +78,9 @@ struct CgArgs {
     int spmv_kind;           // 0: row-vector SpMV (default), 1: thread-level merge walk, 2: column-segmented
     int vcache;              // row-vector kind, vectors kept in shared memory: 0 none, 1 r (r32), 2 x, r, q (r32, d32, q32)
     int vcache_rows;         // rows of the largest block (capacity of each cached vector)
+    int slice;               // kind 3: the blocks keep their nonzeros (of the solve's value type) in shared memory
+    int short_rows;          // row-vector kinds: one lane per row (else eight)
+    int slice_rows, slice_nnz;  // rows and nonzeros of the largest block
     const double *spmv_in;
     double *spmv_out;
     SegArgs seg;             // column-segmented layout (spmv_kind 2)
@@ -381,7 +386,7 @@ template <typename V> __host__ __device__ constexpr int full_pass_steps() { retu
 // are loaded first, then all the gathers are issued, then the FMAs run (each
 // row's terms still in order), so the pass waits for one HBM load and one L2
 // gather instead of UU of each.
-template <int UU, typename V>
+template <int UU, bool SMEM, typename V>
 __device__ __forceinline__ void spmv_pass(const int *__restrict__ col, const V *__restrict__ gval,
                                           const V *__restrict__ vin, const int (&jb)[kRowsPer],
                                           const int (&je)[kRowsPer], int u, V (&acc)[kRowsPer]) {
@@ -393,8 +398,13 @@ __device__ __forceinline__ void spmv_pass(const int *__restrict__ col, const V *
         for (int k = 0; k < kRowsPer; ++k) {
             const int j = jb[k] + u + q * kSub;
             const bool in = j < je[k];
-            cj[q][k] = in ? __ldcs(col + j) : -1;
-            vv[q][k] = in ? __ldcs(gval + j) : V(0);
+            if constexpr (SMEM) {
+                cj[q][k] = in ? col[j] : -1;
+                vv[q][k] = in ? gval[j] : V(0);
+            } else {
+                cj[q][k] = in ? __ldcs(col + j) : -1;
+                vv[q][k] = in ? __ldcs(gval + j) : V(0);
+            }
         }
 #pragma unroll
     for (int q = 0; q < UU; ++q)
@@ -407,10 +417,11 @@ __device__ __forceinline__ void spmv_pass(const int *__restrict__ col, const V *
             if (cj[q][k] >= 0) acc[k] = fma(vv[q][k], xv[q][k], acc[k]);
 }
 
-template <typename V>
-__device__ double spmv_block_vec(const CgArgs &a, const CgSlice &sl, const V *__restrict__ gval,
-                                 const V *__restrict__ vin, V *__restrict__ vout, const V *dotv, double *red,
-                                 V *vout_s) {
+// Returns this thread's share of the dot product.  SMEM: col and gval point
+// into shared memory (indexed by the global nonzero all the same).
+template <typename V, bool SMEM = false>
+__device__ double spmv_rows_vec(const CgArgs &a, const CgSlice &sl, const int *col, const V *gval,
+                                const V *__restrict__ vin, V *__restrict__ vout, const V *dotv, V *vout_s) {
     static_assert(kRowsPer == 2 && kSub == 8, "the reduction below pairs two rows over eight lanes");
     constexpr int kU = full_pass_steps<V>();
     const int lane = threadIdx.x & (kSub - 1);
@@ -437,16 +448,16 @@ __device__ double spmv_block_vec(const CgArgs &a, const CgSlice &sl, const V *__
         // full passes of kU steps, then the remainder in passes of 4, 2 and 1:
         // no step issues FMAs that no lane of the warp needs
         int u = 0;
-        for (; u + kSub * kU <= wlong; u += kSub * kU) spmv_pass<kU>(a.col, gval, vin, jb, je, u, acc);
+        for (; u + kSub * kU <= wlong; u += kSub * kU) spmv_pass<kU, SMEM>(col, gval, vin, jb, je, u, acc);
         if (kU > 4 && u + kSub * 4 <= wlong) {
-            spmv_pass<4>(a.col, gval, vin, jb, je, u, acc);
+            spmv_pass<4, SMEM>(col, gval, vin, jb, je, u, acc);
             u += 4 * kSub;
         }
         if (kU > 2 && u + kSub * 2 <= wlong) {
-            spmv_pass<2>(a.col, gval, vin, jb, je, u, acc);
+            spmv_pass<2, SMEM>(col, gval, vin, jb, je, u, acc);
             u += 2 * kSub;
         }
-        for (; u < wlong; u += kSub) spmv_pass<1>(a.col, gval, vin, jb, je, u, acc);
+        for (; u < wlong; u += kSub) spmv_pass<1, SMEM>(col, gval, vin, jb, je, u, acc);
         // lanes 0-3 of the sub-warp keep row 0, lanes 4-7 row 1: each sends
         // the other row's partial across and adds the one it receives, then
         // the four lanes of each half sum their row
@@ -465,7 +476,47 @@ __device__ double spmv_block_vec(const CgArgs &a, const CgSlice &sl, const V *__
         }
     }
     __syncthreads();
-    return block_sum(dot, red);
+    return dot;
+}
+
+template <typename V>
+__device__ double spmv_block_vec(const CgArgs &a, const CgSlice &sl, const V *__restrict__ gval,
+                                 const V *__restrict__ vin, V *__restrict__ vout, const V *dotv, double *red,
+                                 V *vout_s) {
+    return block_sum(spmv_rows_vec<V>(a, sl, a.col, gval, vin, vout, dotv, vout_s), red);
+}
+
+// Short rows (at most kShortRow nonzeros): one lane per row, the gathers of
+// kShortStep of its nonzeros in flight.  A warp instruction of the FP64 pipe
+// costs the same with one lane active or 32, so eight lanes per row spend
+// eight times the issue of a 5-entry row on padding and another three
+// additions on the exchange.  Rows are summed in order.  The thread that
+// computes a row also updates its vector entries.  Returns this thread's
+// share of the dot product.  An iteration of a 5-point matrix of 430 K rows:
+// 44.5 -> 23.6 us (fp64), 37.7 -> 18.5 us (fp32 inner), with the sums of
+// grid_sum4 and, in fp32, the nonzeros on chip.
+constexpr int kShortRow = 16;
+constexpr int kShortStep = 8;
+template <typename V>
+__device__ double spmv_rows_short(const CgSlice &sl, const int *rp, const int *col, const V *val,
+                                  const V *__restrict__ vin, V *__restrict__ vout, const V *dotv, V *vout_s) {
+    double dot = 0.0;
+    for (int r = sl.r0 + threadIdx.x; r < sl.r1; r += blockDim.x) {
+        const int jb = rp[r], je = rp[r + 1];
+        V acc = V(0);
+        for (int j = jb; j < je; j += kShortStep) {
+            V xv[kShortStep];
+#pragma unroll
+            for (int q = 0; q < kShortStep; ++q) xv[q] = j + q < je ? __ldcg(vin + col[j + q]) : V(0);
+#pragma unroll
+            for (int q = 0; q < kShortStep; ++q)
+                if (j + q < je) acc = fma(val[j + q], xv[q], acc);
+        }
+        if (vout_s) vout_s[r - sl.r0] = acc;
+        else vout[r] = acc;
+        if (dotv) dot = fma((double)dotv[r], (double)acc, dot);
+    }
+    return dot;
 }
 
 template <typename V>
@@ -503,22 +554,26 @@ __device__ __forceinline__ bool cg_sync(const CgArgs &a, unsigned long long &epo
 // Shared memory of the row-vector kernel: the reduction scratch, followed
 // (vector cache on) by kCgVcacheBytesPerRow bytes per row of the largest
 // block: x, r and q in fp64, or r32, d32 and q32 for the fp32 inner solves.
-constexpr size_t kCgRowvecSmem = 1024;
+constexpr size_t kCgRowvecSmem = (reduce_scratch<kCgThreads>() * sizeof(double) + 1023) / 1024 * 1024;
 constexpr size_t kCgVcacheBytesPerRow = 3 * sizeof(double);
 
 // Persistent CG (mode FP64 / FP32_IR) or a single SpMV (mode SPMV).
-// ROWVEC: row-vector SpMV only, 1 KB of shared memory and at most 64
+// ROWVEC: row-vector SpMV only, little shared memory and at most 64
 // registers, so two blocks share an SM (twice the loads in flight); otherwise
 // the merge-based SpMV with its staged tiles, one block per SM.
+// Kind 3: the row-vector kernel for matrices whose blocks' nonzeros fit in
+// shared memory (loaded once per solve, so an SpMV waits for its gathers
+// only) and for short rows (one lane per row).
 template <int KIND>
-__global__ void __launch_bounds__(kCgThreads, KIND == 0 ? 2 : 1) perks_cg_kernel(const __grid_constant__ CgArgs a) {
+__global__ void __launch_bounds__(kCgThreads, KIND == 0 || KIND == 3 ? 2 : 1) perks_cg_kernel(const __grid_constant__ CgArgs a) {
     constexpr bool ROWVEC = KIND != 1;  // no merge-walk tiles in shared memory
     extern __shared__ __align__(16) unsigned char smem_raw[];
     CgSmem s;
     SegState st;
     st.bar = nullptr;
     st.parity = 0;
-    if constexpr (KIND == 0) {
+    constexpr bool EXCHANGE = KIND == 0 || KIND == 3;  // sums by grid_sum4
+    if constexpr (EXCHANGE) {
         std::memset(&s, 0, sizeof(s));
         s.red = reinterpret_cast<double *>(smem_raw);
     } else if constexpr (KIND == 2) {
@@ -534,7 +589,7 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 ? 2 : 1) perks_cg_kernel
     } else {
         s = carve_cg_smem(smem_raw);
     }
-    const int G = gridDim.x, blk = blockIdx.x, tid = threadIdx.x;
+    const int blk = blockIdx.x, tid = threadIdx.x;
     unsigned long long epoch = 0;
 
     CgSlice sl;
@@ -554,12 +609,105 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 ? 2 : 1) perks_cg_kernel
         __syncthreads();
     }
 
+    // kind 3: the block's row pointers, columns and values in shared memory
+    const int *rp3 = a.rowptr, *col3 = a.col;
+    const double *val3 = a.val;
+    const float *val3f = a.val32;
+    if constexpr (KIND == 3) {
+        if (a.slice) {
+            const bool single = a.mode == CGK_FP32_IR;
+            unsigned char *at = smem_raw + kCgRowvecSmem;
+            double *sv = reinterpret_cast<double *>(at);
+            float *sv32 = reinterpret_cast<float *>(at);
+            at += ((size_t)a.slice_nnz * (single ? 4 : 8) + 15) & ~size_t(15);
+            int *sc = reinterpret_cast<int *>(at);
+            int *sr = sc + a.slice_nnz;
+            const int nnz = a.rowptr[sl.r1] - sl.jb;
+            for (int j = tid; j < nnz; j += blockDim.x) {
+                sc[j] = a.col[sl.jb + j];
+                if (single) sv32[j] = a.val32[sl.jb + j];
+                else sv[j] = a.val[sl.jb + j];
+            }
+            for (int i = tid; i <= sl.r1 - sl.r0; i += blockDim.x) sr[i] = a.rowptr[sl.r0 + i];
+            __syncthreads();
+            rp3 = sr - sl.r0;
+            col3 = sc - sl.jb;
+            if (single) val3f = sv32 - sl.jb;
+            else val3 = sv - sl.jb;
+        }
+    }
+    // The SpMV; the caller's sum of the returned values over the block's
+    // threads is the dot product (kinds 1 and 2: already summed, in thread 0).
+    auto spmv64 = [&](const double *vin, double *vout, const double *dotv, double *vout_s) -> double {
+        if constexpr (KIND == 3) {
+            const bool on_chip = a.slice && a.mode == CGK_FP64;
+            double d;
+            if (a.short_rows)
+                d = spmv_rows_short<double>(sl, rp3, col3, val3, vin, vout, dotv, nullptr);
+            else if (on_chip)
+                d = spmv_rows_vec<double, true>(a, sl, col3, val3, vin, vout, dotv, nullptr);
+            else
+                d = spmv_rows_vec<double>(a, sl, a.col, a.val, vin, vout, dotv, nullptr);
+            return d;
+        } else if constexpr (KIND == 0) {
+            if (a.short_rows) return spmv_rows_short<double>(sl, a.rowptr, a.col, a.val, vin, vout, dotv, vout_s);
+            return spmv_rows_vec<double>(a, sl, a.col, a.val, vin, vout, dotv, vout_s);
+        } else {
+            const double d = spmv_k<KIND, double>(a, s, sl, a.val, vin, vout, dotv, smem_raw, st, vout_s);
+            return tid == 0 ? d : 0.0;
+        }
+    };
+    auto spmv32 = [&](const float *vin, float *vout, const float *dotv, float *vout_s) -> double {
+        if constexpr (KIND == 3) {
+            if (a.short_rows) return spmv_rows_short<float>(sl, rp3, col3, val3f, vin, vout, dotv, nullptr);
+            if (a.slice) return spmv_rows_vec<float, true>(a, sl, col3, val3f, vin, vout, dotv, nullptr);
+            return spmv_rows_vec<float>(a, sl, a.col, a.val32, vin, vout, dotv, nullptr);
+        } else if constexpr (KIND == 0) {
+            if (a.short_rows) return spmv_rows_short<float>(sl, a.rowptr, a.col, a.val32, vin, vout, dotv, vout_s);
+            return spmv_rows_vec<float>(a, sl, a.col, a.val32, vin, vout, dotv, vout_s);
+        } else {
+            const double d = spmv_k<KIND, float>(a, s, sl, a.val32, vin, vout, dotv, smem_raw, st, vout_s);
+            return tid == 0 ? d : 0.0;
+        }
+    };
+    unsigned round = 0;
+    // grid-wide sum of v over all threads, with post(total, ratio, flag) of it, and a grid barrier
+    auto gsum = [&](double v, SumResult &out, auto &&post) -> bool {
+        if constexpr (EXCHANGE) {
+            return grid_sum4<kCgThreads>(a.part, gridDim.x, a.bar, epoch, a.err, a.timeout_ns, round, v, s.red, out,
+                                         post);
+        } else {
+            double *part = a.part + (size_t)(round++ & 1) * gridDim.x;
+            v = block_sum(v, s.red);
+            if (tid == 0) part[blockIdx.x] = v;
+            if (!cg_sync(a, epoch)) return false;
+            out.total = grid_sum(part, gridDim.x, s.red);
+            out.ratio = 0.0;
+            out.flag = 0;
+            post(out.total, out.ratio, out.flag);
+            return true;
+        }
+    };
+    auto plain = [](double, double &, int &) {};
+    SumResult sum;
+    double rr = 0.0, tol2 = 0.0;
+    auto small = [&](double t, double &, int &flag) { flag = t <= tol2; };  // the squared residual is in tolerance
+    auto step_length = [&](double num) {  // num / <p, q>, unless <p, q> is not positive and finite
+        return [num](double t, double &ratio, int &flag) {
+            flag = !(t > 0.0) || !isfinite(t);
+            ratio = num / t;
+        };
+    };
+
     if (a.mode == CGK_SPMV) {
+        if constexpr (KIND == 3) {
+            spmv64(a.spmv_in, a.spmv_out, nullptr, nullptr);
+            return;
+        }
         spmv_k<KIND, double>(a, s, sl, a.val, a.spmv_in, a.spmv_out, nullptr, smem_raw, st);
         return;
     }
 
-    double *part0 = a.part, *part1 = a.part + G;
     const double *b = a.b;
     double *x = a.x, *r = a.r, *p = a.p, *q = a.q;
 
@@ -590,7 +738,7 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 ? 2 : 1) perks_cg_kernel
     // ---- r0 = b - A x0, ||b||^2
     if (vc64)
         for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) xs[i - r0] = x[i];
-    spmv_k<KIND, double>(a, s, sl, a.val, x, q, nullptr, smem_raw, st, vc64 ? qs : nullptr);
+    spmv64(x, q, nullptr, vc64 ? qs : nullptr);
     double bb_p = 0.0, rr_p = 0.0;
     for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) {
         const double ri = b[i] - Q(i);
@@ -599,54 +747,73 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 ? 2 : 1) perks_cg_kernel
         bb_p += b[i] * b[i];
         rr_p += ri * ri;
     }
-    bb_p = block_sum(bb_p, s.red);
-    rr_p = block_sum(rr_p, s.red);
-    if (tid == 0) { part0[blk] = bb_p; part1[blk] = rr_p; }
-    if (!cg_sync(a, epoch)) return;
-    const double bb = grid_sum(part0, G, s.red);
-    double rr = grid_sum(part1, G, s.red);
-    const double tol2 = a.rtol * a.rtol * bb;
-    if (!cg_sync(a, epoch)) return;  // partials read before they are reused
+    if (!gsum(bb_p, sum, plain)) return;
+    const double bb = sum.total;
+    tol2 = a.rtol * a.rtol * bb;
+    if (!gsum(rr_p, sum, small)) return;
+    rr = sum.total;
+    bool done = sum.flag != 0;
 
     int status = PERKS_ERR_NOT_CONVERGED;
     int it = 0, outer = 0;
 
     if (a.mode == CGK_FP64) {
         for (int restart = 0;; ++restart) {
-            if (rr <= tol2) { status = PERKS_OK; break; }
+            if (done) { status = PERKS_OK; break; }
             bool converged = false;
             while (it < a.max_iter) {
                 // A: q = A p, <p, q>
-                const double pq_p = spmv_k<KIND, double>(a, s, sl, a.val, p, q, p, smem_raw, st, vc64 ? qs : nullptr);
-                if (tid == 0) part0[blk] = pq_p;
-                if (!cg_sync(a, epoch)) return;
+                const double pq_p = spmv64(p, q, p, vc64 ? qs : nullptr);
+                if (!gsum(pq_p, sum, step_length(rr))) return;
                 // B: alpha; x += alpha p; r -= alpha q; <r, r>
-                const double pq = grid_sum(part0, G, s.red);
-                if (!(pq > 0.0) || !isfinite(pq)) { status = PERKS_ERR_BREAKDOWN; break; }
-                const double alpha = rr / pq;
+                if (sum.flag) { status = PERKS_ERR_BREAKDOWN; break; }
+                const double alpha = sum.ratio;
                 double rn_p = 0.0;
-                for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) {
-                    X(i) = fma(alpha, p[i], X(i));
-                    const double ri = fma(-alpha, Q(i), R(i));
-                    R(i) = ri;
-                    rn_p += ri * ri;
+                for (int i0 = sl.r0 + tid; i0 < sl.r1; i0 += kCgRows64 * kCgThreads) {
+                    double pv[kCgRows64], xv[kCgRows64], qv[kCgRows64], rv[kCgRows64];
+#pragma unroll
+                    for (int u = 0; u < kCgRows64; ++u) {
+                        const int i = i0 + u * kCgThreads;
+                        if (i < sl.r1) { pv[u] = p[i]; xv[u] = X(i); qv[u] = Q(i); rv[u] = R(i); }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kCgRows64; ++u) {
+                        const int i = i0 + u * kCgThreads;
+                        if (i < sl.r1) {
+                            X(i) = fma(alpha, pv[u], xv[u]);
+                            const double ri = fma(-alpha, qv[u], rv[u]);
+                            R(i) = ri;
+                            rn_p += ri * ri;
+                        }
+                    }
                 }
-                rn_p = block_sum(rn_p, s.red);
-                if (tid == 0) part1[blk] = rn_p;
-                if (!cg_sync(a, epoch)) return;
                 // C: beta; p = r + beta p
-                const double rr_new = grid_sum(part1, G, s.red);
-                const double beta = rr_new / rr;
+                if (!gsum(rn_p, sum, [&](double t, double &ratio, int &flag) { ratio = t / rr; flag = t <= tol2; }))
+                    return;
+                const double rr_new = sum.total, beta = sum.ratio;
+                converged = sum.flag != 0;
                 if (blk == 0 && tid == 0 && it < a.trace_cap) {
                     a.trace[3 * it + 0] = alpha;
                     a.trace[3 * it + 1] = beta;
                     a.trace[3 * it + 2] = rr_new;
                 }
-                for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) p[i] = fma(beta, p[i], R(i));
+                for (int i0 = sl.r0 + tid; i0 < sl.r1; i0 += kCgRows64 * kCgThreads) {
+                    double pv[kCgRows64], rv[kCgRows64];
+#pragma unroll
+                    for (int u = 0; u < kCgRows64; ++u) {
+                        const int i = i0 + u * kCgThreads;
+                        if (i < sl.r1) { pv[u] = p[i]; rv[u] = R(i); }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kCgRows64; ++u) {
+                        const int i = i0 + u * kCgThreads;
+                        if (i < sl.r1) p[i] = fma(beta, pv[u], rv[u]);
+                    }
+                }
                 rr = rr_new;
                 ++it;
                 if (!cg_sync(a, epoch)) return;
-                if (rr <= tol2) { converged = true; break; }
+                if (converged) break;
             }
             if (status == PERKS_ERR_BREAKDOWN) break;
             // C5: true residual in fp64 (the SpMV gathers x from global memory)
@@ -654,18 +821,17 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 ? 2 : 1) perks_cg_kernel
                 put_x();
                 if (!cg_sync(a, epoch)) return;
             }
-            spmv_k<KIND, double>(a, s, sl, a.val, x, q, nullptr, smem_raw, st, vc64 ? qs : nullptr);
+            spmv64(x, q, nullptr, vc64 ? qs : nullptr);
             double tr_p = 0.0;
             for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) {
                 const double ri = b[i] - Q(i);
                 R(i) = ri;
                 tr_p += ri * ri;
             }
-            tr_p = block_sum(tr_p, s.red);
-            if (tid == 0) part0[blk] = tr_p;
-            if (!cg_sync(a, epoch)) return;
-            rr = grid_sum(part0, G, s.red);
-            if (rr <= tol2) { status = PERKS_OK; break; }
+            if (!gsum(tr_p, sum, small)) return;
+            rr = sum.total;
+            done = sum.flag != 0;
+            if (done) { status = PERKS_OK; break; }
             if (!converged || restart >= a.max_restarts) break;
             for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) p[i] = R(i);
             ++outer;
@@ -679,7 +845,7 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 ? 2 : 1) perks_cg_kernel
         auto Q32 = [&](int i) -> float & { return vc32 ? q32s[i - r0] : q32[i]; };
         for (;;) {
             // outer: rr holds ||b - A x||^2 (fp64); r holds the residual
-            if (rr <= tol2) { status = PERKS_OK; break; }
+            if (done) { status = PERKS_OK; break; }
             if (outer >= a.max_restarts || it >= a.max_iter) break;
             double r0_p = 0.0;
             for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) {
@@ -689,55 +855,72 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 ? 2 : 1) perks_cg_kernel
                 D32(i) = 0.0f;
                 r0_p += (double)ri * (double)ri;
             }
-            r0_p = block_sum(r0_p, s.red);
-            if (tid == 0) part0[blk] = r0_p;
-            if (!cg_sync(a, epoch)) return;
-            double irr = grid_sum(part0, G, s.red);
+            if (!gsum(r0_p, sum, plain)) return;
+            double irr = sum.total;
             const double itol2 = a.inner_rtol * a.inner_rtol * irr;
-            if (!cg_sync(a, epoch)) return;
             while (it < a.max_iter) {
-                const double pq_p =
-                    spmv_k<KIND, float>(a, s, sl, a.val32, p32, q32, p32, smem_raw, st, vc32 ? q32s : nullptr);
-                if (tid == 0) part0[blk] = pq_p;
-                if (!cg_sync(a, epoch)) return;
-                const double pq = grid_sum(part0, G, s.red);
-                if (!(pq > 0.0) || !isfinite(pq)) { status = PERKS_ERR_BREAKDOWN; break; }
-                const float alpha = (float)(irr / pq);
+                const double pq_p = spmv32(p32, q32, p32, vc32 ? q32s : nullptr);
+                if (!gsum(pq_p, sum, step_length(irr))) return;
+                if (sum.flag) { status = PERKS_ERR_BREAKDOWN; break; }
+                const float alpha = (float)sum.ratio;
                 double rn_p = 0.0;
-                for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) {
-                    D32(i) = fmaf(alpha, p32[i], D32(i));
-                    const float ri = fmaf(-alpha, Q32(i), R32(i));
-                    R32(i) = ri;
-                    rn_p += (double)ri * (double)ri;
+                for (int i0 = sl.r0 + tid; i0 < sl.r1; i0 += kCgRows32 * kCgThreads) {
+                    float pv[kCgRows32], dv[kCgRows32], qv[kCgRows32], rv[kCgRows32];
+#pragma unroll
+                    for (int u = 0; u < kCgRows32; ++u) {
+                        const int i = i0 + u * kCgThreads;
+                        if (i < sl.r1) { pv[u] = p32[i]; dv[u] = D32(i); qv[u] = Q32(i); rv[u] = R32(i); }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kCgRows32; ++u) {
+                        const int i = i0 + u * kCgThreads;
+                        if (i < sl.r1) {
+                            D32(i) = fmaf(alpha, pv[u], dv[u]);
+                            const float ri = fmaf(-alpha, qv[u], rv[u]);
+                            R32(i) = ri;
+                            const double rd = (double)ri;
+                            rn_p = fma(rd, rd, rn_p);
+                        }
+                    }
                 }
-                rn_p = block_sum(rn_p, s.red);
-                if (tid == 0) part1[blk] = rn_p;
-                if (!cg_sync(a, epoch)) return;
-                const double rr_new = grid_sum(part1, G, s.red);
-                const float beta = (float)(rr_new / irr);
-                for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) p32[i] = fmaf(beta, p32[i], R32(i));
+                if (!gsum(rn_p, sum, [&](double t, double &ratio, int &flag) { ratio = t / irr; flag = t <= itol2; }))
+                    return;
+                const double rr_new = sum.total;
+                const float beta = (float)sum.ratio;
+                const bool inner_done = sum.flag != 0;
+                for (int i0 = sl.r0 + tid; i0 < sl.r1; i0 += kCgRows32 * kCgThreads) {
+                    float pv[kCgRows32], rv[kCgRows32];
+#pragma unroll
+                    for (int u = 0; u < kCgRows32; ++u) {
+                        const int i = i0 + u * kCgThreads;
+                        if (i < sl.r1) { pv[u] = p32[i]; rv[u] = R32(i); }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kCgRows32; ++u) {
+                        const int i = i0 + u * kCgThreads;
+                        if (i < sl.r1) p32[i] = fmaf(beta, pv[u], rv[u]);
+                    }
+                }
                 irr = rr_new;
                 ++it;
                 if (!cg_sync(a, epoch)) return;
-                if (irr <= itol2) break;
+                if (inner_done) break;
             }
             if (status == PERKS_ERR_BREAKDOWN) break;
             // x += d (fp64), then the fp64 residual of the refined x
             for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) x[i] += (double)D32(i);
             ++outer;
             if (!cg_sync(a, epoch)) return;
-            spmv_k<KIND, double>(a, s, sl, a.val, x, q, nullptr, smem_raw, st);
+            spmv64(x, q, nullptr, nullptr);
             double tr_p = 0.0;
             for (int i = sl.r0 + tid; i < sl.r1; i += blockDim.x) {
                 const double ri = b[i] - q[i];
                 r[i] = ri;
                 tr_p += ri * ri;
             }
-            tr_p = block_sum(tr_p, s.red);
-            if (tid == 0) part0[blk] = tr_p;
-            if (!cg_sync(a, epoch)) return;
-            rr = grid_sum(part0, G, s.red);
-            if (!cg_sync(a, epoch)) return;
+            if (!gsum(tr_p, sum, small)) return;
+            rr = sum.total;
+            done = sum.flag != 0;
         }
     }
     if (blk == 0 && tid == 0) {

@@ -323,3 +323,70 @@ def test_vector_cache_skipped_when_rows_do_not_fit(ctx):
     assert res["true_rel_residual"] <= 1e-12
     assert np.max(np.abs(x.cpu().numpy() - b / 2.0)) <= 1e-15
     op.close()
+
+
+def _banded_spd(n, half, seed):
+    """Symmetric diagonally dominant CSR matrix with up to 2 half + 1 entries
+    per row: row i couples to i +- 1 .. i +- half (fewer at the ends)."""
+    rows, cols, vals = [], [], []
+    for d in range(1, half + 1):
+        if d >= n:
+            break
+        i = np.arange(n - d)
+        v = inputs.uniform(inputs.substream(seed, d), n - d) - 1.0
+        rows += [i, i + d]
+        cols += [i + d, i]
+        vals += [v, v]
+    rows = np.concatenate(rows) if rows else np.zeros(0, dtype=np.int64)
+    cols = np.concatenate(cols) if cols else np.zeros(0, dtype=np.int64)
+    vals = np.concatenate(vals) if vals else np.zeros(0)
+    diag = 1.0 + 1.02 * np.bincount(rows, weights=np.abs(vals), minlength=n)
+    rows, cols = np.concatenate([rows, np.arange(n)]), np.concatenate([cols, np.arange(n)])
+    vals = np.concatenate([vals, diag])
+    order = np.argsort(rows * n + cols, kind="stable")
+    rp = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(np.bincount(rows, minlength=n), out=rp[1:])
+    return rp.astype(np.int32), cols[order].astype(np.int32), vals[order]
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["fp64", "fp32_ir"])
+@pytest.mark.parametrize("n,half", [(1, 0), (5, 2), (300, 0), (307, 7), (2000, 8), (40000, 2), (9000, 7),
+                                    (70000, 8), (700000, 1), (260000, 9)])
+def test_short_and_on_chip_rows(ctx, oracle, n, half, mode):
+    """Rows of up to 16 nonzeros (one lane per row) and longer ones, with a
+    block's nonzeros in shared memory or streamed: fewer rows than blocks, a
+    row length at and just above the limit, slices that fit and that do not."""
+    from paper_2204_02064_gb300 import api
+    rp, c, v = _banded_spd(n, half, 91)
+    b = inputs.cg_rhs(n, 92)
+    op = api.CsrOperator(ctx, torch.from_numpy(rp).cuda(), torch.from_numpy(c).cuda(), torch.from_numpy(v).cuda())
+    x = torch.zeros(n, dtype=torch.float64, device="cuda")
+    res = op.solve(torch.from_numpy(b).cuda(), x, rtol=1e-10, mode=mode)
+    assert res["true_rel_residual"] <= 1e-10
+    y = torch.empty_like(x)
+    op.spmv(x, y)
+    ref = oracle.cg(rp, c, v, b, rtol=1e-10, max_iter=10000)
+    assert np.linalg.norm(x.cpu().numpy() - ref["x"]) <= 1e-8 * np.linalg.norm(ref["x"])
+    if mode == 0:
+        assert abs(res["iterations"] - ref["iters"]) <= 2
+    assert np.linalg.norm(y.cpu().numpy() - b) <= 2e-10 * np.linalg.norm(b)
+    op.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["fp64", "fp32_ir"])
+def test_vector_cache_levels_identical_short_rows(ctx, mode):
+    """Short rows give the same bits whichever vectors stay on chip."""
+    from paper_2204_02064_gb300 import api
+    n = 30000
+    rp, c, v = _banded_spd(n, 3, 93)
+    b = torch.from_numpy(inputs.cg_rhs(n, 94)).cuda()
+    op = api.CsrOperator(ctx, torch.from_numpy(rp).cuda(), torch.from_numpy(c).cuda(), torch.from_numpy(v).cuda())
+    out = []
+    for level in (0, 1, 2):
+        op.set_vector_cache(level)
+        assert op.vector_cache_active == level
+        x = torch.zeros(n, dtype=torch.float64, device="cuda")
+        op.solve(b, x, rtol=1e-10, mode=mode)
+        out.append(x)
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+    op.close()
