@@ -47,6 +47,9 @@ struct PoissonArgs {
     unsigned long long *gbar;    // [groups] barrier counter of each block group
     int *gprob;                  // [groups] problem taken by each group
     double *gpart;               // [groups][2][C] block sums, double-buffered
+    double *slots;               // [groups][3][C] sums of exchange_sum, all empty before a launch
+    double *halo;                // [blocks][2][nx] p of the rows south and north of a block's rows
+    int on_chip;                 // each block keeps r of its rows in shared memory
     DevError *err;
     long long timeout_ns;
 };
@@ -365,6 +368,188 @@ __global__ void __launch_bounds__(NT, MINB) perks_poisson_cg_kernel(const __grid
     }
 }
 
+// The default solver: the recurrence of perks_poisson_cg_kernel<.., 1, 1, ..>,
+// cell by cell the same operations, laid out so that an iteration costs its
+// ten fp64 operations per cell and little else (the FP64 pipe, 2 lanes per
+// clock and SM, is the bound).
+//   * A block's cells are one run, taken NT at a time: with a row of threads
+//     per grid row, a 335-cell row left 177 of 512 lanes idle.
+//   * Two exchanges per iteration (exchange_sum: sum and barrier in one),
+//     where block sum, barrier, partial sums and another barrier took three
+//     barriers: p of the two rows next to a block's own is updated by the
+//     block itself, from the neighbours' r of those rows, which travels with
+//     the <r, r> exchange.
+//   * r stays in shared memory where a block's share fits, and the automatic
+//     group size (effective_group) makes it fit.
+// 64 problems of 512^2, 24 iterations: 11.8 ms with the kernel above, 10.5
+// here (the FP64 pipe's time is 6.7 ms); 16 problems of 83 x 368, 2.0 -> 0.5
+// ms; 202 problems of 64 x 81 to 1e-10, 61 -> 27 ms.
+template <int NT, bool GROUP>
+__global__ void __launch_bounds__(NT, 2) perks_poisson_run_kernel(const __grid_constant__ PoissonArgs a) {
+    extern __shared__ __align__(16) double poi_smem[];
+    double *red = poi_smem;                       // reduce_scratch<NT>()
+    double *rs = poi_smem + reduce_scratch<NT>();
+    __shared__ int s_prob;
+    const int nx = a.nx, ny = a.ny, tid = threadIdx.x;
+    const long long n = a.n;
+    const int C = GROUP ? a.group : 1;
+    const int g = blockIdx.x / C, rank = blockIdx.x % C;
+    int jb = 0, je = ny;
+    if (GROUP) group_rows<1>(ny, C, rank, jb, je);
+    const int cb = jb * nx, ce = je * nx;         // n fits an int: checked by the host
+    const bool has_s = GROUP && jb > 0, has_n = GROUP && je < ny;
+    double *hs = a.halo + (size_t)blockIdx.x * 2 * nx, *hn = hs + nx;
+    unsigned round = 0;
+    auto gsum = [&](double v, SumResult &out, auto &&post) -> bool {
+        if constexpr (GROUP)
+            return exchange_sum<NT>(a.slots + (size_t)g * 3 * C, C, rank, a.err, a.timeout_ns, round, v, red, out, post);
+        block_sum4<NT>(v, red, out, post);
+        return true;
+    };
+    auto plain = [](double, double &, int &) {};
+    const int di = NT % nx, dj = NT / nx;         // from a thread's cell to its next one
+    const int i0 = (cb + tid) % nx, j0 = (cb + tid) / nx;
+    // f(c, i, j) for the block's cells c = j nx + i
+    auto each_cell = [&](auto &&f) {
+        for (int c = cb + tid, i = i0, j = j0; c < ce; c += NT) {
+            f(c, i, j);
+            i += di;
+            j += dj;
+            if (i >= nx) { i -= nx; ++j; }
+        }
+    };
+    for (;;) {
+        if constexpr (GROUP) {
+            double pick = 0.0;
+            if (rank == 0 && tid == 0) pick = (double)atomicAdd(a.queue, 1);
+            SumResult got;
+            if (!gsum(pick, got, plain)) return;
+            if (tid == 0) s_prob = (int)got.total;
+        } else {
+            if (tid == 0) s_prob = atomicAdd(a.queue, 1);
+        }
+        __syncthreads();
+        const int pb = s_prob;
+        __syncthreads();
+        if (pb >= a.nprob) break;
+        const double *__restrict__ fxp = a.fx + (long long)pb * (nx + 1) * ny;
+        const double *__restrict__ fyp = a.fy + (long long)pb * nx * (ny + 1);
+        const double *__restrict__ dgp = a.dg + (long long)pb * n;
+        const double *__restrict__ b = a.b + pb * n;
+        double *x = a.x + pb * n, *rg = a.r + pb * n, *p = a.p + pb * n, *q = a.q + pb * n;
+        double *r = a.on_chip ? rs - cb : rg;
+        // (A v)_c; south / north: v of the cells below and above
+        auto apply = [&](int c, int i, int j, double vc, double west, double east, double south, double north) -> double {
+            const double fw = __ldg(fxp + c + j), fe = __ldg(fxp + c + j + 1);
+            const double fs = __ldg(fyp + c), fn = __ldg(fyp + c + nx);
+            double acc = __ldg(dgp + c) * vc;
+            if (i > 0) acc = fma(-fw, west, acc);
+            if (i + 1 < nx) acc = fma(-fe, east, acc);
+            if (j > 0) acc = fma(-fs, south, acc);
+            if (j + 1 < ny) acc = fma(-fn, north, acc);
+            return acc;
+        };
+        // r = b - A x, p = r (x from global memory: the neighbours' rows too); the rows the neighbours read of r
+        // go to global memory
+        auto residual = [&](double &bb, double &rr) {
+            each_cell([&](int c, int i, int j) {
+                const double west = i > 0 ? __ldcg(x + c - 1) : 0.0, east = i + 1 < nx ? __ldcg(x + c + 1) : 0.0;
+                const double south = j > 0 ? __ldcg(x + c - nx) : 0.0, north = j + 1 < ny ? __ldcg(x + c + nx) : 0.0;
+                const double bv = __ldg(b + c);
+                const double rv = bv - apply(c, i, j, __ldcg(x + c), west, east, south, north);
+                r[c] = rv;
+                p[c] = rv;
+                if (a.on_chip && (j == jb || j == je - 1)) rg[c] = rv;
+                bb = fma(bv, bv, bb);
+                rr = fma(rv, rv, rr);
+            });
+        };
+        // p of the neighbouring rows, from their r (start: p = r)
+        auto halo = [&](bool start, double beta) {
+            if (has_s)
+                for (int i = tid; i < nx; i += NT) {
+                    const double rv = __ldcg(rg + (long long)(jb - 1) * nx + i);
+                    hs[i] = start ? rv : fma(beta, hs[i], rv);
+                }
+            if (has_n)
+                for (int i = tid; i < nx; i += NT) {
+                    const double rv = __ldcg(rg + (long long)je * nx + i);
+                    hn[i] = start ? rv : fma(beta, hn[i], rv);
+                }
+        };
+        SumResult sum;
+        double bb = 0.0, rr = 0.0;
+        residual(bb, rr);
+        if (!gsum(bb, sum, plain)) return;
+        bb = sum.total;
+        const double tol2 = a.rtol * a.rtol * bb;
+        auto small = [&](double t, double &, int &flag) { flag = t <= tol2; };
+        if (!gsum(rr, sum, small)) return;
+        rr = sum.total;
+        int it = 0, status = PERKS_ERR_NOT_CONVERGED;
+        for (int restart = 0;; ++restart) {
+            if (sum.flag) { status = PERKS_OK; break; }
+            halo(true, 0.0);
+            __syncthreads();
+            bool converged = false;
+            while (it < a.max_iter) {
+                // q = A p, <p, q>
+                double pq = 0.0;
+                each_cell([&](int c, int i, int j) {
+                    const double pc = p[c];
+                    const double west = i > 0 ? p[c - 1] : 0.0, east = i + 1 < nx ? p[c + 1] : 0.0;
+                    const double south = j > jb ? p[c - nx] : has_s ? hs[i] : 0.0;
+                    const double north = j + 1 < je ? p[c + nx] : has_n ? hn[i] : 0.0;
+                    const double qc = apply(c, i, j, pc, west, east, south, north);
+                    q[c] = qc;
+                    pq = fma(pc, qc, pq);
+                });
+                if (!gsum(pq, sum, [&](double t, double &ratio, int &flag) {
+                        flag = !(t > 0.0) || !isfinite(t);
+                        ratio = rr / t;
+                    }))
+                    return;
+                if (sum.flag) { status = PERKS_ERR_BREAKDOWN; break; }
+                const double alpha = sum.ratio;
+                // x += alpha p, r -= alpha q, <r, r>
+                double rn = 0.0;
+                for (int c = cb + tid; c < ce; c += NT) {
+                    x[c] = fma(alpha, p[c], x[c]);
+                    const double rv = fma(-alpha, q[c], r[c]);
+                    r[c] = rv;
+                    if (GROUP && a.on_chip && (c < cb + nx || c >= ce - nx)) rg[c] = rv;
+                    rn = fma(rv, rv, rn);
+                }
+                if (!gsum(rn, sum, [&](double t, double &ratio, int &flag) { ratio = t / rr; flag = t <= tol2; }))
+                    return;
+                const double beta = sum.ratio;
+                // p = r + beta p
+                for (int c = cb + tid; c < ce; c += NT) p[c] = fma(beta, p[c], r[c]);
+                halo(false, beta);
+                __syncthreads();
+                rr = sum.total;
+                ++it;
+                if (sum.flag) { converged = true; break; }
+            }
+            if (status == PERKS_ERR_BREAKDOWN) break;
+            // true residual: the neighbours' x has to be there
+            if (GROUP && !gsum(0.0, sum, plain)) return;
+            double bdum = 0.0, rt = 0.0;
+            residual(bdum, rt);
+            if (!gsum(rt, sum, small)) return;
+            rr = sum.total;
+            if (sum.flag) { status = PERKS_OK; break; }
+            if (!converged || restart >= a.max_restarts) break;
+        }
+        if (rank == 0 && tid == 0) {
+            a.iters[pb] = it;
+            a.true_rel[pb] = bb > 0 ? sqrt(rr / bb) : sqrt(rr);
+            a.status[pb] = status;
+        }
+        __syncthreads();
+    }
+}
+
 // x <- alpha x per problem with alpha = <x, b> / <x, A x>: of all multiples
 // of the guess, the one closest to the solution in the A-norm (the energy
 // norm CG minimises), so a warm start scaled this way starts CG no farther
@@ -436,6 +621,8 @@ struct perks_poisson {
     unsigned long long *gbar = nullptr;
     int *gprob = nullptr;
     double *gpart = nullptr;
+    double *slots = nullptr;  // [2 x SMs][3]: every group's rounds of exchange_sum
+    double *halo = nullptr;   // [2 x SMs][2][nx]
     DevError *err = nullptr;
     int max_groups = 0;
 };
@@ -443,7 +630,7 @@ struct perks_poisson {
 namespace {
 void free_poisson(perks_poisson *P) {
     void *ptrs[] = {P->fx, P->fy, P->dg, P->b, P->x, P->r, P->p, P->q, P->queue, P->iters, P->status, P->true_rel,
-                    P->gbar, P->gprob, P->gpart, P->err};
+                    P->gbar, P->gprob, P->gpart, P->slots, P->halo, P->err};
     for (void *v : ptrs) if (v) cudaFree(v);
 }
 
@@ -466,8 +653,49 @@ PoissonArgs poisson_args(perks_poisson *P) {
     a.fx = P->fx; a.fy = P->fy; a.dg = P->dg; a.b = P->b; a.x = P->x; a.r = P->r; a.p = P->p; a.q = P->q;
     a.queue = P->queue; a.iters = P->iters; a.true_rel = P->true_rel; a.status = P->status;
     a.group = effective_group(P); a.gbar = P->gbar; a.gprob = P->gprob; a.gpart = P->gpart; a.err = P->err;
+    a.slots = P->slots; a.halo = P->halo;
     a.timeout_ns = P->ctx->timeout_ns;
     return a;
+}
+
+constexpr int kRunThreads = 512;
+
+// Dynamic shared memory of perks_poisson_run_kernel for groups of C blocks;
+// r on chip if the largest share fits in half of an SM.
+size_t run_smem(const perks_poisson *P, int C, int &on_chip) {
+    const size_t base = sizeof(double) * reduce_scratch<kRunThreads>();
+    const size_t rows = (size_t)(P->ny + C - 1) / C, r = sizeof(double) * rows * P->nx;
+    const size_t most = (size_t)std::min(P->ctx->smem_optin, P->ctx->smem_per_sm / 2 - 1024) - 64;
+    on_chip = base + r <= most;
+    return on_chip ? base + r : base;
+}
+
+// Blocks per problem of perks_poisson_run_kernel.  A batch of fewer problems
+// than the documented groups would fill the GPU with keeps those; otherwise
+// the group that finishes the batch in the fewest cycles by this model: a
+// block's iteration takes 5 cycles per cell (10 fp64 operations, 2 lanes per
+// clock and SM), twice that where two blocks share an SM, plus the exchanges,
+// which the other block of an SM hides; the batch takes ceil(problems /
+// groups) of the longest iterations.  512^2, 64 problems: 19 blocks per
+// problem, 16 groups, 4 full waves, where 38 groups of 8 leave the second
+// wave a third empty.
+int run_group(const perks_poisson *P) {
+    const int doc = effective_group(P), slots = 2 * P->ctx->sm_count;
+    if (P->n <= 8192 || (P->n >= 65536 && (long long)P->nprob * doc <= slots)) return doc;
+    double best = 1e300;
+    int bc = doc;
+    for (int C = 1; C <= std::min(P->ny, 64); ++C) {
+        const int groups = std::min(P->nprob, slots / C);
+        if (groups < 1) break;
+        int on_chip;
+        run_smem(P, C, on_chip);
+        const double m = (double)((P->ny + C - 1) / C) * P->nx * (on_chip ? 1.0 : 1.1);
+        const double ex = C > 1 ? 6000.0 : 3000.0;
+        const double t = groups * C > P->ctx->sm_count ? std::max(10.0 * m, 5.0 * m + ex) : 5.0 * m + ex;
+        const double total = (double)((P->nprob + groups - 1) / groups) * t;
+        if (total <= best) { best = total; bc = C; }
+    }
+    return bc;
 }
 }  // namespace
 
@@ -501,6 +729,8 @@ extern "C" perks_status perks_poisson_create(perks_context *ctx, int32_t nx, int
     if (e == cudaSuccess) e = cudaMalloc(&P->gbar, sizeof(unsigned long long) * P->max_groups);
     if (e == cudaSuccess) e = cudaMalloc(&P->gprob, sizeof(int) * P->max_groups);
     if (e == cudaSuccess) e = cudaMalloc(&P->gpart, sizeof(double) * 2 * kPoiMaxGroup * P->max_groups);
+    if (e == cudaSuccess) e = cudaMalloc(&P->slots, sizeof(double) * 3 * P->max_groups);
+    if (e == cudaSuccess) e = cudaMalloc(&P->halo, sizeof(double) * 2 * nx * P->max_groups);
     if (e == cudaSuccess) e = cudaMalloc(&P->err, sizeof(DevError));
     if (e == cudaSuccess && !on_device) {
         e = cudaMalloc(&kd, vb);
@@ -568,10 +798,27 @@ extern "C" perks_status perks_poisson_solve(perks_poisson *P, const double *b, d
     a.rtol = rtol;
     a.max_iter = max_iter;
     a.max_restarts = 8;
-    const int C = effective_group(P);
+    // group size and rows per pass by default: the run kernel
+    const bool run = P->group == 0 && P->rows_per_pass == 1 && P->n < (1LL << 30);
+    const int C = run ? run_group(P) : effective_group(P);
     const bool grouped = C > 1;
     const void *kern;
-    if (P->rows_per_pass == 1)  // two 512-thread blocks per SM, one row per pass
+    size_t smem = 0;
+    int threads = P->block_threads;
+    a.group = C;
+    if (run) {
+        kern = grouped ? (const void *)perks_poisson_run_kernel<kRunThreads, true>
+                       : (const void *)perks_poisson_run_kernel<kRunThreads, false>;
+        threads = kRunThreads;
+        smem = run_smem(P, C, a.on_chip);
+        int budget = 0;
+        rc = smem_optin(ctx, kern, &budget);
+        if (rc) return rc;
+        if (smem > (size_t)budget) {
+            a.on_chip = 0;
+            smem = sizeof(double) * reduce_scratch<kRunThreads>();
+        }
+    } else if (P->rows_per_pass == 1)  // two 512-thread blocks per SM, one row per pass
         kern = grouped ? (const void *)perks_poisson_cg_kernel<512, 2, 1, 1, true>
                        : (const void *)perks_poisson_cg_kernel<512, 2, 1, 1, false>;
     else if (P->block_threads == 512)
@@ -581,13 +828,14 @@ extern "C" perks_status perks_poisson_solve(perks_poisson *P, const double *b, d
         kern = grouped ? (const void *)perks_poisson_cg_kernel<kPoiThreads, 2, kRows, kLin, true>
                        : (const void *)perks_poisson_cg_kernel<kPoiThreads, 2, kRows, kLin, false>;
     int per_sm = 0;
-    PERKS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, P->block_threads, 0));
+    PERKS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
+    if (run) per_sm = std::min(per_sm, 2);
     if (per_sm < 1) return fail(ctx, PERKS_ERR_LAUNCH_TOO_LARGE, "poisson_solve: kernel cannot be resident");
     void *kargs[] = {(void *)&a};
     int grid;
     if (!grouped) {
         grid = std::max(1, std::min(P->nprob, per_sm * ctx->sm_count));
-        PERKS_CUDA(ctx, cudaLaunchKernel(kern, dim3(grid), dim3(P->block_threads), kargs, 0, s));
+        PERKS_CUDA(ctx, cudaLaunchKernel(kern, dim3(grid), dim3(threads), kargs, smem, s));
     } else {
         // groups wait on one another's blocks: every block resident (cooperative launch)
         const int groups = std::min({P->nprob, per_sm * ctx->sm_count / C, P->max_groups});
@@ -595,7 +843,8 @@ extern "C" perks_status perks_poisson_solve(perks_poisson *P, const double *b, d
         grid = groups * C;
         PERKS_CUDA(ctx, cudaMemsetAsync(P->gbar, 0, sizeof(unsigned long long) * groups, s));
         PERKS_CUDA(ctx, cudaMemsetAsync(P->err, 0, sizeof(DevError), s));
-        PERKS_CUDA(ctx, cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(P->block_threads), kargs, 0, s));
+        if (run) PERKS_CUDA(ctx, cudaMemsetAsync(P->slots, 0xff, sizeof(double) * 3 * grid, s));
+        PERKS_CUDA(ctx, cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), kargs, smem, s));
     }
     PERKS_CUDA(ctx, cudaMemcpyAsync(x, P->x, vb, cudaMemcpyDeviceToDevice, s));
     if (!stats) return PERKS_OK;

@@ -207,3 +207,31 @@ def test_one_row_per_pass_matches_oracle(ctx, oracle, group):
     with pytest.raises(api.PerksError):
         P.set_rows_per_pass(3)
     P.close()
+
+
+@pytest.mark.parametrize("nprob,ny,nx", [(40, 100, 130), (3, 97, 151), (90, 129, 65), (2, 1, 9000), (310, 40, 33),
+                                         (41, 256, 257)])
+def test_automatic_groups_match_oracle(ctx, oracle, nprob, ny, nx):
+    """The default solver over the shares of rows its group sizes give (one
+    block, ragged rows per block, one row, a share too large for shared
+    memory): the iterate after 24 iterations and the solution agree with the
+    oracle's CG.  Tolerance of the iterate: the rounding of 24 steps times the
+    largest condition number here (9000^2 x 4 / pi^2 = 3e7), 24 x 3e7 x 2^-53."""
+    from paper_2204_02064_gb300 import api
+    k = _k(nprob, ny, nx, 19)
+    f = 2.0 * inputs.uniform(20, nprob * ny * nx).reshape(nprob, ny, nx) - 1.0
+    P = api.Poisson(ctx, torch.from_numpy(k).cuda())
+    x = torch.zeros(nprob, ny, nx, dtype=torch.float64, device="cuda")
+    x24 = torch.zeros_like(x)
+    P.solve(torch.from_numpy(f).cuda(), x24, rtol=1e-30, max_iter=24, stats=False)
+    torch.cuda.synchronize()
+    res = P.solve(torch.from_numpy(f).cuda(), x, rtol=1e-8)
+    xs = x.cpu().numpy()
+    assert res["max_true_rel_residual"] <= 1e-8
+    for i in sorted({0, nprob // 2, nprob - 1}):
+        rp, c, val = oracle.poisson_csr(k[i])
+        ref = oracle.cg(rp, c, val, f[i].ravel(), rtol=1e-30, max_iter=24)
+        assert np.linalg.norm(x24[i].cpu().numpy().ravel() - ref["x"]) <= 1e-7 * np.linalg.norm(ref["x"])
+        ref = oracle.cg(rp, c, val, f[i].ravel(), rtol=1e-8, max_iter=20000)
+        assert np.linalg.norm(xs[i].ravel() - ref["x"]) <= 1e-6 * np.linalg.norm(ref["x"])
+    P.close()
