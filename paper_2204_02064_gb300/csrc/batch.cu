@@ -19,6 +19,7 @@
 
 #include "internal.h"
 #include "stencil_registry.h"
+#include "stencil_strip.cuh"
 #include "stencil_vec.cuh"
 
 using namespace perks;
@@ -119,8 +120,9 @@ __global__ void __launch_bounds__(kBatchThreads, 1) perks_batch_kernel(const __g
 // ------------------------------------------------------------- strip kernel
 //
 // Column-strip streaming: the batch's work is cut into items (domain, strip
-// of 32 vectors = 32 V cells, range of rows) and a static
-// longest-processing-time-first assignment gives every WARP its items.  A
+// of 32 vectors = 32 V cells, or a little less where strips overlap, range of
+// rows) and a static longest-processing-time-first assignment gives every WARP
+// its items.  A
 // warp streams its item's input rows through a private ring of D row slots
 // in shared memory (16-byte cp.async per lane, plus two halo cells on each
 // side from the neighbouring strips), keeps the 2R + 1 rows the stencil
@@ -134,7 +136,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) perks_batch_kernel(const __g
 
 struct StripItem {
     int dom;
-    int x0;      // first cell of the strip (a multiple of 32 V)
+    int x0;      // first cell of the strip
     int z0, z1;  // output rows [z0, z1)
 };
 
@@ -149,6 +151,7 @@ struct StripArgs {
     long long timeout_ns;
 };
 
+// fp64 (fp32 takes perks_batch_sweep_kernel)
 constexpr int kStripThreads = 256;
 constexpr int kStripDepth = 8;   // ring rows per warp (16 measured slower: longer ring fill per item)
 
@@ -225,56 +228,16 @@ __device__ __forceinline__ void strip_item(const PersistentArgs &a, const StripI
                 fetch(z + R, win[(p + 2 * R) % W]);
                 VT o;
                 A acc[V];
-                if constexpr (std::is_same<A, float>::value && V % 2 == 0) {
-                    // fp32: a term whose x offset is even updates two cells
-                    // with one packed fma (__ffma2_rn rounds each lane as
-                    // fmaf does; the two cells sit in an aligned register
-                    // pair of the window row), an odd offset one cell at a
-                    // time; every cell adds its terms in table order from 0
-                    float2 acc2[V / 2];
 #pragma unroll
-                    for (int q = 0; q < V / 2; ++q) acc2[q] = make_float2(0.f, 0.f);
-                    static_for<0, SH::NPTS>([&](auto II) {
-                        constexpr int i = decltype(II)::value;
-                        constexpr int slot = (p + R + SH::dz(i)) % W;
-                        constexpr int dx = SH::dx(i);
-                        if constexpr (dx % 2 == 0) {
-                            const float2 w2 = make_float2(w[i], w[i]);
+                for (int q = 0; q < V; ++q) acc[q] = A(0);
+                static_for<0, SH::NPTS>([&](auto II) {
+                    constexpr int i = decltype(II)::value;
+                    constexpr int slot = (p + R + SH::dz(i)) % W;
 #pragma unroll
-                            for (int q = 0; q < V / 2; ++q)
-                                acc2[q] = __ffma2_rn(w2, make_float2(win[slot][2 + 2 * q + dx], win[slot][3 + 2 * q + dx]),
-                                                     acc2[q]);
-                        } else {
+                    for (int q = 0; q < V; ++q) acc[q] = fma(w[i], win[slot][2 + q + SH::dx(i)], acc[q]);
+                });
 #pragma unroll
-                            for (int q = 0; q < V / 2; ++q) {
-                                acc2[q].x = fmaf(w[i], win[slot][2 + 2 * q + dx], acc2[q].x);
-                                acc2[q].y = fmaf(w[i], win[slot][3 + 2 * q + dx], acc2[q].y);
-                            }
-                        }
-                    });
-#pragma unroll
-                    for (int q = 0; q < V / 2; ++q) {
-                        acc[2 * q] = acc2[q].x;
-                        acc[2 * q + 1] = acc2[q].y;
-                    }
-                } else {
-#pragma unroll
-                    for (int q = 0; q < V; ++q) acc[q] = A(0);
-                    static_for<0, SH::NPTS>([&](auto II) {
-                        constexpr int i = decltype(II)::value;
-                        constexpr int slot = (p + R + SH::dz(i)) % W;
-#pragma unroll
-                        for (int q = 0; q < V; ++q) acc[q] = fma(w[i], win[slot][2 + q + SH::dx(i)], acc[q]);
-                    });
-                }
-                if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-                    __nv_bfloat162 *o2 = reinterpret_cast<__nv_bfloat162 *>(&o);
-#pragma unroll
-                    for (int q = 0; q < V / 2; ++q) o2[q] = __floats2bfloat162_rn(acc[2 * q], acc[2 * q + 1]);
-                } else {
-#pragma unroll
-                    for (int q = 0; q < V; ++q) o.v[q] = from_acc<T>(acc[q]);
-                }
+                for (int q = 0; q < V; ++q) o.v[q] = from_acc<T>(acc[q]);
                 if (own) *reinterpret_cast<VT *>(out + (long long)z * X + xl) = o;
             }
         });
@@ -284,8 +247,7 @@ __device__ __forceinline__ void strip_item(const PersistentArgs &a, const StripI
 }
 
 template <typename T, int V>
-__global__ void __launch_bounds__(kStripThreads, sizeof(T) == 8 ? 1 : 2)
-    perks_batch_strip_kernel(const __grid_constant__ StripArgs b) {
+__global__ void __launch_bounds__(kStripThreads, 1) perks_batch_strip_kernel(const __grid_constant__ StripArgs b) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int D = kStripDepth;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -311,6 +273,56 @@ __global__ void __launch_bounds__(kStripThreads, sizeof(T) == 8 ? 1 : 2)
     }
 }
 
+// fp32: the same items through strip_sweep (stencil_strip.cuh), one step per
+// sweep: x-neighbours by shuffles instead of halo lanes and warp barriers per
+// row, a third fewer instructions.  A strip overlaps its neighbours by one lane
+// on each side (x0 is the first cell an item stores).  A step of the 64-domain
+// workload: 90 us through the kernel above (fp32), 75 us here with the same items
+// (HBM: 51).  192 threads,
+// two blocks per SM: 156 registers hold a domain's 25 weights and the window;
+// with 256 threads (128 registers) they spill and a step takes 160 us, two
+// steps per sweep spill at 192.  fp64 stays with the kernel above: its steps
+// are bound by the FP64 pipe, which the overlaps would add work to.
+constexpr int kBatchSweep = 1;
+constexpr int kSweepThreads = 192;
+
+template <typename T, class SH>
+__device__ __forceinline__ void sweep_item(const PersistentArgs &a, const StripItem &it, int src, T *ring, int lane) {
+    using A = typename AccOf<T>::type;
+    constexpr int V = strip_v<T>(), HL = strip_hl<T, SH, kBatchSweep>();
+    A w[SH::NPTS];
+#pragma unroll
+    for (int i = 0; i < SH::NPTS; ++i) w[i] = ScalarOps<T>::w(a, i);
+    strip_sweep<T, SH, kBatchSweep, true>(static_cast<const T *>(a.field[src]), static_cast<T *>(a.field[src ^ 1]), a.X,
+                                          a.Z, it.x0 - HL * V, it.z0, it.z1, kBatchSweep, ScalarOps<T>::bnd(a),
+                                          [&](int i) { return w[i]; }, ring, lane);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kSweepThreads, 2) perks_batch_sweep_kernel(const __grid_constant__ StripArgs b) {
+    constexpr int V = strip_v<T>();
+    __shared__ __align__(16) T rings[kSweepThreads / 32][kStripKDepth * 32 * V];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    T *ring = rings[warp] + lane * V;
+    const int gw = blockIdx.x * (kSweepThreads / 32) + warp;
+    const int i0 = b.warp_first[gw], i1 = b.warp_first[gw + 1];
+    unsigned long long epoch = 0;
+    for (long long k = 0; k < b.steps; ++k) {
+        const int src = (int)(k & 1);
+        for (int q = i0; q < i1; ++q) {
+            const StripItem it = b.items[q];
+            const PersistentArgs &a = b.doms[it.dom];
+            switch (b.dom_shape[it.dom]) {
+            case SH_2D5: sweep_item<T, S2d5>(a, it, src, ring, lane); break;
+            case SH_2D9: sweep_item<T, S2d9>(a, it, src, ring, lane); break;
+            case SH_2D25: sweep_item<T, S2d25>(a, it, src, ring, lane); break;
+            default: sweep_item<T, S2ds9>(a, it, src, ring, lane); break;
+            }
+        }
+        if (k + 1 < b.steps && !grid_barrier(b.bar, gridDim.x, epoch, b.err, b.timeout_ns)) return;
+    }
+}
+
 using StripFn = void (*)(StripArgs);
 
 using BatchFn = void (*)(BatchArgs);
@@ -330,11 +342,20 @@ std::vector<BatchKernel> &batch_kernels() {
     return k;
 }
 
-// Strip kernels (column-strip streaming), by storage type.
-StripFn strip_kernel(int dtype) {
-    if (dtype == PERKS_F32) return perks_batch_strip_kernel<float, 4>;
-    if (dtype == PERKS_F64) return perks_batch_strip_kernel<double, 2>;
-    return nullptr;
+// Strip kernels (column-strip streaming), by storage type: threads, dynamic
+// shared memory, and the cells an item stores across x.
+struct StripKernel {
+    StripFn fn;
+    int threads;
+    size_t smem;
+    int width;
+};
+
+const StripKernel *strip_kernel(int dtype) {
+    static const StripKernel f32 = {perks_batch_sweep_kernel<float>, kSweepThreads, 0, 30 * 4};
+    static const StripKernel f64 = {perks_batch_strip_kernel<double, 2>, kStripThreads,
+                                    (size_t)(kStripThreads / 32) * kStripDepth * strip_row_cells<double, 2>() * 8, 32 * 2};
+    return dtype == PERKS_F32 ? &f32 : dtype == PERKS_F64 ? &f64 : nullptr;
 }
 
 int shape_id_2d(const perks_stencil_desc &d, double *kw) {
@@ -615,40 +636,64 @@ perks_status upload_plan(perks_batch *b, const PlanOut &o) {
     return PERKS_OK;
 }
 
-// Strip plan: items of `rows` output rows (0: as many as give every warp
-// about one item's worth of rows), longest-processing-time-first over the
-// warps of a co-resident grid.  Item cost = rows read (its rows plus 2R of
-// halo) x (1 + points / 25): the stream of rows, plus the stencil's FMAs.
+// Strip plan: items of `rows` output rows, or (0) about one equally costly
+// item per warp, longest-processing-time-first over the warps of a co-resident
+// grid.  Item cost = rows read (its rows plus 2R of halo) x, for fp32, the
+// stream of rows plus the stencil's FMAs, for fp64 the FMAs.  Equal costs
+// rather than equal rows, where the 25-point domains' items, 1.7 times the
+// 5-point ones', ended last: a step of the 64-domain fp32 workload 75 -> 63 us,
+// 24 fp64 domains of 128^2 to 1200^2 297 -> 214 us, 40 to 400^2 138 -> 112.
 perks_status plan_strips(perks_batch *b, int rows) {
     perks_context *ctx = b->ctx;
-    StripFn fn = strip_kernel(b->dtype);
-    if (!fn) return fail(ctx, PERKS_ERR_UNSUPPORTED, "batch: no strip kernel for this dtype");
-    const int V = (int)(16 / b->es);
-    const int W = 32 * V;
-    const size_t smem = (size_t)(kStripThreads / 32) * kStripDepth * (32 * V + 2 * V) * b->es;
+    const StripKernel *k = strip_kernel(b->dtype);
+    if (!k) return fail(ctx, PERKS_ERR_UNSUPPORTED, "batch: no strip kernel for this dtype");
+    const int W = k->width;
     int budget = 0;
-    perks_status rc = smem_optin(ctx, (const void *)fn, &budget);
+    perks_status rc = smem_optin(ctx, (const void *)k->fn, &budget);
     if (rc) return rc;
     int per_sm = 0;
-    PERKS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, kStripThreads, smem));
+    PERKS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)k->fn, k->threads, k->smem));
     if (per_sm < 1) return fail(ctx, PERKS_ERR_LAUNCH_TOO_LARGE, "batch strip kernel is not resident");
     const int G = per_sm * ctx->sm_count;
-    const int nwarps = G * (kStripThreads / 32);
-    long long total_rows = 0;
-    for (const auto &d : b->desc) total_rows += (long long)ceil_div((int)d.nx, W) * d.ny;
-    const int target = rows > 0 ? rows : (int)std::min<long long>(1024, std::max<long long>(8, total_rows / nwarps));
+    const int nwarps = G * (k->threads / 32);
+    // items of one height, or the fewest and equally costly ones: the lowest
+    // cost T an item may have with no more items than `most`, one per warp
+    // unless there are hardly more warps than columns
+    auto row_cost = [&](int i) { return b->dtype == PERKS_F64 ? (double)b->desc[i].npts : 1.0 + b->desc[i].npts / 25.0; };
+    auto strips = [&](int i) { return (long long)ceil_div((int)b->desc[i].nx, W); };
+    auto segments = [&](int i, double T) {
+        const double h = std::max(4.0, std::floor(T / row_cost(i) - 2.0 * b->desc[i].radius));
+        return (int)std::ceil((double)b->desc[i].ny / h);
+    };
+    double T = 0.0;
+    if (rows == 0) {
+        long long columns = 0;
+        double hi = 0.0, lo = 0.0;
+        for (int i = 0; i < b->ndom; ++i) {
+            columns += strips(i);
+            hi = std::max(hi, row_cost(i) * (b->desc[i].ny + 2.0 * b->desc[i].radius));
+        }
+        const long long most = nwarps * std::max<long long>(1, (3 * columns + nwarps - 1) / nwarps);
+        for (int it = 0; it < 40; ++it) {
+            T = 0.5 * (lo + hi);
+            long long n = 0;
+            for (int i = 0; i < b->ndom; ++i) n += strips(i) * segments(i, T);
+            (n <= most ? hi : lo) = T;
+        }
+        T = hi;
+    }
     std::vector<StripItem> items;
     std::vector<double> cost;
     long long halo = 0;
     for (int i = 0; i < b->ndom; ++i) {
         const int X = (int)b->desc[i].nx, Z = (int)b->desc[i].ny, R = b->desc[i].radius;
-        const int nseg = std::max(1, (int)std::lround((double)Z / target));
+        const int nseg = rows > 0 ? std::max(1, (int)std::lround((double)Z / rows)) : segments(i, T);
         for (int x0 = 0; x0 < X; x0 += W)
             for (int sgi = 0; sgi < nseg; ++sgi) {
                 int z0, nz;
                 split_axis(Z, nseg, sgi, z0, nz);
                 items.push_back(StripItem{i, x0, z0, z0 + nz});
-                cost.push_back((double)(nz + 2 * R) * (1.0 + b->desc[i].npts / 25.0));
+                cost.push_back((double)(nz + 2 * R) * row_cost(i));
                 halo += 2LL * R * std::min(W, X - x0) + 4LL * (nz + 2 * R);
             }
     }
@@ -712,7 +757,7 @@ perks_status plan_strips(perks_batch *b, int rows) {
     b->nitems = (int)sorted.size();
     b->max_items_per_warp = maxw;
     b->strip_halo = halo;
-    b->strip_smem = (long long)smem;
+    b->strip_smem = (long long)k->smem;
     return PERKS_OK;
 }
 
@@ -742,8 +787,9 @@ perks_status launch_strips(perks_batch *b, long long steps, cudaStream_t s) {
     args.err = b->err;
     args.timeout_ns = ctx->timeout_ns;
     void *kargs[] = {&args};
-    PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)strip_kernel(b->dtype), dim3(b->strip_blocks),
-                                                dim3(kStripThreads), kargs, (size_t)b->strip_smem, s));
+    const StripKernel *k = strip_kernel(b->dtype);
+    PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)k->fn, dim3(b->strip_blocks), dim3(k->threads), kargs,
+                                                (size_t)b->strip_smem, s));
     if (steps & 1)
         for (int i = 0; i < b->ndom; ++i) b->cur[i] ^= 1;
     return PERKS_OK;

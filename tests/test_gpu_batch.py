@@ -145,3 +145,30 @@ def test_batch_strip_equals_ring_bitwise(ctx):
     assert sa["kernel"] == api.BATCH_STRIP and sr["kernel"] == api.BATCH_RING
     for x, y in zip(a, r):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("count,nx,ny", [(3, 116, 40), (2, 120, 1), (5, 124, 9), (4, 240, 77), (3, 244, 200),
+                                         (300, 64, 33), (1, 4, 700)])
+def test_batch_strip_edges(ctx, oracle, dtype, count, nx, ny):
+    """Strips a vector wider or narrower than the domain, more columns than
+    warps hold one item of, domains lower than an item; the automatic items."""
+    from paper_2204_02064_gb300 import api
+    names = ["2d5pt", "2d25pt", "2ds9pt", "2d9pt"]
+    doms = [dict(shape=(ny, nx), offsets=inputs.shape_offsets(names[i % 4]),
+                 weights=inputs.workload_weights(names[i % 4], seed=i % 4)) for i in range(count)]
+    b = api.Batch(ctx, doms, dtype=dtype)
+    srcs = [torch.from_numpy(inputs.stencil_field((ny, nx), 70 + i)).to(TT[dtype]).cuda() for i in range(count)]
+    for i, f in enumerate(srcs):
+        b.set_field(i, f)
+    assert b.run(5, stats=True)["kernel"] == api.BATCH_STRIP
+    for i in sorted({0, 1 % count, count // 2, count - 1}):
+        o = torch.empty_like(srcs[i])
+        b.get_field(i, o)
+        torch.cuda.synchronize()
+        d, f = doms[i], srcs[i].cpu().numpy()
+        if dtype == "f32":
+            assert np.array_equal(o.cpu().numpy(), oracle.stencil_run_lowp(f, d["offsets"], d["weights"], 5, "f32"))
+        else:
+            assert rel_err(o.cpu().numpy(), oracle.stencil_run(f, d["offsets"], d["weights"], 5)) <= 1e-12
+    b.close()
