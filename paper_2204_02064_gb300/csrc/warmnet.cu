@@ -522,101 +522,147 @@ __global__ void __launch_bounds__(256) reduce_grad_kernel(const float *__restric
 }
 
 // A column's share of a coarse cell's mean log: the product of the values'
-// significands (each in [1, 2), so at most 2^32 for 32 rows), the sum of their
-// exponents, and the logarithms of the values that are not normal positive
-// numbers (0, subnormal, negative, infinite, NaN), which log itself answers.
+// significands (each in [1, 2)), the sum of their exponents, and the
+// logarithms of the values that are not normal positive numbers (0, subnormal,
+// negative, infinite, NaN), which log itself answers.  The product is a 64-bit
+// fixed-point number m 2^-63 2^e, multiplied by the integer units: eleven more
+// bits than fp64 carries, without the FP64 pipe.  A factor takes up to one bit
+// of m, which normalise() returns after eight of them, so a factor's
+// truncation is at most 2^-55 of the product.
 struct LogProd {
-    double m = 1.0, s = 0.0;
+    unsigned long long m = 1ull << 63;
+    double s = 0.0;
     int e = 0;
+    __device__ __forceinline__ void mul_significand(unsigned long long sig) {  // sig 2^-63 in [1, 2)
+        m = __umul64hi(m, sig);
+        e += 1;
+    }
     __device__ __forceinline__ void mul(double v) {
         const int hi = __double2hiint(v);
-        if (hi >= 0x00100000 && hi < 0x7ff00000) {
+        if ((unsigned)(hi - 0x00100000) < 0x7fe00000u) {
             e += (hi >> 20) - 1023;
-            m *= __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(v));
+            mul_significand(((unsigned long long)__double_as_longlong(v) << 11) | (1ull << 63));
         } else {
             s += log(v);
         }
     }
-    __device__ __forceinline__ void normalise() {  // m back into [1, 2)
-        const int hi = __double2hiint(m);
-        e += (hi >> 20) - 1023;
-        m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(m));
+    __device__ __forceinline__ void normalise() {  // m back into [2^63, 2^64)
+        const int n = __clzll((long long)m);
+        m <<= n;
+        e -= n;
     }
-    __device__ __forceinline__ double value() const { return fma((double)e, 0.69314718055994530942, log(m)) + s; }
+    // sum of the logarithms; m normalised
+    __device__ __forceinline__ double value() const {
+        const double d = __ull2double_rn(m);  // in [2^63, 2^64]
+        const double x = __hiloint2double(__double2hiint(d) - (63 << 20), __double2loint(d));
+        return fma((double)e, 0.69314718055994530942, log(x)) + s;
+    }
 };
 
 constexpr int kPoolThreads = 256;
+constexpr int kPoolJobs = 8;  // jobs per round, at most
+
+// Dynamic shared memory of a round of nj jobs: every column's sums.
+size_t pool_smem(int nj, bool train) { return (size_t)nj * kPoolThreads * (3 * 8 + 4 + (train ? 8 : 0)); }
 
 // Network input: channel 0 = log k, channel 1 = f, each averaged over the
 // F x F fine cells of a coarse cell (F = 1: the cells themselves); with u also
 // the training target ut, the mean of u over the same cells.
 //
-// Bound: HBM (16 or 24 B per fine cell) once the logarithms are out of the
-// way: a coarse cell's mean log is one log of the product of its F^2
-// significands plus the exponents' sum times ln 2, so a fine cell costs one
-// fp64 multiply instead of one log (about 25 fp64 operations on a pipe of two
-// per clock and SM).  A block takes a run of whole coarse cells of one coarse
-// row: thread t reads fine column t of the F rows (coalesced, 2 F loads in
-// flight), then one thread per coarse cell combines its F columns.
-// 256 images of 512^2, F = 8: 4140 -> 548 us.
+// Bound: HBM (16 or 24 B per fine cell) and the FP64 pipe (two operations per
+// clock and SM: one addition per fine cell, some 50 per coarse cell), once the
+// logarithms are out of the way: a coarse cell's mean log is one log of the
+// product of its F^2 significands plus the exponents' sum times ln 2, and the
+// product is the integer units'.  A job is a run of whole coarse cells of one
+// coarse row: thread t reads fine column t of the F rows (coalesced, 16 loads
+// in flight).  After a round of nj jobs one thread per coarse cell combines
+// its F columns, so that all warps take part in the logarithms: an fp64
+// instruction holds a quarter of the SM for 64 cycles, and with a round per job
+// one warp's chain of them held up the other seven.  256 images of 512^2, F = 8:
+// 4140 us with a log per fine cell, 548 with fp64 products, a load per use and
+// warp 0 combining every job, 270 now (FP64 pipe 74 % busy).
 template <typename S>
-__global__ void __launch_bounds__(kPoolThreads) features_kernel(const double *__restrict__ k,
-                                                               const double *__restrict__ f,
-                                                               const double *__restrict__ u, S *__restrict__ x0,
-                                                               double *__restrict__ ut, int ny, int nx, int F,
-                                                               int nimg) {
-    __shared__ double s_m[kPoolThreads], s_s[kPoolThreads], s_f[kPoolThreads], s_u[kPoolThreads];
-    __shared__ int s_e[kPoolThreads];
+__global__ void __launch_bounds__(kPoolThreads, 3) features_kernel(const double *__restrict__ k,
+                                                                  const double *__restrict__ f,
+                                                                  const double *__restrict__ u, S *__restrict__ x0,
+                                                                  double *__restrict__ ut, int ny, int nx, int F,
+                                                                  int njobs, int nj) {
+    extern __shared__ __align__(16) unsigned char pool_raw[];
+    unsigned long long *s_m = reinterpret_cast<unsigned long long *>(pool_raw);
+    double *s_s = reinterpret_cast<double *>(s_m + nj * kPoolThreads), *s_f = s_s + nj * kPoolThreads;
+    double *s_u = s_f + nj * kPoolThreads;        // with u only
+    int *s_e = reinterpret_cast<int *>(u ? s_u + nj * kPoolThreads : s_u);
     const int H = ny / F, W = nx / F;
     const long long plane = (long long)H * W;
     const double inv = 1.0 / ((double)F * F);
-    const int cells = kPoolThreads / F;           // coarse cells per block
+    const int cells = kPoolThreads / F;           // coarse cells per job
     const int nchunk = (W + cells - 1) / cells;
-    const long long total = (long long)nimg * H * nchunk;
     const int t = threadIdx.x;
-    for (long long job = blockIdx.x; job < total; job += gridDim.x) {
-        const int X0 = (int)(job % nchunk) * cells;
-        const long long row = job / nchunk;       // img * H + Y
-        const int ncell = min(cells, W - X0);
-        if (t < ncell * F) {
-            const long long c0 = row * F * nx + (long long)X0 * F + t;
-            LogProd lp;
-            double ff = 0.0, uu = 0.0, kv = 0.0;
+    for (int first = blockIdx.x * nj; first < njobs; first += gridDim.x * nj) {
+        const int n = min(nj, njobs - first);
+        for (int i = 0; i < n; ++i) {
+            const int row = (first + i) / nchunk, X0 = (first + i) % nchunk * cells;  // row: img * H + Y
+            if (t < min(cells, W - X0) * F) {
+                const long long c0 = (long long)row * F * nx + (long long)X0 * F + t;
+                LogProd lp;
+                double ff = 0.0, uu = 0.0, kv = 0.0;
+                for (int dy0 = 0; dy0 < F; dy0 += 8) {
+                    double kr[8], fr[8];          // all eight rows' loads before the first is used
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (dy0 + j < F) {
+                            kr[j] = k[c0 + (long long)(dy0 + j) * nx];
+                            fr[j] = f[c0 + (long long)(dy0 + j) * nx];
+                        }
+                    kv = kr[0];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (dy0 + j < F) {
+                            if (F > 1) lp.mul(kr[j]);
+                            ff += fr[j];
+                        }
+                    lp.normalise();
+                }
+                if (u)
 #pragma unroll 8
-            for (int dy = 0; dy < F; ++dy) {
-                kv = k[c0 + (long long)dy * nx];
-                lp.mul(kv);
-                ff += f[c0 + (long long)dy * nx];
+                    for (int dy = 0; dy < F; ++dy) uu += u[c0 + (long long)dy * nx];
+                const int q = i * kPoolThreads + t;
+                s_m[q] = lp.m;
+                s_s[q] = F > 1 ? lp.s : kv;
+                s_e[q] = lp.e;
+                s_f[q] = ff;
+                if (u) s_u[q] = uu;
             }
-            if (u)
-#pragma unroll 8
-                for (int dy = 0; dy < F; ++dy) uu += u[c0 + (long long)dy * nx];
-            if (F > 1) lp.normalise();
-            s_m[t] = F > 1 ? lp.m : kv;
-            s_s[t] = lp.s;
-            s_e[t] = lp.e;
-            s_f[t] = ff;
-            s_u[t] = uu;
         }
         __syncthreads();
-        if (t < ncell) {
+        for (int c = t; c < n * cells; c += kPoolThreads) {
+            const int i = c / cells, cell = c % cells;
+            const int row = (first + i) / nchunk, X = (first + i) % nchunk * cells + cell;
+            if (X >= W) continue;
+            const int q0 = i * kPoolThreads + cell * F;
             double lk, ff = 0.0, uu = 0.0;
             if (F == 1) {
-                lk = log(s_m[t]);
-                ff = s_f[t];
-                uu = s_u[t];
+                lk = log(s_s[q0]);
+                ff = s_f[q0];
+                if (u) uu = s_u[q0];
             } else {
                 LogProd lp;
-                for (int dx = 0; dx < F; ++dx) {
-                    lp.m *= s_m[t * F + dx];
-                    lp.s += s_s[t * F + dx];
-                    lp.e += s_e[t * F + dx];
-                    ff += s_f[t * F + dx];
-                    uu += s_u[t * F + dx];
+                for (int dx0 = 0; dx0 < F; dx0 += 8) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (dx0 + j < F) {
+                            const int q = q0 + dx0 + j;
+                            lp.mul_significand(s_m[q]);
+                            lp.e += s_e[q];
+                            if (__double_as_longlong(s_s[q]) != 0) lp.s += s_s[q];
+                            ff += s_f[q];
+                            if (u) uu += s_u[q];
+                        }
+                    lp.normalise();
                 }
                 lk = lp.value();
             }
-            const long long img = row / H, p = (row % H) * W + X0 + t;
+            const long long img = row / H, p = (long long)(row % H) * W + X;
             x0[(img * 2 + 0) * plane + p] = st_f<S>((float)(lk * inv));
             x0[(img * 2 + 1) * plane + p] = st_f<S>((float)(ff * inv));
             if (u) ut[img * plane + p] = uu * inv;
@@ -628,22 +674,41 @@ __global__ void __launch_bounds__(kPoolThreads) features_kernel(const double *__
 constexpr int kUpThreads = 128;
 constexpr int kUpRows = 64;  // fine rows per thread, about
 
+// (double)x and isfinite(x) by the integer units: a conversion or comparison
+// of doubles is an instruction of the FP64 pipe.
+// The rare cases stay out of line: inlined they are evaluated for every value
+// and one of the two results picked.
+__device__ __noinline__ double widen_special(float x) { return (double)x; }
+__device__ __noinline__ double two_weights(double w, double a, double b) { return (1.0 - w) * a + w * b; }
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), e = b & 0x7f800000u;
+    if (e == 0u ? b << 1 != 0u : e == 0x7f800000u) return widen_special(x);  // subnormal, infinite, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | (e == 0u ? 0u : (b >> 3 & 0x0fffffffu) + 0x38000000u)),
+                            (int)(b << 29));
+}
+__device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
 // u = scale * bilinear interpolation of the coarse output at the fine cell
 // centres (coarse cell centres at (Y + 1/2) F - 1/2, clamped at the edges).
 //
-// Bound: HBM writes (8 B per fine cell).  A thread owns V neighbouring fine
+// Bound: the FP64 pipe (HBM writes of 8 B per fine cell take half as long).  A thread owns V neighbouring fine
 // columns and walks down a run of rows: the x-interpolation of a coarse row
 // is done once for the F fine rows between two coarse centres, so a fine cell
 // costs one fma and its share of the store instead of some 20 fp64 operations
 // of index arithmetic and weights.  V = 2 (16-byte stores) where nx is even
-// and u is 16-byte aligned, else 1.  256 images of 512^2, F = 8: 6060 ->
-// 325 us.
+// and u is 16-byte aligned, else 1; the two columns share the coarse cells'
+// conversions and difference where they lie between the same centres.  256
+// images of 512^2, F = 8: 6060 us, 325 with conversions, finiteness checks and
+// the two-weight form on the FP64 pipe for every value and 2432 blocks walking
+// 4096 runs in two uneven turns, 184 now (FP64 pipe 92 % busy, 1.6 operations
+// per fine cell).
 template <int V>
 __global__ void __launch_bounds__(kUpThreads) upsample_kernel(const float *__restrict__ out, float scale, int ny,
                                                              int nx, int F, int nimg, double *__restrict__ u) {
     __shared__ double s_w[32];  // weight of the lower coarse row, i rows below the upper one's centre
     const int H = ny / F, W = nx / F;
     const int odd = F & 1;
+    const double dscale = widen(scale);
     if (threadIdx.x < F) s_w[threadIdx.x] = (2.0 * threadIdx.x + (odd ? 0.0 : 1.0)) / (2.0 * F);
     __syncthreads();
     const int ncol = (nx + kUpThreads * V - 1) / (kUpThreads * V);
@@ -667,14 +732,22 @@ __global__ void __launch_bounds__(kUpThreads) upsample_kernel(const float *__res
             xr[v] = min(j + 1, W - 1);
             wx[v] = j < 0 || j + 1 >= W ? 0.0 : s_w[x + v - first_of(j)];
         }
+        const bool same = V > 1 && xl[0] == xl[V - 1] && xr[0] == xr[V - 1];
         const float *o = out + img * (long long)H * W;
         auto coarse_row = [&](int Y, double (&m)[V]) {
             const float *r = o + (long long)min(max(Y, 0), H - 1) * W;
+            double a = widen(r[xl[0]]), b = widen(r[xr[0]]), df = b - a;
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                const double a = (double)r[xl[v]], b = (double)r[xr[v]];
-                const double df = b - a;  // not finite (a network that overflowed): the two-weight form
-                m[v] = (isfinite(df) ? fma(wx[v], df, a) : (1.0 - wx[v]) * a + wx[v] * b) * (double)scale;
+                if (v > 0 && !same) {
+                    a = widen(r[xl[v]]);
+                    b = widen(r[xr[v]]);
+                    df = b - a;
+                }
+                double t;
+                if (finite(df)) t = fma(wx[v], df, a);
+                else t = two_weights(wx[v], a, b);  // a network that overflowed
+                m[v] = t * dscale;
             }
         };
         int y = ya, j = interval(ya);
@@ -690,7 +763,7 @@ __global__ void __launch_bounds__(kUpThreads) upsample_kernel(const float *__res
             int i = y - first_of(j);
             bool fin = true;
 #pragma unroll
-            for (int v = 0; v < V; ++v) fin = fin && isfinite(d[v]);
+            for (int v = 0; v < V; ++v) fin = fin && finite(d[v]);
             if (!fin) {
                 for (; y < y1; ++y, ++i) {
                     const double w = j < 0 || j + 1 >= H ? 0.0 : s_w[i];
@@ -852,9 +925,15 @@ perks_status forward(perks_warmnet *n, int nimg, int ny, int nx, const double *k
     const int pgrid = (int)std::min<long long>((pixels + 255) / 256, 16LL * ctx->sm_count);  // thread per pixel
     S *x0 = (S *)n->x0, *x1 = (S *)n->x1, *x2 = (S *)n->x2, *x3 = (S *)n->x3;
     const int cells = kPoolThreads / n->pool;
-    const long long jobs = (long long)nimg * H * ((W + cells - 1) / cells);
-    features_kernel<S><<<(int)std::min<long long>(jobs, 8LL * ctx->sm_count), kPoolThreads, 0, s>>>(
-        k, f, u, x0, n->ut, ny, nx, n->pool, nimg);
+    // jobs of F fine rows: far below 2^31 for any k that fits in memory.  A round per block where that fills three
+    // blocks per SM, rounds of several jobs beyond
+    const int jobs = (int)((long long)nimg * H * ((W + cells - 1) / cells));
+    const int nj = std::max(1, std::min(kPoolJobs, jobs / (3 * ctx->sm_count)));
+    const size_t fsm = pool_smem(nj, u != nullptr);
+    perks_status frc = set_smem(ctx, features_kernel<S>, pool_smem(kPoolJobs, true));
+    if (frc) return frc;
+    features_kernel<S><<<std::min((jobs + nj - 1) / nj, 3 * ctx->sm_count), kPoolThreads, fsm, s>>>(
+        k, f, u, x0, n->ut, ny, nx, n->pool, jobs, nj);
     const float *P = n->params;
     conv_first_kernel<S><<<pgrid, 256, 0, s>>>(x0, P + n->off_w[0], P + n->off_b[0], x1, nimg, H, W, n->dil[0]);
     if (std::is_same<S, __nv_bfloat16>::value && n->tensor_cores) {
@@ -1068,7 +1147,7 @@ extern "C" perks_status perks_warmnet_predict(perks_warmnet *n, int32_t nimg, in
         const int V = pairs ? 2 : 1;
         const long long jobs = (long long)nimg * ((ny + kUpRows - 1) / kUpRows) *
                                ((nx + kUpThreads * V - 1) / (kUpThreads * V));
-        const int grid = (int)std::min<long long>(jobs, 16LL * n->ctx->sm_count);
+        const int grid = (int)std::min<long long>(jobs, 1 << 30);
         if (pairs) upsample_kernel<2><<<grid, kUpThreads, 0, s>>>(n->outb, n->out_scale, ny, nx, n->pool, nimg, u);
         else upsample_kernel<1><<<grid, kUpThreads, 0, s>>>(n->outb, n->out_scale, ny, nx, n->pool, nimg, u);
     }

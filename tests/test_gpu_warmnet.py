@@ -437,3 +437,25 @@ def test_log_of_extreme_coefficients(ctx, F, value):
     torch.cuda.synchronize()
     ref = _bilinear(_pool(np.log(k), F), F)
     assert np.max(np.abs(u.cpu().numpy() - ref)) <= 2.0 ** -22 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("F,ny,nx,nimg", [(1, 13, 300, 75), (2, 40, 258, 61), (3, 60, 255, 97), (8, 64, 264, 150),
+                                          (32, 64, 320, 500)])
+def test_pooling_rounds_of_jobs(ctx, F, ny, nx, nimg):
+    """Large batches pool several rows of coarse cells per round, single images
+    one: the same bits for every image, a partly filled last round included."""
+    from paper_2204_02064_gb300 import api
+    k = np.exp(6.0 * inputs.uniform(71, nimg * ny * nx) - 3.0).reshape(nimg, ny, nx)
+    f = (2.0 * inputs.uniform(72, nimg * ny * nx) - 1.0).reshape(nimg, ny, nx)
+    k[nimg - 1, 0, 0] = 5e-324                                    # a logarithm of its own
+    net = api.WarmNet(ctx, storage=api.F32, dilations=DIL, seed=3, pool=F)
+    net.scale = 1.5
+    dk, df = _dev(k), _dev(f)
+    u = torch.zeros((nimg, ny, nx), dtype=torch.float64, device="cuda")
+    net.predict(dk, df, u)
+    one = torch.zeros((1, ny, nx), dtype=torch.float64, device="cuda")
+    for i in (0, 1, nimg // 2, nimg - 2, nimg - 1):
+        net.predict(dk[i:i + 1].contiguous(), df[i:i + 1].contiguous(), one)
+        torch.cuda.synchronize()
+        assert torch.equal(one[0], u[i]), i
+    net.close()
