@@ -207,3 +207,16 @@ def test_resident_default_at_192_cubed(ctx, dtype):
     st.close()
     assert d["kernel"] == 1 and d["cached_cells"] == d["cells"]
     assert d["algorithmic_bytes"] < 0.25 * 2 * 1000 * d["cells"] * {"f32": 4, "bf16": 2}[dtype]
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("shape,tiles", [((40, 28, 48), (3, 2, 1)), ((33, 27, 48), (3, 1, 1)), ((9, 5, 48), (6, 5, 1)),
+                                         ((23, 18, 96), (3, 2, 3))])
+def test_resident_warps_of_uneven_groups(ctx, oracle, dtype, shape, tiles):
+    """Warps that hold threads of two plane groups (segments of different
+    length), idle lanes beside busy ones, and no row at all."""
+    f = inputs.stencil_field(shape, 71)
+    for rows in (1, 2):
+        src, out, stats, _ = _run(ctx, "3d7pt", f, 7, dtype, plan=dict(tiles=tiles, rows=rows))
+        assert (stats["tiles_x"], stats["tiles_y"], stats["tiles_z"]) == tiles
+        _check(oracle, "3d7pt", src, out, 7, dtype)
