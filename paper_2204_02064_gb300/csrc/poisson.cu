@@ -670,18 +670,20 @@ size_t run_smem(const perks_poisson *P, int C, int &on_chip) {
     return on_chip ? base + r : base;
 }
 
-// Blocks per problem of perks_poisson_run_kernel.  A batch of fewer problems
-// than the documented groups would fill the GPU with keeps those; otherwise
-// the group that finishes the batch in the fewest cycles by this model: a
-// block's iteration takes 5 cycles per cell (10 fp64 operations, 2 lanes per
-// clock and SM), twice that where two blocks share an SM, plus the exchanges,
-// which the other block of an SM hides; the batch takes ceil(problems /
-// groups) of the longest iterations.  512^2, 64 problems: 19 blocks per
-// problem, 16 groups, 4 full waves, where 38 groups of 8 leave the second
-// wave a third empty.
+// Blocks per problem of perks_poisson_run_kernel.  The documented group where
+// it gives every block at most 8192 cells and all of the batch runs at once;
+// otherwise the group that finishes the batch in the fewest cycles by this
+// model: a block's iteration takes 6.5 cycles per cell (10 fp64 operations, 2
+// lanes per clock and SM, and the rest of an iteration; 7.5 with r in global
+// memory), nearly twice that where two blocks share an SM, plus the exchanges;
+// the batch takes ceil(problems / groups) of the longest iterations.  Measured
+// (ms, the group picked / documented / others): 64 problems of 512^2, 24
+// iterations, 19 blocks 10.2 / 8: 12.4 / 25: 10.5; 256 of 355 x 94, 7 blocks
+// 3.1 / 1: 3.8 / 19: 4.9; 24 of 332 x 441, 12 blocks 1.4 / 8: 2.1 / 25: 1.4;
+// 256 of 146 x 75, one block 1.56 / 2: 1.71.
 int run_group(const perks_poisson *P) {
     const int doc = effective_group(P), slots = 2 * P->ctx->sm_count;
-    if (P->n <= 8192 || (P->n >= 65536 && (long long)P->nprob * doc <= slots)) return doc;
+    if (P->n <= 8192 || (P->n <= 8192LL * doc && (long long)P->nprob * doc <= slots)) return doc;
     double best = 1e300;
     int bc = doc;
     for (int C = 1; C <= std::min(P->ny, 64); ++C) {
@@ -689,11 +691,12 @@ int run_group(const perks_poisson *P) {
         if (groups < 1) break;
         int on_chip;
         run_smem(P, C, on_chip);
-        const double m = (double)((P->ny + C - 1) / C) * P->nx * (on_chip ? 1.0 : 1.1);
-        const double ex = C > 1 ? 6000.0 : 3000.0;
-        const double t = groups * C > P->ctx->sm_count ? std::max(10.0 * m, 5.0 * m + ex) : 5.0 * m + ex;
+        const double m = (double)((P->ny + C - 1) / C) * P->nx;
+        const double ex = 5000.0 + 3500.0 * std::log2((double)C);
+        const double t = groups * C > P->ctx->sm_count ? (on_chip ? 12.3 : 14.5) * m + ex
+                                                       : (on_chip ? 6.5 : 7.5) * m + 1.2 * ex;
         const double total = (double)((P->nprob + groups - 1) / groups) * t;
-        if (total <= best) { best = total; bc = C; }
+        if (total < best) { best = total; bc = C; }
     }
     return bc;
 }
