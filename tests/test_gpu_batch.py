@@ -148,8 +148,8 @@ def test_batch_strip_equals_ring_bitwise(ctx):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
-@pytest.mark.parametrize("count,nx,ny", [(3, 116, 40), (2, 120, 1), (5, 124, 9), (4, 240, 77), (3, 244, 200),
-                                         (300, 64, 33), (1, 4, 700)])
+@pytest.mark.parametrize("count,nx,ny", [(3, 116, 40), (2, 120, 5), (5, 124, 9), (4, 240, 77), (3, 244, 200),
+                                         (300, 64, 33), (1, 8, 700)])
 def test_batch_strip_edges(ctx, oracle, dtype, count, nx, ny):
     """Strips a vector wider or narrower than the domain, more columns than
     warps hold one item of, domains lower than an item; the automatic items."""
