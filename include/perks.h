@@ -158,7 +158,8 @@ typedef struct {
                                            automatic); STRIP: time steps per sweep (1, 2 or 4
                                            where compiled, 0 = automatic), tiles_z the runs of
                                            rows (0 = automatic); reserved[2] = kernel body
-                                           (PERKS_KERNEL_AUTO / _RESIDENT / _STREAMING / _STRIP;
+                                           (PERKS_KERNEL_AUTO / _RESIDENT / _STREAMING / _STRIP /
+                                           _SLAB;
                                            AUTO in a plan means STREAMING, AUTO with no plan
                                            picks the resident tile when every tile fits in shared
                                            memory, the column strips for other 2-D domains);
@@ -204,9 +205,12 @@ enum {
                                     shared-memory ring, caching some planes in registers / shared
                                     memory */
     PERKS_KERNEL_PER_STEP = 3,   /* one launch per step (PERKS_PER_STEP) */
-    PERKS_KERNEL_STRIP = 4       /* column strips (2-D: 2d5pt, 2ds9pt, 2d9pt, 2d25pt): every warp streams a strip of
+    PERKS_KERNEL_STRIP = 4,      /* column strips (2-D: 2d5pt, 2ds9pt, 2d9pt, 2d25pt): every warp streams a strip of
                                     rows through register windows, several time steps per sweep; a sweep, not a
                                     step, ends at the grid barrier.  Not used while a step trace is on */
+    PERKS_KERNEL_SLAB = 5        /* slab streaming (3-D: 3d7pt, 3d13pt, 3d27pt, poisson; any row length): rows of
+                                    neighbouring lanes, several rows per thread, planes through a shared-memory
+                                    ring, no caches.  Not used while a step trace is on */
 };
 
 /* Creates a stencil over a device-resident domain described by *desc (the

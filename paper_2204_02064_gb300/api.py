@@ -19,10 +19,10 @@ MAX_POINTS = 125
 F64, F32, BF16 = 0, 1, 2
 PERSISTENT, PER_STEP = 0, 1
 KERNEL_AUTO, KERNEL_RESIDENT, KERNEL_STREAMING, KERNEL_PER_STEP = 0, 1, 2, 3
-KERNEL_STRIP = 4
+KERNEL_STRIP, KERNEL_SLAB = 4, 5
 BATCH_RING, BATCH_STRIP = 0, 1
 KERNEL_NAMES = {KERNEL_RESIDENT: "resident", KERNEL_STREAMING: "streaming", KERNEL_PER_STEP: "per_step",
-                KERNEL_STRIP: "strip"}
+                KERNEL_STRIP: "strip", KERNEL_SLAB: "slab"}
 CG_FP64, CG_FP32_IR, CG_FP64_MULTI = 0, 1, 2
 SPMV_ROWVEC, SPMV_MERGE, SPMV_SEG = 0, 1, 2
 
@@ -371,7 +371,8 @@ class Stencil:
         resident-tile kernel (``tiles`` and ``threads`` 256/512 apply to
         it, 0 = automatic), KERNEL_STRIP the column-strip kernel of 2-D
         domains (``planes_per_barrier`` = time steps per sweep, ``tiles[2]``
-        = runs of rows), KERNEL_STREAMING / KERNEL_AUTO the plane-streaming
+        = runs of rows), KERNEL_SLAB the slab-streaming kernel of 3-D domains,
+        KERNEL_STREAMING / KERNEL_AUTO the plane-streaming
         kernel; ``rows`` (1 or 2, 0 = automatic) is the resident kernel's
         rows per thread; ``balanced`` (cache-free plane streaming only) cuts
         the tile columns' planes into equal shares, one per co-resident

@@ -5,12 +5,14 @@
 #include <algorithm>
 #include <array>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <vector>
 
 #include "internal.h"
 #include "stencil_registry.h"
+#include "stencil_slab.cuh"
 #include "stencil_strip.cuh"
 #include "stencil_tile.cuh"
 
@@ -140,6 +142,17 @@ std::vector<StripKEntry> &strip_registry() {
     return table;
 }
 
+std::vector<SlabEntry> &slab_registry() {
+    static std::vector<SlabEntry> table = [] {
+        std::vector<SlabEntry> t;
+        register_slab_f64(t);
+        register_slab_f32(t);
+        register_slab_bf16(t);
+        return t;
+    }();
+    return table;
+}
+
 // Planes per block barrier preferred by default where both variants exist.
 constexpr int kDefaultPlanesPerBarrier = 2;
 
@@ -182,6 +195,10 @@ struct Plan {
     long long FS = 0;
     // column-strip kernel (2-D): ntx strips across x, ntz runs of rows
     StripKEntry *sk = nullptr;
+    double cost = 0.0;         // column strips: modelled SM cycles per step
+    // slab-streaming kernel (3-D): ntx x nty columns, 2^loglx lanes per row
+    SlabEntry *lk = nullptr;
+    int loglx = 0;
 };
 
 }  // namespace
@@ -373,7 +390,7 @@ perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts, int want_
                 const double cyc =
                     std::max({quarter * rs * stage, rounds * (rs * stage + 160.0 * iters), bytes / rate}) + 3500.0;
                 if (cyc / e.ts < best) {
-                    best = cyc / e.ts;
+                    best = bp.cost = cyc / e.ts;
                     bp.sk = &e;
                     bp.ntx = nsx; bp.nty = 1; bp.ntz = nch;
                     bp.txmax = outw; bp.tymax = 1; bp.tzmax = ceil_div(Z, nch);
@@ -386,6 +403,59 @@ perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts, int want_
     // halo cells: the overlap each item reads beyond its own cells, per step
     bp.halo_cells = ((long long)bp.ntx * bp.ntz * 32 * bp.sk->v * (2LL * bp.sk->ts * shape_by_id(st->shape_id).radius) +
                      (long long)bp.ntx * 2 * bp.sk->hl * bp.sk->v * Z) / bp.sk->ts;
+    pl = bp;
+    return PERKS_OK;
+}
+
+// Plan of the slab-streaming kernel (3-D domains): the lanes per row that
+// need the fewest columns (every plane of a column costs the same, full or
+// not; the wider row on a tie), and two blocks per SM, or one per plane where
+// there are fewer planes: parts of columns walked in step where they use 90 %
+// of those blocks and the step is not bound by the FP64 pipe, else equal
+// shares.
+perks_status make_slab_plan(perks_stencil *st, Plan &pl) {
+    perks_context *ctx = st->ctx;
+    const int dt = st->desc.dtype, X = st->X, Y = st->Y, Z = st->Z;
+    Plan bp;
+    if (st->desc.ndim == 3 && (dt != PERKS_BF16 || X % 8 == 0))
+        for (SlabEntry &e : slab_registry()) {
+            if (e.dtype != dt || e.shape != st->shape_id || e.aligned != (X % e.v == 0)) continue;
+            const int R = shape_by_id(st->shape_id).radius;
+            long long fewest = LLONG_MAX;
+            for (int lg = 5; lg >= 3; --lg) {
+                const int rows = (kSlabThreads >> lg) * e.ry;
+                const int nsx = ceil_div(X, e.v << lg), nsy = ceil_div(Y, rows);
+                if ((long long)nsx * nsy >= fewest) continue;
+                fewest = (long long)nsx * nsy;
+                bp.lk = &e;
+                bp.loglx = lg;
+                bp.ntx = nsx; bp.nty = nsy; bp.ntz = 1;
+                bp.txmax = e.v << lg; bp.tymax = rows; bp.tzmax = Z;
+                bp.PW = (e.v << lg) + 2 * e.v;
+                bp.PH = rows + 2 * R;
+            }
+            bp.plane = bp.PW * bp.PH;
+            bp.smem = (long long)e.slots * bp.plane * st->es;
+            const long long planes = fewest * Z, most = 2LL * ctx->sm_count;
+            bp.ntz = (int)std::min<long long>(Z, most / fewest);
+            bp.balanced = dt == PERKS_F64 || bp.ntz == 0 || fewest * bp.ntz * 10 < std::min(planes, most) * 9;
+            bp.blocks = bp.balanced ? (int)std::min(planes, most) : (int)fewest * bp.ntz;
+            if (bp.balanced) bp.ntz = 1;
+            // halo cells read per step: the rows and columns around every column's planes, and the planes
+            // above and below each share
+            bp.halo_cells = planes * ((long long)bp.plane - (long long)bp.txmax * bp.tymax) +
+                            (long long)bp.blocks * 2 * R * bp.plane;
+        }
+    if (!bp.lk)
+        return fail(ctx, PERKS_ERR_UNSUPPORTED, "slab-streaming kernel: 3-D stencils 3d7pt, 3d13pt, 3d27pt, poisson only");
+    int budget = 0;
+    const perks_status rc = smem_optin(ctx, (const void *)bp.lk->fn, &budget);
+    if (rc) return rc;
+    int per_sm = 0;
+    PERKS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)bp.lk->fn, kSlabThreads,
+                                                                  (size_t)bp.smem));
+    if (bp.smem > budget || (long long)per_sm * ctx->sm_count < bp.blocks)
+        return fail(ctx, PERKS_ERR_LAUNCH_TOO_LARGE, "slab-streaming kernel: %d blocks are not co-resident", bp.blocks);
     pl = bp;
     return PERKS_OK;
 }
@@ -590,24 +660,86 @@ perks_status make_base_plan(perks_stencil *st, Plan &pl, bool per_step = false) 
 // domain stays resident (small domains are held on chip by default).
 bool strip_beats_resident(const perks_stencil *st) { return st->desc.dtype != PERKS_F64 || st->cells > 65536; }
 
-// The plan a run uses.  A 2-D domain without a plan takes the column-strip
-// kernel where the other kernels could host the domain at all (so the domains
-// that are refused stay the same) and it is the faster one; a traced run keeps
-// the kernels that mark every step.
+// A 3-D domain without a plan whose other plan is `base`: the slab kernel?
+// (Figures: us per step, other plan / slab.)
+// In place of plane streaming, fp32 / bf16: yes (3d27pt fp32 251 x 246 x 233
+// 130 / 33, 256^3 92 / 32; 3d7pt 384^3 fp32 97 / 74, bf16 66 / 41).  fp64,
+// bound by the FP64 pipe: where the threads own cells and the blocks planes for
+// the better part (3d27pt 128^3, 0.96, 128 / 116; 344 x 279 x 52, 0.94, 301 / 280;
+// 80 x 304 x 81, 0.90, 113 / 118; 100 x 96 x 88, 0.68, 57 / 69; 64^3, two planes per
+// SM, 21.5 / 19.4), or 70 % of them against the one-cell-per-thread body
+// (187 x 143 x 117 3d13pt 102 / 91), and never in place of the 3d7pt bodies for
+// rows of whole vectors.
+// In place of the resident kernel (3d7pt): fp32 and fp64 where its tiles fill
+// few of its threads (fp32 64^3, a fifth, 3.6 / 3.0, 72^3, 30 %, 3.8 / 3.9, 192^3
+// 8.1 / 9.6; fp64 48^3, a third, 6.4 / 4.9, 256 x 200 x 24, two thirds, 20.3 /
+// 22.2); bf16, whose slab threads own eight cells, by the two kernels' times:
+// 3.4 us + 1 per chunk of the resident one, 3.3 + 0.75 per million cells of
+// filled lanes of the slab (64^3 4.1 / 3.2, 128^3 5.0 / 4.7, 144^3 5.9 / 6.9, 32 x
+// 202 x 212, half of the lanes, 4.5 / 5.4).
+bool slab_beats(const perks_stencil *st, const Plan &base, const Plan &slab) {
+    const int dt = st->desc.dtype;
+    const int lx = 1 << slab.loglx, rows = (kSlabThreads >> slab.loglx) * slab.lk->ry;
+    const double lanes = (double)st->X / ((double)slab.ntx * lx * slab.lk->v);
+    if (base.resident) {
+        const double slots = (double)base.chunks * base.tk->m * base.tk->nt * base.tk->r * base.tk->v;
+        const double used = (double)st->cells / (st->ctx->sm_count * slots);
+        if (dt == PERKS_BF16) return 0.75e-6 * (double)st->cells / lanes < 0.1 + base.chunks + 0.6 * used;
+        return used < (dt == PERKS_F64 ? 0.5 : 0.25);
+    }
+    if (dt != PERKS_F64) return true;
+    if (st->shape_id == SH_3D7 && st->X % 2 == 0) return false;
+    const long long planes = (long long)slab.ntx * slab.nty * st->Z;
+    const long long most = (planes + slab.blocks - 1) / slab.blocks;  // of a block
+    const double used = lanes * st->Y / ((double)slab.nty * rows) * (double)planes / ((double)slab.blocks * most);
+    return used >= (base.k && base.k->v == 1 ? 0.7 : most <= 2 ? 0.75 : 0.92);
+}
+
+// fp64 3d7pt with rows of whole vectors, from 4 M cells: the cache-free body
+// with 256 threads (two blocks per SM, one's FP64 work under the other's
+// barriers) in balanced shares: 384^3 838 -> 746 us per step, 256^3 265 ->
+// 228, 192^3 108 -> 101.
+void choose_f64_3d7(perks_stencil *st, Plan &pl) {
+    const std::string saved_msg = st->ctx->last_error;
+    const perks_stencil_plan saved = st->plan;
+    Plan alt;
+    st->plan = perks_stencil_plan{};
+    st->plan.reserved[1] = 4;
+    st->plan.reserved[3] = 256;
+    st->plan.balanced = 1;
+    st->has_plan = true;
+    if (make_base_plan(st, alt, false) == PERKS_OK) pl = alt;
+    st->has_plan = false;
+    st->plan = saved;
+    st->ctx->last_error = saved_msg;
+}
+
+// The plan a run uses.  A domain without a plan takes, where the other kernels
+// could host it at all (so the domains that are refused stay the same), the
+// column-strip kernel (2-D) or the slab kernel (3-D)
+// where that is the faster one; a traced run keeps the kernels that mark every
+// step.
 perks_status make_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
-    const bool asked = !per_step && st->has_plan && st->plan.reserved[2] == PERKS_KERNEL_STRIP;
-    const bool open = !per_step && !st->has_plan && !st->no_resident && !st->trace && st->desc.ndim == 2;
+    const int kind = st->has_plan ? st->plan.reserved[2] : PERKS_KERNEL_AUTO;
+    const bool asked = !per_step && (kind == PERKS_KERNEL_STRIP || kind == PERKS_KERNEL_SLAB);
+    const bool open = !per_step && !st->has_plan && !st->no_resident && !st->trace;
     if (!asked && !open) return make_base_plan(st, pl, per_step);
     st->has_plan = false;
     perks_status rc = make_base_plan(st, pl, false);
     st->has_plan = asked;
     if (rc) return rc;
-    if (asked) return make_strip_plan(st, pl, st->plan.reserved[1], st->plan.tiles_z);
-    if (pl.resident && !strip_beats_resident(st)) return PERKS_OK;
+    if (kind == PERKS_KERNEL_STRIP) return make_strip_plan(st, pl, st->plan.reserved[1], st->plan.tiles_z);
+    if (kind == PERKS_KERNEL_SLAB) return make_slab_plan(st, pl);
     const std::string saved_msg = st->ctx->last_error;
     Plan sp;
-    if (make_strip_plan(st, sp, 0, 0) == PERKS_OK) pl = sp;
-    else st->ctx->last_error = saved_msg;
+    if (st->desc.ndim == 2) {
+        if ((!pl.resident || strip_beats_resident(st)) && make_strip_plan(st, sp, 0, 0) == PERKS_OK) pl = sp;
+    } else {
+        if (make_slab_plan(st, sp) == PERKS_OK && slab_beats(st, pl, sp)) pl = sp;
+        else if (st->shape_id == SH_3D7 && st->desc.dtype == PERKS_F64 && st->X % 2 == 0 && st->cells >= (1 << 22))
+            choose_f64_3d7(st, pl);
+    }
+    st->ctx->last_error = saved_msg;
     return PERKS_OK;
 }
 
@@ -618,7 +750,17 @@ void fill_stats(const perks_stencil *st, const Plan *pl, long long steps, int va
     o->variant = variant;
     o->cells = st->cells;
     const double S = st->es;
-    if (variant == PERKS_PERSISTENT && pl && pl->sk) {
+    if (variant == PERKS_PERSISTENT && pl && pl->lk) {
+        o->kernel = PERKS_KERNEL_SLAB;
+        o->grid_blocks = pl->blocks;
+        o->threads_per_block = kSlabThreads;
+        o->tiles_x = pl->ntx; o->tiles_y = pl->nty; o->tiles_z = pl->ntz;
+        o->prefetch_planes = pl->lk->ahead;
+        o->planes_per_sync = 1;
+        o->smem_bytes_per_block = pl->smem;
+        o->halo_cells_per_step = pl->halo_cells;
+        o->algorithmic_bytes = S * (double)steps * (2.0 * (double)st->cells + (double)pl->halo_cells);
+    } else if (variant == PERKS_PERSISTENT && pl && pl->sk) {
         o->kernel = PERKS_KERNEL_STRIP;
         o->grid_blocks = pl->blocks;
         o->threads_per_block = pl->sk->nt;
@@ -753,6 +895,37 @@ perks_status run_strip(perks_stencil *st, long long steps, cudaStream_t s, const
     return PERKS_OK;
 }
 
+// One cooperative launch of the slab-streaming kernel.
+perks_status run_slab(perks_stencil *st, long long steps, cudaStream_t s, const Plan &pl) {
+    perks_context *ctx = st->ctx;
+    if (!st->bar) PERKS_CUDA(ctx, cudaMalloc(&st->bar, sizeof(unsigned long long)));
+    if (!st->err) PERKS_CUDA(ctx, cudaMalloc(&st->err, sizeof(DevError)));
+    SlabArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.X = st->X; a.Y = st->Y; a.Z = st->Z;
+    a.XY = (long long)st->X * st->Y;
+    a.loglx = pl.loglx;
+    a.nsx = pl.ntx; a.nsy = pl.nty;
+    a.nz = pl.balanced ? 0 : pl.ntz;
+    a.PW = pl.PW; a.plane = pl.plane;
+    a.steps = steps;
+    a.boundary = st->desc.boundary;
+    a.boundary_f = (float)st->desc.boundary;
+    for (int i = 0; i < 27; ++i) { a.w[i] = st->kw[i]; a.wf[i] = (float)st->kw[i]; }
+    a.field[0] = st->field[st->cur];
+    a.field[1] = st->field[st->cur ^ 1];
+    a.bar = st->bar;
+    a.err = st->err;
+    a.timeout_ns = ctx->timeout_ns;
+    PERKS_CUDA(ctx, cudaMemsetAsync(st->bar, 0, sizeof(unsigned long long), s));
+    PERKS_CUDA(ctx, cudaMemsetAsync(st->err, 0, sizeof(DevError), s));
+    void *args[] = {&a};
+    PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)pl.lk->fn, dim3(pl.blocks), dim3(kSlabThreads), args,
+                                                (size_t)pl.smem, s));
+    if (steps & 1) st->cur ^= 1;
+    return PERKS_OK;
+}
+
 perks_status ensure_persistent_buffers(perks_stencil *st, const Plan &pl) {
     perks_context *ctx = st->ctx;
     const int RX = shape_by_id(st->shape_id).radius;
@@ -817,6 +990,7 @@ perks_status run_persistent(perks_stencil *st, long long steps, cudaStream_t s, 
     if (rc) return rc;
     if (pl.resident) return run_resident(st, steps, s, pl);
     if (pl.sk) return run_strip(st, steps, s, pl);
+    if (pl.lk) return run_slab(st, steps, s, pl);
     rc = ensure_persistent_buffers(st, pl);
     if (rc) return rc;
     int per_sm = 0;
@@ -1006,9 +1180,10 @@ extern "C" perks_status perks_stencil_set_plan(perks_stencil *st, const perks_st
     if (plan->reserved[1] != 0 && plan->reserved[1] != 2 && plan->reserved[1] != 4 &&
         !(plan->reserved[2] == PERKS_KERNEL_STRIP && plan->reserved[1] == 1))
         return fail(st->ctx, PERKS_ERR_INVALID_ARG, "stencil_set_plan: planes per barrier must be 0, 2 or 4");
-    if (plan->reserved[2] < PERKS_KERNEL_AUTO || (plan->reserved[2] > PERKS_KERNEL_STREAMING && plan->reserved[2] != PERKS_KERNEL_STRIP))
+    if (plan->reserved[2] < PERKS_KERNEL_AUTO || (plan->reserved[2] > PERKS_KERNEL_STREAMING && plan->reserved[2] != PERKS_KERNEL_STRIP &&
+         plan->reserved[2] != PERKS_KERNEL_SLAB))
         return fail(st->ctx, PERKS_ERR_INVALID_ARG,
-                    "stencil_set_plan: kernel must be AUTO, RESIDENT, STREAMING or STRIP");
+                    "stencil_set_plan: kernel must be AUTO, RESIDENT, STREAMING, STRIP or SLAB");
     if (plan->reserved[3] != 0 && plan->reserved[3] != 256 && plan->reserved[3] != 512 && plan->reserved[3] != 1024)
         return fail(st->ctx, PERKS_ERR_INVALID_ARG, "stencil_set_plan: threads must be 0, 256, 512 or 1024");
     st->plan = *plan;
@@ -1215,6 +1390,20 @@ extern "C" perks_status perks_stencil_autotune(perks_stencil *st, int32_t varian
             }
             ctx->last_error = saved_msg;
         }
+    // slab-streaming kernel
+    if (!per_step && !st->no_resident && st->desc.ndim == 3) {
+        perks_stencil_plan p{};
+        p.reserved[2] = PERKS_KERNEL_SLAB;
+        st->plan = p;
+        st->has_plan = true;
+        Plan probe;
+        const std::string saved_msg = ctx->last_error;
+        if (make_plan(st, probe, false) == PERKS_OK) {
+            p.tiles_x = probe.ntx; p.tiles_y = probe.nty; p.tiles_z = probe.ntz;
+            plans.push_back(p);
+        }
+        ctx->last_error = saved_msg;
+    }
     // plane-streaming kernels compiled with 256 threads (two blocks per SM): the model's tiling,
     // one tile per block and in balanced shares
     if (!per_step)

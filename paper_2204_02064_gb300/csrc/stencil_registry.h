@@ -53,6 +53,11 @@ void register_strip_f64(std::vector<StripKEntry> &out);
 void register_strip_f32(std::vector<StripKEntry> &out);
 void register_strip_bf16(std::vector<StripKEntry> &out);
 
+struct SlabEntry;  // stencil_slab.cuh
+void register_slab_f64(std::vector<SlabEntry> &out);
+void register_slab_f32(std::vector<SlabEntry> &out);
+void register_slab_bf16(std::vector<SlabEntry> &out);
+
 struct TileKernelEntry;  // stencil_tile.cuh
 void register_tile_kernels(std::vector<TileKernelEntry> &out);
 

@@ -1,0 +1,59 @@
+"""GPU parity of the slab-streaming kernel (3-D) against the oracle, at the
+edges of its tiles: rows that no vector width divides, fewer rows than a thread
+owns, columns cut in the middle of a block's share.
+fp64 within 1e-12 of the local value (floored at 1e-3 of the field maximum);
+fp32 / bf16 storage bit for bit against the low-precision oracle."""
+import numpy as np
+import pytest
+
+from paper_2204_02064_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+TT = {"f64": torch.float64, "f32": torch.float32, "bf16": torch.bfloat16}
+
+
+def rel_err(g, o):
+    floor = 1e-3 * max(np.max(np.abs(o)), 1e-300)
+    return float(np.max(np.abs(g - o) / np.maximum(np.abs(o), floor)))
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2204_02064_gb300 import api
+    return api.Context(0)
+
+
+def _check(ctx, oracle, name, dtype, shape, steps, kernel, **plan):
+    from paper_2204_02064_gb300 import api
+    offs, w = inputs.shape_offsets(name), inputs.workload_weights(name, seed=5)
+    st = api.Stencil(ctx, shape, offs, w, dtype=dtype, boundary=0.375)
+    st.set_plan(kernel=kernel, **plan)
+    src = torch.from_numpy(inputs.stencil_field(shape, 51)).to(TT[dtype]).cuda()
+    st.set_field(src)
+    stats = st.run(steps, stats=True)
+    assert stats["kernel"] == kernel
+    out = torch.empty_like(src)
+    st.get_field(out)
+    torch.cuda.synchronize()
+    st.close()
+    if dtype == "f64":
+        ref = oracle.stencil_run(src.cpu().numpy(), offs, w, steps, boundary=0.375)
+        assert rel_err(out.cpu().numpy(), ref) <= 1e-12
+    else:
+        ref = oracle.stencil_run_lowp(src.float().cpu().numpy(), offs, w, steps, dtype, boundary=0.375)
+        got = out.float().cpu().numpy()
+        assert np.array_equal(got, ref), float(np.max(np.abs(got - ref)))
+    return stats
+
+
+@pytest.mark.parametrize("name", ["3d7pt", "3d13pt", "3d27pt", "poisson"])
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("shape,steps", [((7, 6, 16), 4), ((61, 9, 33), 3), ((23, 67, 129), 2), ((40, 37, 255), 3),
+                                         ((30, 129, 72), 2), ((331, 5, 40), 3)])
+def test_slab_matches_oracle(ctx, oracle, name, dtype, shape, steps):
+    from paper_2204_02064_gb300 import api
+    if dtype == "bf16":
+        shape = shape[:2] + (shape[2] // 8 * 8,)
+    _check(ctx, oracle, name, dtype, shape, steps, api.KERNEL_SLAB)
