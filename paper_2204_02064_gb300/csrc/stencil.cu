@@ -226,6 +226,11 @@ struct perks_stencil {
     void *tfaces[2] = {nullptr, nullptr};  // resident-tile kernel: face buffers by step parity
     size_t tfaces_bytes = 0;
     bool no_resident = false;             // plan the plane-streaming kernel only
+    // The last plan made and what it was made for: a run of the same stencil under the same plan settings uses it
+    // again (searching the tilings takes the host 50 to 400 us, as long as many runs).
+    bool kept = false, kept_has_plan = false, kept_per_step = false, kept_no_resident = false, kept_trace = false;
+    perks_stencil_plan kept_request{};
+    Plan kept_plan;
 };
 
 namespace {
@@ -719,7 +724,7 @@ void choose_f64_3d7(perks_stencil *st, Plan &pl) {
 // column-strip kernel (2-D) or the slab kernel (3-D)
 // where that is the faster one; a traced run keeps the kernels that mark every
 // step.
-perks_status make_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
+perks_status search_plan(perks_stencil *st, Plan &pl, bool per_step) {
     const int kind = st->has_plan ? st->plan.reserved[2] : PERKS_KERNEL_AUTO;
     const bool asked = !per_step && (kind == PERKS_KERNEL_STRIP || kind == PERKS_KERNEL_SLAB);
     const bool open = !per_step && !st->has_plan && !st->no_resident && !st->trace;
@@ -740,6 +745,26 @@ perks_status make_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
             choose_f64_3d7(st, pl);
     }
     st->ctx->last_error = saved_msg;
+    return PERKS_OK;
+}
+
+perks_status make_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
+    const bool traced = st->trace != nullptr;
+    if (st->kept && st->kept_per_step == per_step && st->kept_no_resident == st->no_resident &&
+        st->kept_trace == traced && st->kept_has_plan == st->has_plan &&
+        (!st->has_plan || std::memcmp(&st->kept_request, &st->plan, sizeof(st->plan)) == 0)) {
+        pl = st->kept_plan;
+        return PERKS_OK;
+    }
+    const perks_status rc = search_plan(st, pl, per_step);
+    st->kept = rc == PERKS_OK;
+    if (rc) return rc;
+    st->kept_per_step = per_step;
+    st->kept_no_resident = st->no_resident;
+    st->kept_trace = traced;
+    st->kept_has_plan = st->has_plan;
+    st->kept_request = st->plan;
+    st->kept_plan = pl;
     return PERKS_OK;
 }
 

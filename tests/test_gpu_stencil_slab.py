@@ -57,3 +57,22 @@ def test_slab_matches_oracle(ctx, oracle, name, dtype, shape, steps):
     if dtype == "bf16":
         shape = shape[:2] + (shape[2] // 8 * 8,)
     _check(ctx, oracle, name, dtype, shape, steps, api.KERNEL_SLAB)
+
+
+def test_plan_is_kept_until_the_request_changes(ctx):
+    """Runs of one stencil reuse its plan; set_plan, a trace and the autotuner still take effect."""
+    from paper_2204_02064_gb300 import api
+    st = api.Stencil(ctx, (96, 128), inputs.shape_offsets("2d9pt"), inputs.workload_weights("2d9pt"), dtype="f32")
+    first = st.describe(10)
+    assert st.describe(10) == first
+    st.set_plan(kernel=api.KERNEL_STRIP, tiles=(0, 0, 7))
+    assert st.describe(10)["kernel"] == api.KERNEL_STRIP and st.describe(10)["tiles_z"] == 7
+    st.set_plan(kernel=api.KERNEL_STRIP, tiles=(0, 0, 5))
+    assert st.describe(10)["tiles_z"] == 5
+    st.reset_plan()
+    assert st.describe(10) == first
+    st.set_trace(2)
+    assert st.describe(10)["kernel"] == api.KERNEL_STREAMING
+    st.set_trace(0)
+    assert st.describe(10) == first
+    st.close()
