@@ -159,7 +159,7 @@ typedef struct {
                                            where compiled, 0 = automatic), tiles_z the runs of
                                            rows (0 = automatic); reserved[2] = kernel body
                                            (PERKS_KERNEL_AUTO / _RESIDENT / _STREAMING / _STRIP /
-                                           _SLAB;
+                                           _SLAB / _PATCH;
                                            AUTO in a plan means STREAMING, AUTO with no plan
                                            picks the resident tile when every tile fits in shared
                                            memory, the column strips for other 2-D domains);
@@ -208,9 +208,13 @@ enum {
     PERKS_KERNEL_STRIP = 4,      /* column strips (2-D: 2d5pt, 2ds9pt, 2d9pt, 2d25pt): every warp streams a strip of
                                     rows through register windows, several time steps per sweep; a sweep, not a
                                     step, ends at the grid barrier.  Not used while a step trace is on */
-    PERKS_KERNEL_SLAB = 5        /* slab streaming (3-D: 3d7pt, 3d13pt, 3d27pt, poisson; any row length): rows of
+    PERKS_KERNEL_SLAB = 5,       /* slab streaming (3-D: 3d7pt, 3d13pt, 3d27pt, poisson; any row length): rows of
                                     neighbouring lanes, several rows per thread, planes through a shared-memory
                                     ring, no caches.  Not used while a step trace is on */
+    PERKS_KERNEL_PATCH = 6       /* patches (small 2-D domains, the column strips' shapes): every block keeps its tile
+                                    and a halo some steps deep in shared memory and meets its neighbours, not the
+                                    grid, every few steps (planes_per_sync; plan: reserved[1] = steps per exchange,
+                                    tiles_x, tiles_z = tiles, 0 = automatic).  Not used while a step trace is on */
 };
 
 /* Creates a stencil over a device-resident domain described by *desc (the

@@ -19,10 +19,10 @@ MAX_POINTS = 125
 F64, F32, BF16 = 0, 1, 2
 PERSISTENT, PER_STEP = 0, 1
 KERNEL_AUTO, KERNEL_RESIDENT, KERNEL_STREAMING, KERNEL_PER_STEP = 0, 1, 2, 3
-KERNEL_STRIP, KERNEL_SLAB = 4, 5
+KERNEL_STRIP, KERNEL_SLAB, KERNEL_PATCH = 4, 5, 6
 BATCH_RING, BATCH_STRIP = 0, 1
 KERNEL_NAMES = {KERNEL_RESIDENT: "resident", KERNEL_STREAMING: "streaming", KERNEL_PER_STEP: "per_step",
-                KERNEL_STRIP: "strip", KERNEL_SLAB: "slab"}
+                KERNEL_STRIP: "strip", KERNEL_SLAB: "slab", KERNEL_PATCH: "patch"}
 CG_FP64, CG_FP32_IR, CG_FP64_MULTI = 0, 1, 2
 SPMV_ROWVEC, SPMV_MERGE, SPMV_SEG = 0, 1, 2
 
@@ -372,6 +372,8 @@ class Stencil:
         it, 0 = automatic), KERNEL_STRIP the column-strip kernel of 2-D
         domains (``planes_per_barrier`` = time steps per sweep, ``tiles[2]``
         = runs of rows), KERNEL_SLAB the slab-streaming kernel of 3-D domains,
+        KERNEL_PATCH the patch kernel of small 2-D domains
+        (``planes_per_barrier`` = steps per exchange),
         KERNEL_STREAMING / KERNEL_AUTO the plane-streaming
         kernel; ``rows`` (1 or 2, 0 = automatic) is the resident kernel's
         rows per thread; ``balanced`` (cache-free plane streaming only) cuts

@@ -12,6 +12,7 @@
 
 #include "internal.h"
 #include "stencil_registry.h"
+#include "stencil_patch.cuh"
 #include "stencil_slab.cuh"
 #include "stencil_strip.cuh"
 #include "stencil_tile.cuh"
@@ -142,6 +143,15 @@ std::vector<StripKEntry> &strip_registry() {
     return table;
 }
 
+std::vector<PatchEntry> &patch_registry() {
+    static std::vector<PatchEntry> table = [] {
+        std::vector<PatchEntry> t;
+        register_patch_kernels(t);
+        return t;
+    }();
+    return table;
+}
+
 std::vector<SlabEntry> &slab_registry() {
     static std::vector<SlabEntry> table = [] {
         std::vector<SlabEntry> t;
@@ -195,7 +205,9 @@ struct Plan {
     long long FS = 0;
     // column-strip kernel (2-D): ntx strips across x, ntz runs of rows
     StripKEntry *sk = nullptr;
-    double cost = 0.0;         // column strips: modelled SM cycles per step
+    double cost = 0.0;         // column strips and patches: modelled SM cycles per step
+    // patch kernel (2-D): ntx x ntz tiles, shared buffers of PW x PH cells
+    PatchEntry *qk = nullptr;
     // slab-streaming kernel (3-D): ntx x nty columns, 2^loglx lanes per row
     SlabEntry *lk = nullptr;
     int loglx = 0;
@@ -225,6 +237,7 @@ struct perks_stencil {
     int trace_steps = 0, trace_blocks = 0, trace_grid = 0;
     void *tfaces[2] = {nullptr, nullptr};  // resident-tile kernel: face buffers by step parity
     size_t tfaces_bytes = 0;
+    unsigned long long *pflags = nullptr;  // patch kernel: exchange counts, one per SM
     bool no_resident = false;             // plan the plane-streaming kernel only
     // The last plan made and what it was made for: a run of the same stencil under the same plan settings uses it
     // again (searching the tilings takes the host 50 to 400 us, as long as many runs).
@@ -408,6 +421,63 @@ perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts, int want_
     // halo cells: the overlap each item reads beyond its own cells, per step
     bp.halo_cells = ((long long)bp.ntx * bp.ntz * 32 * bp.sk->v * (2LL * bp.sk->ts * shape_by_id(st->shape_id).radius) +
                      (long long)bp.ntx * 2 * bp.sk->hl * bp.sk->v * Z) / bp.sk->ts;
+    pl = bp;
+    return PERKS_OK;
+}
+
+// Plan of the patch kernel (2-D domains whose tiles, with their halos, fit in
+// shared memory twice): the tiles by a model in SM cycles.  A step costs its cells' FP64 instructions at 16 cycles a warp (or
+// their issue slots at 4 a cycle), at least the latency of a pass and a block
+// barrier; an exchange some 4000 cycles.
+perks_status make_patch_plan(perks_stencil *st, Plan &pl, int want_k, int want_x, int want_z) {
+    perks_context *ctx = st->ctx;
+    const int dt = st->desc.dtype, X = st->X, Z = st->Z, SM = ctx->sm_count;
+    const int es = dt == PERKS_F64 ? 8 : 4;  // the buffers hold the accumulator type
+    double best = 1e300;
+    Plan bp;
+    if (st->desc.ndim == 2 && (dt != PERKS_BF16 || X % 8 == 0))
+        for (PatchEntry &e : patch_registry()) {
+            if (e.dtype != dt || e.shape != st->shape_id || (want_k > 0 && e.k != want_k)) continue;
+            int budget = 0;
+            const perks_status rc = smem_optin(ctx, (const void *)e.fn, &budget);
+            if (rc) return rc;
+            const ShapeInfo &sh = shape_by_id(st->shape_id);
+            const int R = sh.radius, H = e.k * R;
+            for (int ntx = want_x > 0 ? want_x : 1; ntx <= (want_x > 0 ? want_x : std::min(X, SM)); ++ntx) {
+                const int ntz = want_z > 0 ? want_z : std::min(std::max(Z / std::max(H, 4), 1), SM / ntx);
+                if (ntx < 1 || ntz < 1 || (long long)ntx * ntz > SM || ntx > X || ntz > Z) continue;
+                if ((ntx > 1 && X / ntx < H) || (ntz > 1 && Z / ntz < H)) continue;  // a halo reaches one tile far
+                const int tx = ceil_div(X, ntx), tz = ceil_div(Z, ntz);
+                const long long EW = tx + 2 * H, EH = tz + 2 * H;
+                if (2 * EW * EH * es > budget) continue;
+                double cyc = 4000.0;
+                for (int s = 1; s <= e.k; ++s) {
+                    const double cells = (tx + 2.0 * R * (e.k - s)) * (tz + 2.0 * R * (e.k - s));
+                    const double pass = std::ceil(cells / kPatchThreads);
+                    cyc += dt == PERKS_F64 ? std::max(cells / 2.0 * sh.npts, pass * 64.0 * sh.npts) + 400.0
+                                           : std::max(cells / 128.0 * (2.0 * sh.npts + 16.0), pass * (6.0 * sh.npts + 60.0)) + 250.0;
+                }
+                if (cyc / e.k < best) {
+                    best = cyc / e.k;
+                    bp.qk = &e;
+                    bp.ntx = ntx; bp.nty = 1; bp.ntz = ntz;
+                    bp.txmax = tx; bp.tymax = 1; bp.tzmax = tz;
+                    bp.PW = (int)EW; bp.PH = (int)EH;
+                    bp.smem = 2 * EW * EH * es;
+                    bp.blocks = ntx * ntz;
+                    bp.cached_cells = st->cells;
+                    bp.halo_cells = 2 * ((long long)ntx * ntz) * (EW * EH - (long long)tx * tz) / e.k;
+                }
+            }
+        }
+    if (!bp.qk)
+        return fail(ctx, PERKS_ERR_UNSUPPORTED,
+                    "patch kernel: 2-D stencils 2d5pt, 2ds9pt, 2d9pt, 2d25pt whose tiles fit in shared memory twice");
+    int per_sm = 0;
+    PERKS_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)bp.qk->fn, kPatchThreads,
+                                                                  (size_t)bp.smem));
+    if ((long long)per_sm * SM < bp.blocks)
+        return fail(ctx, PERKS_ERR_LAUNCH_TOO_LARGE, "patch kernel: %d blocks are not co-resident", bp.blocks);
     pl = bp;
     return PERKS_OK;
 }
@@ -658,12 +728,18 @@ perks_status make_base_plan(perks_stencil *st, Plan &pl, bool per_step = false) 
     return PERKS_OK;
 }
 
-// 2d5pt domains that fit on chip whole.  fp32 / bf16: the strips are faster at
-// every size (1.43 us per step against 2.66 at 256^2 fp32, 2.2 against 5.0 at
-// 1000^2).  fp64, both on the fp64 pipe: 5.9 against 8.5 us at 700 x 500, 12.1
-// against 13.9 at 1000^2; up to 64 K cells, where it is 3.1 against 3.9, the
-// domain stays resident (small domains are held on chip by default).
-bool strip_beats_resident(const perks_stencil *st) { return st->desc.dtype != PERKS_F64 || st->cells > 65536; }
+// A 2-D domain without a plan: the patch kernel rather than the column strips?
+// Up to the sizes below (us per step, patch / strips).  fp64, where a strip's
+// overlap costs FP64 cycles: 2d5pt as long as the domain fits (256^2 2.4 / 3.0,
+// 1000^2 12.0 / 12.9), 2d9pt 640^2 9.6 / 10.3 (1000^2 20.2 / 20.0), radius 2
+// 400^2 2d25pt 12.2 / 12.8 (640^2 24.5 / 23.4).  fp32 / bf16: 2d5pt 64^2 0.98 /
+// 1.31, 100^2 1.19 / 1.33 (256^2 1.47 / 1.43), radius 2 64^2 1.66 / 1.95 (100^2
+// 2.1 / 2.0).
+bool patch_beats(const perks_stencil *st) {
+    const bool r1 = shape_by_id(st->shape_id).radius == 1;
+    if (st->desc.dtype != PERKS_F64) return st->cells <= (r1 ? 1 << 15 : 1 << 13);
+    return st->shape_id == SH_2D5 || st->cells <= (r1 ? 1 << 19 : 1 << 18);
+}
 
 // A 3-D domain without a plan whose other plan is `base`: the slab kernel?
 // (Figures: us per step, other plan / slab.)
@@ -721,12 +797,12 @@ void choose_f64_3d7(perks_stencil *st, Plan &pl) {
 
 // The plan a run uses.  A domain without a plan takes, where the other kernels
 // could host it at all (so the domains that are refused stay the same), the
-// column-strip kernel (2-D) or the slab kernel (3-D)
+// patch or column-strip kernel (2-D) or the slab kernel (3-D)
 // where that is the faster one; a traced run keeps the kernels that mark every
 // step.
 perks_status search_plan(perks_stencil *st, Plan &pl, bool per_step) {
     const int kind = st->has_plan ? st->plan.reserved[2] : PERKS_KERNEL_AUTO;
-    const bool asked = !per_step && (kind == PERKS_KERNEL_STRIP || kind == PERKS_KERNEL_SLAB);
+    const bool asked = !per_step && (kind == PERKS_KERNEL_STRIP || kind == PERKS_KERNEL_SLAB || kind == PERKS_KERNEL_PATCH);
     const bool open = !per_step && !st->has_plan && !st->no_resident && !st->trace;
     if (!asked && !open) return make_base_plan(st, pl, per_step);
     st->has_plan = false;
@@ -734,11 +810,16 @@ perks_status search_plan(perks_stencil *st, Plan &pl, bool per_step) {
     st->has_plan = asked;
     if (rc) return rc;
     if (kind == PERKS_KERNEL_STRIP) return make_strip_plan(st, pl, st->plan.reserved[1], st->plan.tiles_z);
+    if (kind == PERKS_KERNEL_PATCH)
+        return make_patch_plan(st, pl, st->plan.reserved[1], st->plan.tiles_x, st->plan.tiles_z);
     if (kind == PERKS_KERNEL_SLAB) return make_slab_plan(st, pl);
     const std::string saved_msg = st->ctx->last_error;
-    Plan sp;
+    Plan sp, qp;
     if (st->desc.ndim == 2) {
-        if ((!pl.resident || strip_beats_resident(st)) && make_strip_plan(st, sp, 0, 0) == PERKS_OK) pl = sp;
+        const bool strip = make_strip_plan(st, sp, 0, 0) == PERKS_OK;
+        const bool patch = make_patch_plan(st, qp, 0, 0, 0) == PERKS_OK;
+        if (patch && (!strip || patch_beats(st))) pl = qp;
+        else if (strip) pl = sp;
     } else {
         if (make_slab_plan(st, sp) == PERKS_OK && slab_beats(st, pl, sp)) pl = sp;
         else if (st->shape_id == SH_3D7 && st->desc.dtype == PERKS_F64 && st->X % 2 == 0 && st->cells >= (1 << 22))
@@ -775,7 +856,17 @@ void fill_stats(const perks_stencil *st, const Plan *pl, long long steps, int va
     o->variant = variant;
     o->cells = st->cells;
     const double S = st->es;
-    if (variant == PERKS_PERSISTENT && pl && pl->lk) {
+    if (variant == PERKS_PERSISTENT && pl && pl->qk) {
+        o->kernel = PERKS_KERNEL_PATCH;
+        o->grid_blocks = pl->blocks;
+        o->threads_per_block = kPatchThreads;
+        o->tiles_x = pl->ntx; o->tiles_y = pl->nty; o->tiles_z = pl->ntz;
+        o->planes_per_sync = pl->qk->k;  // steps per exchange
+        o->smem_bytes_per_block = pl->smem;
+        o->cached_cells = pl->cached_cells;
+        o->halo_cells_per_step = pl->halo_cells;
+        o->algorithmic_bytes = steps > 0 ? S * (2.0 * (double)st->cells + (double)steps * pl->halo_cells) : 0.0;
+    } else if (variant == PERKS_PERSISTENT && pl && pl->lk) {
         o->kernel = PERKS_KERNEL_SLAB;
         o->grid_blocks = pl->blocks;
         o->threads_per_block = kSlabThreads;
@@ -920,6 +1011,35 @@ perks_status run_strip(perks_stencil *st, long long steps, cudaStream_t s, const
     return PERKS_OK;
 }
 
+// One cooperative launch of the patch kernel.
+perks_status run_patch(perks_stencil *st, long long steps, cudaStream_t s, const Plan &pl) {
+    perks_context *ctx = st->ctx;
+    const size_t flag_bytes = sizeof(unsigned long long) * ctx->sm_count;
+    if (!st->pflags) PERKS_CUDA(ctx, cudaMalloc(&st->pflags, flag_bytes));
+    if (!st->err) PERKS_CUDA(ctx, cudaMalloc(&st->err, sizeof(DevError)));
+    PatchArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.X = st->X; a.Z = st->Z;
+    a.ntx = pl.ntx; a.nty = pl.ntz;
+    a.EW = pl.PW; a.EH = pl.PH;
+    a.steps = steps;
+    a.boundary = st->desc.boundary;
+    a.boundary_f = (float)st->desc.boundary;
+    for (int i = 0; i < 25; ++i) { a.w[i] = st->kw[i]; a.wf[i] = (float)st->kw[i]; }
+    a.field[0] = st->field[st->cur];
+    a.field[1] = st->field[st->cur ^ 1];
+    a.flags = st->pflags;
+    a.err = st->err;
+    a.timeout_ns = ctx->timeout_ns;
+    PERKS_CUDA(ctx, cudaMemsetAsync(st->pflags, 0, flag_bytes, s));
+    PERKS_CUDA(ctx, cudaMemsetAsync(st->err, 0, sizeof(DevError), s));
+    void *args[] = {&a};
+    PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)pl.qk->fn, dim3(pl.blocks), dim3(kPatchThreads), args,
+                                                (size_t)pl.smem, s));
+    if (((steps + pl.qk->k - 1) / pl.qk->k) & 1) st->cur ^= 1;
+    return PERKS_OK;
+}
+
 // One cooperative launch of the slab-streaming kernel.
 perks_status run_slab(perks_stencil *st, long long steps, cudaStream_t s, const Plan &pl) {
     perks_context *ctx = st->ctx;
@@ -1016,6 +1136,7 @@ perks_status run_persistent(perks_stencil *st, long long steps, cudaStream_t s, 
     if (pl.resident) return run_resident(st, steps, s, pl);
     if (pl.sk) return run_strip(st, steps, s, pl);
     if (pl.lk) return run_slab(st, steps, s, pl);
+    if (pl.qk) return run_patch(st, steps, s, pl);
     rc = ensure_persistent_buffers(st, pl);
     if (rc) return rc;
     int per_sm = 0;
@@ -1164,6 +1285,7 @@ extern "C" perks_status perks_stencil_destroy(perks_stencil *st) {
     if (st->bar) cudaFree(st->bar);
     if (st->err) cudaFree(st->err);
     if (st->trace) cudaFree(st->trace);
+    if (st->pflags) cudaFree(st->pflags);
     delete st;
     return PERKS_OK;
 }
@@ -1206,9 +1328,9 @@ extern "C" perks_status perks_stencil_set_plan(perks_stencil *st, const perks_st
         !(plan->reserved[2] == PERKS_KERNEL_STRIP && plan->reserved[1] == 1))
         return fail(st->ctx, PERKS_ERR_INVALID_ARG, "stencil_set_plan: planes per barrier must be 0, 2 or 4");
     if (plan->reserved[2] < PERKS_KERNEL_AUTO || (plan->reserved[2] > PERKS_KERNEL_STREAMING && plan->reserved[2] != PERKS_KERNEL_STRIP &&
-         plan->reserved[2] != PERKS_KERNEL_SLAB))
+         plan->reserved[2] != PERKS_KERNEL_SLAB && plan->reserved[2] != PERKS_KERNEL_PATCH))
         return fail(st->ctx, PERKS_ERR_INVALID_ARG,
-                    "stencil_set_plan: kernel must be AUTO, RESIDENT, STREAMING, STRIP or SLAB");
+                    "stencil_set_plan: kernel must be AUTO, RESIDENT, STREAMING, STRIP, SLAB or PATCH");
     if (plan->reserved[3] != 0 && plan->reserved[3] != 256 && plan->reserved[3] != 512 && plan->reserved[3] != 1024)
         return fail(st->ctx, PERKS_ERR_INVALID_ARG, "stencil_set_plan: threads must be 0, 256, 512 or 1024");
     st->plan = *plan;
@@ -1415,10 +1537,10 @@ extern "C" perks_status perks_stencil_autotune(perks_stencil *st, int32_t varian
             }
             ctx->last_error = saved_msg;
         }
-    // slab-streaming kernel
-    if (!per_step && !st->no_resident && st->desc.ndim == 3) {
+    // slab-streaming (3-D) or patch (2-D) kernel
+    if (!per_step && !st->no_resident) {
         perks_stencil_plan p{};
-        p.reserved[2] = PERKS_KERNEL_SLAB;
+        p.reserved[2] = st->desc.ndim == 3 ? PERKS_KERNEL_SLAB : PERKS_KERNEL_PATCH;
         st->plan = p;
         st->has_plan = true;
         Plan probe;

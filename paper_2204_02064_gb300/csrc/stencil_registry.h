@@ -58,6 +58,9 @@ void register_slab_f64(std::vector<SlabEntry> &out);
 void register_slab_f32(std::vector<SlabEntry> &out);
 void register_slab_bf16(std::vector<SlabEntry> &out);
 
+struct PatchEntry;  // stencil_patch.cuh
+void register_patch_kernels(std::vector<PatchEntry> &out);
+
 struct TileKernelEntry;  // stencil_tile.cuh
 void register_tile_kernels(std::vector<TileKernelEntry> &out);
 

@@ -1,6 +1,7 @@
-"""GPU parity of the slab-streaming kernel (3-D) against the oracle, at the
-edges of its tiles: rows that no vector width divides, fewer rows than a thread
-owns, columns cut in the middle of a block's share.
+"""GPU parity of the slab-streaming kernel (3-D) and the patch kernel (small
+2-D domains) against the oracle, at the edges of their tiles: rows that no
+vector width divides, fewer rows than a thread owns, columns cut in the middle
+of a block's share, halos as deep as a tile, fewer steps than an exchange.
 fp64 within 1e-12 of the local value (floored at 1e-3 of the field maximum);
 fp32 / bf16 storage bit for bit against the low-precision oracle."""
 import numpy as np
@@ -57,6 +58,43 @@ def test_slab_matches_oracle(ctx, oracle, name, dtype, shape, steps):
     if dtype == "bf16":
         shape = shape[:2] + (shape[2] // 8 * 8,)
     _check(ctx, oracle, name, dtype, shape, steps, api.KERNEL_SLAB)
+
+
+@pytest.mark.parametrize("name", ["2d5pt", "2ds9pt", "2d9pt", "2d25pt"])
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("shape,steps,tiles", [((8, 16), 5, 0), ((16, 24), 7, 3), ((64, 104), 1, 13), ((131, 93), 10, 0),
+                                               ((257, 64), 3, 1), ((90, 328), 6, 0)])
+def test_patch_matches_oracle(ctx, oracle, name, dtype, shape, steps, tiles):
+    from paper_2204_02064_gb300 import api
+    if dtype == "bf16":
+        shape = (shape[0], shape[1] // 8 * 8)
+    stats = _check(ctx, oracle, name, dtype, shape, steps, api.KERNEL_PATCH, tiles=(tiles, 0, 0))
+    assert stats["cached_cells"] == shape[0] * shape[1]
+
+
+def test_patch_wait_timeout_reported(ctx, oracle):
+    """A block that waits for its neighbours past the limit ends the run with
+    BARRIER_TIMEOUT; the context keeps working."""
+    from paper_2204_02064_gb300 import api
+    f = inputs.stencil_field((256, 256), 52)
+    offs, w = inputs.shape_offsets("2d5pt"), inputs.workload_weights("2d5pt")
+    st = api.Stencil(ctx, f.shape, offs, w)
+    src = torch.from_numpy(f).cuda()
+    st.set_field(src)
+    assert st.describe(40)["kernel"] == api.KERNEL_PATCH
+    ctx.set_barrier_timeout(0)
+    try:
+        with pytest.raises(api.PerksError) as ei:
+            st.run(40, stats=True)
+        assert ei.value.name == "BARRIER_TIMEOUT"
+    finally:
+        ctx.set_barrier_timeout(2_000_000_000)
+    st.set_field(src)
+    st.run(13, stats=True)
+    out = torch.empty_like(src)
+    st.get_field(out)
+    torch.cuda.synchronize()
+    assert rel_err(out.cpu().numpy(), oracle.stencil_run(f, offs, w, 13)) <= 1e-12
 
 
 def test_plan_is_kept_until_the_request_changes(ctx):

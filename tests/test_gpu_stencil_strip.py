@@ -74,7 +74,7 @@ def test_strip_barrier_timeout_and_trace(ctx, oracle):
     """A barrier wait between two sweeps that gives up is reported and the
     context keeps working; a traced run marks every step (another kernel)."""
     from paper_2204_02064_gb300 import api
-    f = inputs.stencil_field((300, 512), 48)
+    f = inputs.stencil_field((1200, 1024), 48)
     offs, w = inputs.shape_offsets("2d9pt"), inputs.workload_weights("2d9pt")
     st = api.Stencil(ctx, f.shape, offs, w)
     src = torch.from_numpy(f).cuda()
