@@ -184,7 +184,7 @@ def field_error(torch, got, ref):
 
 
 def kernel_name(desc):
-    return {1: "resident", 2: "streaming", 3: "per_step"}.get(desc.get("kernel"), "unknown")
+    return {1: "resident", 2: "streaming", 3: "per_step", 4: "strip", 5: "slab", 6: "patch"}.get(desc.get("kernel"), "unknown")
 
 
 def stencil2d_leg(api, torch, ctx, L, steps, variant, K, W):

@@ -447,6 +447,32 @@ __device__ __forceinline__ void sum_over_warps(const float (&v)[N], float *s, fl
     }
 }
 
+// A warp's walk over the pixels q, q + step, ...: image and pixel
+// within the image by additions, where q / plane and q % plane are 64-bit
+// divisions of some hundred instructions each.
+struct PixelWalk {
+    long long q, step;
+    int img, p, plane, dimg, dp;
+    __device__ __forceinline__ PixelWalk(long long first, long long stride, long long plane_)
+        : q(first), step(stride), img((int)(first / plane_)), p((int)(first % plane_)), plane((int)plane_),
+          dimg((int)(stride / plane_)), dp((int)(stride % plane_)) {}
+    __device__ __forceinline__ void next() {
+        q += step;
+        img += dimg;
+        p += dp;
+        if (p >= plane) {
+            p -= plane;
+            ++img;
+        }
+    }
+};
+
+// Pixels whose loads a warp of the first and last layers' weight gradients has
+// in flight: their bound is the latency of a pixel's loads (16 images of 64^2:
+// 27 us each with one pixel at a time and two 64-bit divisions per pixel, 14
+// and 16 now).
+constexpr int kWgAhead = 4;
+
 // Last layer (32 -> 1): part[block][ci][tap] = sum_q dy[q - off(tap)] x3[q][ci]; a warp visits pixels, lane = ci,
 // so every activation is read once.  The bias sum rides along.
 template <typename S>
@@ -457,17 +483,28 @@ __global__ void __launch_bounds__(256) wgrad_last_kernel(const S *__restrict__ x
     const int lane = threadIdx.x & 31;
     const long long plane = (long long)H * W, total = plane * nimg;
     float acc[10] = {};
-    for (long long q = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; q < total;
-         q += ((long long)gridDim.x * blockDim.x) >> 5) {
-        const int p = (int)(q % plane), y = p / W, x = p % W;
-        const float v = ld_f(x3 + q * kMaxC + lane);
+    PixelWalk at((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5, ((long long)gridDim.x * blockDim.x) >> 5, plane);
+    while (at.q < total) {
+        float v[kWgAhead], d[kWgAhead][10];
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-            const int oy = -(tap / 3 - 1) * dil, ox = -(tap % 3 - 1) * dil;
-            const bool inside = y + oy >= 0 && y + oy < H && x + ox >= 0 && x + ox < W;
-            acc[tap] = fmaf(inside ? dy[q + (long long)oy * W + ox] : 0.f, v, acc[tap]);
+        for (int u = 0; u < kWgAhead; ++u, at.next()) {
+            const bool in = at.q < total;
+            const int y = at.p / W, x = at.p % W;
+            v[u] = in ? ld_f(x3 + at.q * kMaxC + lane) : 0.f;
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap) {
+                const int oy = -(tap / 3 - 1) * dil, ox = -(tap % 3 - 1) * dil;
+                const bool inside = in && y + oy >= 0 && y + oy < H && x + ox >= 0 && x + ox < W;
+                d[u][tap] = inside ? dy[at.q + (long long)oy * W + ox] : 0.f;
+            }
+            d[u][9] = in ? dy[at.q] : 0.f;
         }
-        if (lane == 0) acc[9] += dy[q];
+#pragma unroll
+        for (int u = 0; u < kWgAhead; ++u) {
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap) acc[tap] = fmaf(d[u][tap], v[u], acc[tap]);
+            if (lane == 0) acc[9] += d[u][9];
+        }
     }
     sum_over_warps(acc, s, part + (long long)blockIdx.x * nparams,
                    [&](int i, int l) { return i < 9 ? off_w + l * 9 + i : l == 0 ? off_b : -1; });
@@ -482,21 +519,25 @@ __global__ void __launch_bounds__(256) wgrad_first_kernel(const S *__restrict__ 
     const int lane = threadIdx.x & 31;
     const long long plane = (long long)H * W, total = plane * nimg;
     float acc[19] = {};
-    for (long long q = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; q < total;
-         q += ((long long)gridDim.x * blockDim.x) >> 5) {
-        const long long img = q / plane;
-        const int p = (int)(q % plane), y = p / W, x = p % W;
-        const float d = dy[q * kMaxC + lane];
-        // lanes 0..17 load the 18 inputs of the pixel, shuffles hand them to every lane
-        float mine = 0.f;
-        if (lane < 18) {
-            const int ci = lane / 9, tap = lane % 9;
-            const int yy = y + (tap / 3 - 1) * dil, xx = x + (tap % 3 - 1) * dil;
-            if (yy >= 0 && yy < H && xx >= 0 && xx < W) mine = ld_f(x0 + (img * 2 + ci) * plane + (long long)yy * W + xx);
+    const int ci = lane / 9, oy = (lane % 9 / 3 - 1) * dil, ox = (lane % 3 - 1) * dil;  // lane's input (9 = 3 x 3 taps)
+    PixelWalk at((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5, ((long long)gridDim.x * blockDim.x) >> 5, plane);
+    while (at.q < total) {
+        // lanes 0..17 load the 18 inputs of a pixel, shuffles hand them to every lane
+        float d[kWgAhead], mine[kWgAhead];
+#pragma unroll
+        for (int u = 0; u < kWgAhead; ++u, at.next()) {
+            const bool in = at.q < total;
+            const int yy = at.p / W + oy, xx = at.p % W + ox;
+            d[u] = in ? dy[at.q * kMaxC + lane] : 0.f;
+            mine[u] = in && lane < 18 && yy >= 0 && yy < H && xx >= 0 && xx < W
+                          ? ld_f(x0 + ((long long)at.img * 2 + ci) * plane + (long long)yy * W + xx) : 0.f;
         }
 #pragma unroll
-        for (int i = 0; i < 18; ++i) acc[i] = fmaf(d, __shfl_sync(0xffffffffu, mine, i), acc[i]);
-        acc[18] += d;
+        for (int u = 0; u < kWgAhead; ++u) {
+#pragma unroll
+            for (int i = 0; i < 18; ++i) acc[i] = fmaf(d[u], __shfl_sync(0xffffffffu, mine[u], i), acc[i]);
+            acc[18] += d[u];
+        }
     }
     sum_over_warps(acc, s, part + (long long)blockIdx.x * nparams,
                    [&](int i, int l) { return i < 18 ? off_w + l * 18 + i : off_b + l; });
@@ -925,10 +966,10 @@ perks_status forward(perks_warmnet *n, int nimg, int ny, int nx, const double *k
     const int pgrid = (int)std::min<long long>((pixels + 255) / 256, 16LL * ctx->sm_count);  // thread per pixel
     S *x0 = (S *)n->x0, *x1 = (S *)n->x1, *x2 = (S *)n->x2, *x3 = (S *)n->x3;
     const int cells = kPoolThreads / n->pool;
-    // jobs of F fine rows: far below 2^31 for any k that fits in memory.  A round per block where that fills three
-    // blocks per SM, rounds of several jobs beyond
+    // jobs of F fine rows: far below 2^31 for any k that fits in memory.  One round per block of three blocks per SM,
+    // as long as that takes no more than kPoolJobs (16 images: rounds of 4 in two turns 44 us, of 5 in one 35)
     const int jobs = (int)((long long)nimg * H * ((W + cells - 1) / cells));
-    const int nj = std::max(1, std::min(kPoolJobs, jobs / (3 * ctx->sm_count)));
+    const int nj = std::min(kPoolJobs, (jobs + 3 * ctx->sm_count - 1) / (3 * ctx->sm_count));
     const size_t fsm = pool_smem(nj, u != nullptr);
     perks_status frc = set_smem(ctx, features_kernel<S>, pool_smem(kPoolJobs, true));
     if (frc) return frc;
