@@ -537,8 +537,10 @@ perks_status perks_poisson_solve(perks_poisson *p, const double *b, double *x, d
  * block is faster (256 problems of 512^2 to 1e-8, before the diagonal was
  * precomputed: 23.6 s vs 31.8 s).  Errors: INVALID_ARG. */
 perks_status perks_poisson_set_block_threads(perks_poisson *p, int32_t threads);
-/* Blocks per problem: 1, 2, 4 or 8, or 0 (the default: for problems of
- * 65536 cells and more 8 with one row per pass, 4 with four, and 1 below;
+/* Blocks per problem: 1, 2, 4 or 8, or 0 (the default: with one row per
+ * pass the number that finishes the batch soonest by a cost model, 8 for
+ * problems of 65536 cells and 1 up to 8192 cells where all of the batch runs
+ * at once; with four rows per pass 4 for problems of 65536 cells and more;
  * 256 problems of 512^2 to 1e-8 at four rows per pass take 20.2 s with C =
  * 1, 16.4 s with 2 and 15.9 s with 4).  With C > 1 each problem's
  * rows are split over a group of C blocks that meet at a bounded barrier of
