@@ -426,9 +426,10 @@ perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts, int want_
 }
 
 // Plan of the patch kernel (2-D domains whose tiles, with their halos, fit in
-// shared memory twice): the tiles by a model in SM cycles.  A step costs its cells' FP64 instructions at 16 cycles a warp (or
-// their issue slots at 4 a cycle), at least the latency of a pass and a block
-// barrier; an exchange some 4000 cycles.
+// shared memory twice): the tiles by a model in SM cycles.  A step costs its
+// cells' FP64 instructions at 16 cycles a warp (or their issue slots at 4 a
+// cycle), at least the latency of a pass and a block barrier; an exchange some
+// 4000 cycles.
 perks_status make_patch_plan(perks_stencil *st, Plan &pl, int want_k, int want_x, int want_z) {
     perks_context *ctx = st->ctx;
     const int dt = st->desc.dtype, X = st->X, Z = st->Z, SM = ctx->sm_count;
