@@ -800,11 +800,19 @@ void choose_f64_3d7(perks_stencil *st, Plan &pl) {
 // could host it at all (so the domains that are refused stay the same), the
 // patch or column-strip kernel (2-D) or the slab kernel (3-D)
 // where that is the faster one; a traced run keeps the kernels that mark every
-// step.
+// step, also under a plan that names one of the three (such a plan is what the
+// autotuner may have left).
 perks_status search_plan(perks_stencil *st, Plan &pl, bool per_step) {
     const int kind = st->has_plan ? st->plan.reserved[2] : PERKS_KERNEL_AUTO;
-    const bool asked = !per_step && (kind == PERKS_KERNEL_STRIP || kind == PERKS_KERNEL_SLAB || kind == PERKS_KERNEL_PATCH);
+    const bool named = kind == PERKS_KERNEL_STRIP || kind == PERKS_KERNEL_SLAB || kind == PERKS_KERNEL_PATCH;
+    const bool asked = !per_step && named && !st->trace;
     const bool open = !per_step && !st->has_plan && !st->no_resident && !st->trace;
+    if (named && st->trace && !per_step) {
+        st->has_plan = false;
+        const perks_status rt = make_base_plan(st, pl, false);
+        st->has_plan = true;
+        return rt;
+    }
     if (!asked && !open) return make_base_plan(st, pl, per_step);
     st->has_plan = false;
     perks_status rc = make_base_plan(st, pl, false);
@@ -1522,8 +1530,9 @@ extern "C" perks_status perks_stencil_autotune(perks_stencil *st, int32_t varian
             }
             ctx->last_error = saved_msg;
         }
-    // column-strip kernel: the model's runs of rows for each compiled number of steps per sweep
-    if (!per_step && !st->no_resident && st->desc.ndim == 2)
+    // column-strip kernel: the model's runs of rows for each compiled number of steps per sweep (not
+    // while a trace is on: a traced run would take another kernel)
+    if (!per_step && !st->no_resident && !st->trace && st->desc.ndim == 2)
         for (int ts : {1, 2, 4}) {
             perks_stencil_plan p{};
             p.reserved[1] = ts;
@@ -1539,7 +1548,7 @@ extern "C" perks_status perks_stencil_autotune(perks_stencil *st, int32_t varian
             ctx->last_error = saved_msg;
         }
     // slab-streaming (3-D) or patch (2-D) kernel
-    if (!per_step && !st->no_resident) {
+    if (!per_step && !st->no_resident && !st->trace) {
         perks_stencil_plan p{};
         p.reserved[2] = st->desc.ndim == 3 ? PERKS_KERNEL_SLAB : PERKS_KERNEL_PATCH;
         st->plan = p;

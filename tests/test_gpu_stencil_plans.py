@@ -1,0 +1,85 @@
+"""What a stencil does under a plan that names the column-strip, slab or patch
+kernel and in the calls that plan is not made for: traced runs, per-step runs,
+captured runs, tilings the kernel cannot take.  fp64 within 1e-12 of the local
+value (floored at 1e-3 of the field maximum); fp32 bit for bit."""
+import numpy as np
+import pytest
+
+from paper_2204_02064_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+TT = {"f64": torch.float64, "f32": torch.float32, "bf16": torch.bfloat16}
+
+
+def rel_err(g, o):
+    floor = 1e-3 * max(np.max(np.abs(o)), 1e-300)
+    return float(np.max(np.abs(g - o) / np.maximum(np.abs(o), floor)))
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2204_02064_gb300 import api
+    return api.Context(0)
+
+
+# kernel, stencil, grid shape
+NAMED = [("STRIP", "2d9pt", (200, 256)), ("STRIP", "2d5pt", (1200, 1024)), ("PATCH", "2d5pt", (96, 128)),
+         ("SLAB", "3d7pt", (20, 24, 32)), ("SLAB", "3d27pt", (33, 29, 40))]
+
+
+class Case:
+    def __init__(self, ctx, name, shape, dtype="f64"):
+        from paper_2204_02064_gb300 import api
+        self.dtype = dtype
+        self.offs, self.w = inputs.shape_offsets(name), inputs.workload_weights(name, seed=5)
+        self.st = api.Stencil(ctx, shape, self.offs, self.w, dtype=dtype, boundary=0.25)
+        self.src = torch.from_numpy(inputs.stencil_field(shape, 81)).to(TT[dtype]).cuda()
+        self.st.set_field(self.src)
+
+    def check(self, oracle, steps):
+        out = torch.empty_like(self.src)
+        self.st.get_field(out)
+        torch.cuda.synchronize()
+        f = self.src.cpu().numpy()
+        if self.dtype == "f64":
+            assert rel_err(out.cpu().numpy(), oracle.stencil_run(f, self.offs, self.w, steps, boundary=0.25)) <= 1e-12
+        else:
+            ref = oracle.stencil_run_lowp(f, self.offs, self.w, steps, self.dtype, boundary=0.25)
+            assert np.array_equal(out.float().cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("kernel,name,shape", NAMED)
+def test_trace_under_a_plan_that_names_a_kernel_without_marks(ctx, oracle, kernel, name, shape):
+    """A traced run marks every step whatever the plan names; without the trace the plan holds again."""
+    from paper_2204_02064_gb300 import api
+    c = Case(ctx, name, shape)
+    want = getattr(api, "KERNEL_" + kernel)
+    c.st.set_plan(kernel=want)
+    assert c.st.run(2, stats=True)["kernel"] == want
+    c.st.set_trace(3)
+    assert c.st.describe(5)["kernel"] in (api.KERNEL_RESIDENT, api.KERNEL_STREAMING)
+    stats = c.st.run(5, stats=True)
+    tr = c.st.trace().astype(np.int64)
+    assert tr.shape == (4, stats["grid_blocks"], 2)
+    assert (tr[1:] > 0).all() and (tr[1:, :, 1] >= tr[1:, :, 0]).all()
+    c.st.set_trace(0)
+    assert c.st.run(1, stats=True)["kernel"] == want
+    c.check(oracle, 8)
+    c.st.close()
+
+
+@pytest.mark.parametrize("name,shape", [("2d9pt", (200, 256)), ("3d27pt", (33, 29, 40))])
+def test_autotune_then_trace(ctx, oracle, name, shape):
+    """The plan the autotuner leaves, whichever kernel it names, can be traced; tuned under a
+    trace it names one that marks its steps."""
+    from paper_2204_02064_gb300 import api
+    c = Case(ctx, name, shape)
+    c.st.autotune(probe_steps=4)
+    c.st.set_trace(2)
+    stats = c.st.run(3, stats=True)
+    assert c.st.trace().shape == (3, stats["grid_blocks"], 2)
+    assert c.st.autotune(probe_steps=4)["kernel"] in ("resident", "streaming")
+    c.check(oracle, 3)
+    c.st.close()
