@@ -799,17 +799,18 @@ void choose_f64_3d7(perks_stencil *st, Plan &pl) {
 // The plan a run uses.  A domain without a plan takes, where the other kernels
 // could host it at all (so the domains that are refused stay the same), the
 // patch or column-strip kernel (2-D) or the slab kernel (3-D)
-// where that is the faster one; a traced run keeps the kernels that mark every
-// step, also under a plan that names one of the three (such a plan is what the
-// autotuner may have left).
+// where that is the faster one.  A plan that names one of the three (it may be
+// the autotuner's) is for untraced persistent runs: a traced run keeps the
+// kernels that mark every step, and a per-step run, which such a plan's tiles
+// do not fit, takes the tiling it takes without a plan.
 perks_status search_plan(perks_stencil *st, Plan &pl, bool per_step) {
     const int kind = st->has_plan ? st->plan.reserved[2] : PERKS_KERNEL_AUTO;
     const bool named = kind == PERKS_KERNEL_STRIP || kind == PERKS_KERNEL_SLAB || kind == PERKS_KERNEL_PATCH;
     const bool asked = !per_step && named && !st->trace;
     const bool open = !per_step && !st->has_plan && !st->no_resident && !st->trace;
-    if (named && st->trace && !per_step) {
+    if (named && !asked) {
         st->has_plan = false;
-        const perks_status rt = make_base_plan(st, pl, false);
+        const perks_status rt = make_base_plan(st, pl, per_step);
         st->has_plan = true;
         return rt;
     }

@@ -83,3 +83,19 @@ def test_autotune_then_trace(ctx, oracle, name, shape):
     assert c.st.autotune(probe_steps=4)["kernel"] in ("resident", "streaming")
     c.check(oracle, 3)
     c.st.close()
+
+
+@pytest.mark.parametrize("kernel,name,shape", NAMED)
+def test_per_step_run_under_a_plan_that_names_a_persistent_kernel(ctx, oracle, kernel, name, shape):
+    """Such a plan's tiles (as the autotuner leaves them) are the persistent kernel's; a per-step run takes its own."""
+    from paper_2204_02064_gb300 import api
+    c = Case(ctx, name, shape)
+    want = getattr(api, "KERNEL_" + kernel)
+    c.st.set_plan(kernel=want)
+    d = c.st.describe(4)
+    c.st.set_plan(kernel=want, tiles=(d["tiles_x"], d["tiles_y"], d["tiles_z"]))
+    assert c.st.run(2, stats=True)["kernel"] == want
+    c.st.run(3, api.PER_STEP)
+    assert c.st.run(1, stats=True)["kernel"] == want
+    c.check(oracle, 6)
+    c.st.close()
