@@ -227,7 +227,7 @@ struct perks_stencil {
     int cur = 0;
     void *faces[2] = {nullptr, nullptr};
     size_t faces_bytes = 0;
-    unsigned long long *bar = nullptr;
+    unsigned long long *bar = nullptr;     // barrier counter, then the patch kernel's exchange counts, one per SM
     DevError *err = nullptr;
     int shape_id = -1;
     double kw[kMaxKernelPoints] = {};
@@ -237,7 +237,6 @@ struct perks_stencil {
     int trace_steps = 0, trace_blocks = 0, trace_grid = 0;
     void *tfaces[2] = {nullptr, nullptr};  // resident-tile kernel: face buffers by step parity
     size_t tfaces_bytes = 0;
-    unsigned long long *pflags = nullptr;  // patch kernel: exchange counts, one per SM
     bool no_resident = false;             // plan the plane-streaming kernel only
     // The last plan made and what it was made for: a run of the same stencil under the same plan settings uses it
     // again (searching the tilings takes the host 50 to 400 us, as long as many runs).
@@ -931,6 +930,16 @@ void fill_stats(const perks_stencil *st, const Plan *pl, long long steps, int va
     }
 }
 
+// The counters and the error record of every persistent kernel: whichever runs
+// first allocates them for all, so that a later run under capture, where
+// nothing can be allocated, may take another one.
+perks_status ensure_sync(perks_stencil *st) {
+    perks_context *ctx = st->ctx;
+    if (!st->bar) PERKS_CUDA(ctx, cudaMalloc(&st->bar, sizeof(unsigned long long) * (1 + (size_t)ctx->sm_count)));
+    if (!st->err) PERKS_CUDA(ctx, cudaMalloc(&st->err, sizeof(DevError)));
+    return PERKS_OK;
+}
+
 perks_status ensure_tile_buffers(perks_stencil *st, const Plan &pl) {
     perks_context *ctx = st->ctx;
     const size_t need = (size_t)pl.blocks * (size_t)pl.FS * st->es;
@@ -943,9 +952,7 @@ perks_status ensure_tile_buffers(perks_stencil *st, const Plan &pl) {
         for (int i = 0; i < 2; ++i) PERKS_CUDA(ctx, cudaMalloc(&st->tfaces[i], need));
         st->tfaces_bytes = need;
     }
-    if (!st->bar) PERKS_CUDA(ctx, cudaMalloc(&st->bar, sizeof(unsigned long long)));
-    if (!st->err) PERKS_CUDA(ctx, cudaMalloc(&st->err, sizeof(DevError)));
-    return PERKS_OK;
+    return ensure_sync(st);
 }
 
 // One cooperative launch of the resident-tile kernel: reads field[cur] before
@@ -996,8 +1003,8 @@ perks_status run_resident(perks_stencil *st, long long steps, cudaStream_t s, co
 // One cooperative launch of the column-strip kernel, sk->ts steps per sweep.
 perks_status run_strip(perks_stencil *st, long long steps, cudaStream_t s, const Plan &pl) {
     perks_context *ctx = st->ctx;
-    if (!st->bar) PERKS_CUDA(ctx, cudaMalloc(&st->bar, sizeof(unsigned long long)));
-    if (!st->err) PERKS_CUDA(ctx, cudaMalloc(&st->err, sizeof(DevError)));
+    const perks_status rc = ensure_sync(st);
+    if (rc) return rc;
     StripKArgs a;
     std::memset(&a, 0, sizeof(a));
     a.X = st->X; a.Z = st->Z;
@@ -1024,9 +1031,8 @@ perks_status run_strip(perks_stencil *st, long long steps, cudaStream_t s, const
 // One cooperative launch of the patch kernel.
 perks_status run_patch(perks_stencil *st, long long steps, cudaStream_t s, const Plan &pl) {
     perks_context *ctx = st->ctx;
-    const size_t flag_bytes = sizeof(unsigned long long) * ctx->sm_count;
-    if (!st->pflags) PERKS_CUDA(ctx, cudaMalloc(&st->pflags, flag_bytes));
-    if (!st->err) PERKS_CUDA(ctx, cudaMalloc(&st->err, sizeof(DevError)));
+    const perks_status rc = ensure_sync(st);
+    if (rc) return rc;
     PatchArgs a;
     std::memset(&a, 0, sizeof(a));
     a.X = st->X; a.Z = st->Z;
@@ -1038,10 +1044,10 @@ perks_status run_patch(perks_stencil *st, long long steps, cudaStream_t s, const
     for (int i = 0; i < 25; ++i) { a.w[i] = st->kw[i]; a.wf[i] = (float)st->kw[i]; }
     a.field[0] = st->field[st->cur];
     a.field[1] = st->field[st->cur ^ 1];
-    a.flags = st->pflags;
+    a.flags = st->bar + 1;
     a.err = st->err;
     a.timeout_ns = ctx->timeout_ns;
-    PERKS_CUDA(ctx, cudaMemsetAsync(st->pflags, 0, flag_bytes, s));
+    PERKS_CUDA(ctx, cudaMemsetAsync(st->bar + 1, 0, sizeof(unsigned long long) * ctx->sm_count, s));
     PERKS_CUDA(ctx, cudaMemsetAsync(st->err, 0, sizeof(DevError), s));
     void *args[] = {&a};
     PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)pl.qk->fn, dim3(pl.blocks), dim3(kPatchThreads), args,
@@ -1053,8 +1059,8 @@ perks_status run_patch(perks_stencil *st, long long steps, cudaStream_t s, const
 // One cooperative launch of the slab-streaming kernel.
 perks_status run_slab(perks_stencil *st, long long steps, cudaStream_t s, const Plan &pl) {
     perks_context *ctx = st->ctx;
-    if (!st->bar) PERKS_CUDA(ctx, cudaMalloc(&st->bar, sizeof(unsigned long long)));
-    if (!st->err) PERKS_CUDA(ctx, cudaMalloc(&st->err, sizeof(DevError)));
+    const perks_status rc = ensure_sync(st);
+    if (rc) return rc;
     SlabArgs a;
     std::memset(&a, 0, sizeof(a));
     a.X = st->X; a.Y = st->Y; a.Z = st->Z;
@@ -1095,9 +1101,7 @@ perks_status ensure_persistent_buffers(perks_stencil *st, const Plan &pl) {
         for (int i = 0; i < 2; ++i) PERKS_CUDA(ctx, cudaMalloc(&st->faces[i], need));
         st->faces_bytes = need;
     }
-    if (!st->bar) PERKS_CUDA(ctx, cudaMalloc(&st->bar, sizeof(unsigned long long)));
-    if (!st->err) PERKS_CUDA(ctx, cudaMalloc(&st->err, sizeof(DevError)));
-    return PERKS_OK;
+    return ensure_sync(st);
 }
 
 perks_status read_dev_error(perks_stencil *st, cudaStream_t s) {
@@ -1295,7 +1299,6 @@ extern "C" perks_status perks_stencil_destroy(perks_stencil *st) {
     if (st->bar) cudaFree(st->bar);
     if (st->err) cudaFree(st->err);
     if (st->trace) cudaFree(st->trace);
-    if (st->pflags) cudaFree(st->pflags);
     delete st;
     return PERKS_OK;
 }

@@ -99,3 +99,29 @@ def test_per_step_run_under_a_plan_that_names_a_persistent_kernel(ctx, oracle, k
     assert c.st.run(1, stats=True)["kernel"] == want
     c.check(oracle, 6)
     c.st.close()
+
+
+@pytest.mark.parametrize("first", ["trace", "plan"])
+@pytest.mark.parametrize("name,shape,dtype", [("2d5pt", (96, 128), "f64"), ("2d5pt", (1200, 1024), "f64"),
+                                              ("3d27pt", (33, 29, 40), "f32")])
+def test_captured_run_after_a_run_of_another_kernel(ctx, oracle, name, shape, dtype, first):
+    """Whichever persistent kernel ran first (a traced run's, a plan's), a later run by default needs no allocation and
+    can be captured in a graph."""
+    from paper_2204_02064_gb300 import api
+    c = Case(ctx, name, shape, dtype)
+    if first == "trace":
+        c.st.set_trace(2)
+        c.st.run(4)
+        c.st.set_trace(0)
+    else:
+        c.st.set_plan(kernel=api.KERNEL_STREAMING, tiles=(0, 0, 0))
+        c.st.run(4)
+        c.st.reset_plan()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        c.st.run(8)            # an even number of exchanges or sweeps: every replay starts where the last ended
+    graph.replay()
+    torch.cuda.synchronize()
+    c.check(oracle, 12)
+    c.st.close()
