@@ -377,7 +377,7 @@ perks_status make_tile_plan(perks_stencil *st, Plan &pl) {
 // its warps' row-stages, the chip streams the field in and out, and a sweep
 // adds the grid barrier.  Measured against all runs from 8 to 256 at sides of
 // 256 to 4096, the plan it picks is within 10 % of the fastest.
-perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts, int want_nch) {
+perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts = 0, int want_x = 0, int want_nch = 0) {
     perks_context *ctx = st->ctx;
     const int dt = st->desc.dtype, X = st->X, Z = st->Z, SM = ctx->sm_count;
     double best = 1e300;
@@ -389,6 +389,7 @@ perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts, int want_
             const ShapeInfo &sh = shape_by_id(st->shape_id);
             const int outw = (32 - 2 * e.hl) * e.v;
             const int nsx = ceil_div(X, outw);
+            if (want_x > 0 && want_x != nsx) continue;
             const double points = (double)e.v * sh.npts, R = sh.radius;
             const double stage = dt == PERKS_F64 ? 64.0 * points : 0.75 * points + 4.0 * R + (dt == PERKS_BF16 ? 28 : 20);
             // bytes per cycle the chip streams: from L2 while both fields fit there, else from HBM
@@ -416,7 +417,9 @@ perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts, int want_
             }
         }
     if (!bp.sk)
-        return fail(ctx, PERKS_ERR_UNSUPPORTED, "column-strip kernel: 2-D stencils 2d5pt, 2ds9pt, 2d9pt, 2d25pt only");
+        return fail(ctx, PERKS_ERR_UNSUPPORTED,
+                    "column-strip kernel: 2-D stencils 2d5pt, 2ds9pt, 2d9pt, 2d25pt only, with the steps per sweep and "
+                    "strips across x it is compiled for");
     // halo cells: the overlap each item reads beyond its own cells, per step
     bp.halo_cells = ((long long)bp.ntx * bp.ntz * 32 * bp.sk->v * (2LL * bp.sk->ts * shape_by_id(st->shape_id).radius) +
                      (long long)bp.ntx * 2 * bp.sk->hl * bp.sk->v * Z) / bp.sk->ts;
@@ -429,7 +432,7 @@ perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts, int want_
 // cells' FP64 instructions at 16 cycles a warp (or their issue slots at 4 a
 // cycle), at least the latency of a pass and a block barrier; an exchange some
 // 4000 cycles.
-perks_status make_patch_plan(perks_stencil *st, Plan &pl, int want_k, int want_x, int want_z) {
+perks_status make_patch_plan(perks_stencil *st, Plan &pl, int want_k = 0, int want_x = 0, int want_z = 0) {
     perks_context *ctx = st->ctx;
     const int dt = st->desc.dtype, X = st->X, Z = st->Z, SM = ctx->sm_count;
     const int es = dt == PERKS_F64 ? 8 : 4;  // the buffers hold the accumulator type
@@ -487,8 +490,9 @@ perks_status make_patch_plan(perks_stencil *st, Plan &pl, int want_k, int want_x
 // not; the wider row on a tie), and two blocks per SM, or one per plane where
 // there are fewer planes: parts of columns walked in step where they use 90 %
 // of those blocks and the step is not bound by the FP64 pipe, else equal
-// shares.
-perks_status make_slab_plan(perks_stencil *st, Plan &pl) {
+// shares (ntz = 1).  A plan may ask for the columns another number of lanes
+// per row gives, and for another number of parts.
+perks_status make_slab_plan(perks_stencil *st, Plan &pl, int want_x = 0, int want_y = 0, int want_z = 0) {
     perks_context *ctx = st->ctx;
     const int dt = st->desc.dtype, X = st->X, Y = st->Y, Z = st->Z;
     Plan bp;
@@ -500,6 +504,7 @@ perks_status make_slab_plan(perks_stencil *st, Plan &pl) {
             for (int lg = 5; lg >= 3; --lg) {
                 const int rows = (kSlabThreads >> lg) * e.ry;
                 const int nsx = ceil_div(X, e.v << lg), nsy = ceil_div(Y, rows);
+                if ((want_x > 0 && nsx != want_x) || (want_y > 0 && nsy != want_y)) continue;
                 if ((long long)nsx * nsy >= fewest) continue;
                 fewest = (long long)nsx * nsy;
                 bp.lk = &e;
@@ -509,6 +514,7 @@ perks_status make_slab_plan(perks_stencil *st, Plan &pl) {
                 bp.PW = (e.v << lg) + 2 * e.v;
                 bp.PH = rows + 2 * R;
             }
+            if (bp.lk != &e) continue;  // no number of lanes gives the columns asked for
             bp.plane = bp.PW * bp.PH;
             bp.smem = (long long)e.slots * bp.plane * st->es;
             const long long planes = fewest * Z, most = 2LL * ctx->sm_count;
@@ -516,13 +522,24 @@ perks_status make_slab_plan(perks_stencil *st, Plan &pl) {
             bp.balanced = dt == PERKS_F64 || bp.ntz == 0 || fewest * bp.ntz * 10 < std::min(planes, most) * 9;
             bp.blocks = bp.balanced ? (int)std::min(planes, most) : (int)fewest * bp.ntz;
             if (bp.balanced) bp.ntz = 1;
+            if (want_z > 0 && want_z != bp.ntz) {
+                if (want_z > Z || fewest * want_z > most) {
+                    bp.lk = nullptr;
+                    continue;
+                }
+                bp.balanced = false;
+                bp.ntz = want_z;
+                bp.blocks = (int)fewest * want_z;
+            }
             // halo cells read per step: the rows and columns around every column's planes, and the planes
             // above and below each share
             bp.halo_cells = planes * ((long long)bp.plane - (long long)bp.txmax * bp.tymax) +
                             (long long)bp.blocks * 2 * R * bp.plane;
         }
     if (!bp.lk)
-        return fail(ctx, PERKS_ERR_UNSUPPORTED, "slab-streaming kernel: 3-D stencils 3d7pt, 3d13pt, 3d27pt, poisson only");
+        return fail(ctx, PERKS_ERR_UNSUPPORTED,
+                    "slab-streaming kernel: 3-D stencils 3d7pt, 3d13pt, 3d27pt, poisson only, in columns of 8, 16 or 32 "
+                    "lanes per row cut into parts for two blocks per SM at most");
     int budget = 0;
     const perks_status rc = smem_optin(ctx, (const void *)bp.lk->fn, &budget);
     if (rc) return rc;
@@ -818,15 +835,17 @@ perks_status search_plan(perks_stencil *st, Plan &pl, bool per_step) {
     perks_status rc = make_base_plan(st, pl, false);
     st->has_plan = asked;
     if (rc) return rc;
-    if (kind == PERKS_KERNEL_STRIP) return make_strip_plan(st, pl, st->plan.reserved[1], st->plan.tiles_z);
-    if (kind == PERKS_KERNEL_PATCH)
-        return make_patch_plan(st, pl, st->plan.reserved[1], st->plan.tiles_x, st->plan.tiles_z);
-    if (kind == PERKS_KERNEL_SLAB) return make_slab_plan(st, pl);
+    const perks_stencil_plan &want = st->plan;
+    if (asked && st->desc.ndim == 2 && want.tiles_y > 1)
+        return fail(st->ctx, PERKS_ERR_UNSUPPORTED, "a 2-D domain has one tile along the middle axis, not %d", want.tiles_y);
+    if (kind == PERKS_KERNEL_STRIP) return make_strip_plan(st, pl, want.reserved[1], want.tiles_x, want.tiles_z);
+    if (kind == PERKS_KERNEL_PATCH) return make_patch_plan(st, pl, want.reserved[1], want.tiles_x, want.tiles_z);
+    if (kind == PERKS_KERNEL_SLAB) return make_slab_plan(st, pl, want.tiles_x, want.tiles_y, want.tiles_z);
     const std::string saved_msg = st->ctx->last_error;
     Plan sp, qp;
     if (st->desc.ndim == 2) {
-        const bool strip = make_strip_plan(st, sp, 0, 0) == PERKS_OK;
-        const bool patch = make_patch_plan(st, qp, 0, 0, 0) == PERKS_OK;
+        const bool strip = make_strip_plan(st, sp) == PERKS_OK;
+        const bool patch = make_patch_plan(st, qp) == PERKS_OK;
         if (patch && (!strip || patch_beats(st))) pl = qp;
         else if (strip) pl = sp;
     } else {

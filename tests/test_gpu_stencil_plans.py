@@ -125,3 +125,34 @@ def test_captured_run_after_a_run_of_another_kernel(ctx, oracle, name, shape, dt
     torch.cuda.synchronize()
     c.check(oracle, 12)
     c.st.close()
+
+
+def test_tilings_a_kernel_cannot_take_are_refused(ctx, oracle):
+    """Strips, slabs and patches take the tiles they are asked for or refuse them; the planner's own are taken."""
+    from paper_2204_02064_gb300 import api
+    flat, box = Case(ctx, "2d9pt", (200, 256)), Case(ctx, "3d7pt", (30, 70, 96), "f32")
+    for c, kernel, bad in ((flat, api.KERNEL_STRIP, [(17, 0, 0), (0, 2, 0)]),
+                           (flat, api.KERNEL_PATCH, [(0, 2, 0), (200, 0, 0)]),
+                           (box, api.KERNEL_SLAB, [(17, 0, 0), (0, 17, 0), (2, 2, 0), (0, 0, 31)])):
+        c.st.set_plan(kernel=kernel)
+        d = c.st.describe(4)
+        own = (d["tiles_x"], d["tiles_y"], d["tiles_z"])
+        c.st.set_plan(kernel=kernel, tiles=own)
+        assert c.st.describe(4) == d
+        for tiles in bad:
+            c.st.set_plan(kernel=kernel, tiles=tiles)
+            with pytest.raises(api.PerksError) as ei:
+                c.st.run(1)
+            assert ei.value.name == "UNSUPPORTED"
+    # rows of 32, 16 or 8 lanes, four cells each, two rows per thread: columns of 128 x 16, 64 x 32 or 32 x 64 cells
+    steps = 0
+    for tiles in ((1, 5, 0), (2, 3, 0), (3, 2, 5), (2, 0, 7), (0, 0, 7), (0, 5, 30)):
+        box.st.set_plan(kernel=api.KERNEL_SLAB, tiles=tiles)
+        d = box.st.run(3, stats=True)
+        steps += 3
+        assert d["kernel"] == api.KERNEL_SLAB
+        assert all(want in (0, got) for want, got in zip(tiles, (d["tiles_x"], d["tiles_y"], d["tiles_z"])))
+        assert d["grid_blocks"] <= 2 * ctx.info()["sm_count"]
+    box.check(oracle, steps)
+    flat.st.close()
+    box.st.close()
