@@ -203,9 +203,11 @@ struct Plan {
     TileKernelEntry *tk = nullptr;
     int tx = 0, PP = 0, XGS = 0, groups = 0, chunks = 0, per_plane = 0;
     long long FS = 0;
-    // column-strip kernel (2-D): ntx strips across x, ntz runs of rows
-    StripKEntry *sk = nullptr;
-    double cost = 0.0;         // column strips and patches: modelled SM cycles per step
+    // column-strip kernel (2-D): ntx strips across x, ntz runs of rows; and rk, one step per sweep, for steps left over
+    // from whole sweeps
+    StripKEntry *sk = nullptr, *rk = nullptr;
+    int rest_x = 0, rest_z = 0, rest_blocks = 0;
+    double cost = 0.0, rest_cost = 0.0;  // modelled SM cycles per step
     // patch kernel (2-D): ntx x ntz tiles, shared buffers of PW x PH cells
     PatchEntry *qk = nullptr;
     // slab-streaming kernel (3-D): ntx x nty columns, 2^loglx lanes per row
@@ -377,14 +379,15 @@ perks_status make_tile_plan(perks_stencil *st, Plan &pl) {
 // its warps' row-stages, the chip streams the field in and out, and a sweep
 // adds the grid barrier.  Measured against all runs from 8 to 256 at sides of
 // 256 to 4096, the plan it picks is within 10 % of the fastest.
-perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts = 0, int want_x = 0, int want_nch = 0) {
+perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts = 0, int want_x = 0, int want_nch = 0,
+                             bool rest = false) {
     perks_context *ctx = st->ctx;
     const int dt = st->desc.dtype, X = st->X, Z = st->Z, SM = ctx->sm_count;
     double best = 1e300;
     Plan bp;
     if (st->desc.ndim == 2 && (dt != PERKS_BF16 || X % 8 == 0))
         for (StripKEntry &e : strip_registry()) {
-            if (e.dtype != dt || e.shape != st->shape_id || e.aligned != (X % e.v == 0)) continue;
+            if (e.dtype != dt || e.shape != st->shape_id || e.aligned != (X % e.v == 0) || (e.rest && !rest)) continue;
             if (want_ts > 0 && e.ts != want_ts) continue;
             const ShapeInfo &sh = shape_by_id(st->shape_id);
             const int outw = (32 - 2 * e.hl) * e.v;
@@ -423,6 +426,13 @@ perks_status make_strip_plan(perks_stencil *st, Plan &pl, int want_ts = 0, int w
     // halo cells: the overlap each item reads beyond its own cells, per step
     bp.halo_cells = ((long long)bp.ntx * bp.ntz * 32 * bp.sk->v * (2LL * bp.sk->ts * shape_by_id(st->shape_id).radius) +
                      (long long)bp.ntx * 2 * bp.sk->hl * bp.sk->v * Z) / bp.sk->ts;
+    Plan one;
+    if (bp.sk->ts > 1 && make_strip_plan(st, one, 1, 0, 0, true) == PERKS_OK) {
+        bp.rk = one.sk;
+        bp.rest_x = one.ntx; bp.rest_z = one.ntz;
+        bp.rest_blocks = one.blocks;
+        bp.rest_cost = one.cost;
+    }
     pl = bp;
     return PERKS_OK;
 }
@@ -877,6 +887,21 @@ perks_status make_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
     return PERKS_OK;
 }
 
+// A run of column strips: do the steps left over from whole sweeps run as one
+// sweep each of the one-step kernel?  Otherwise they are a last sweep that
+// passes the levels it does not need through, with the checks of an item's
+// first rows in every one (fp64 half of a whole sweep's time, two steps per
+// sweep 0.75, four 1.35 to 1.55).  The kernel of their own costs a launch, some
+// 5 us = 10000 cycles behind another one.  One step of 2d5pt: fp32 3072^2 20 us
+// by itself, 33 as such a sweep, bf16 15 and 36; three steps: 46 and 36, bf16 38
+// and 40.
+bool strip_rest_alone(const perks_stencil *st, const Plan &pl, long long steps) {
+    const long long over = steps % pl.sk->ts;
+    const double part = st->desc.dtype == PERKS_F64 ? 0.5 : pl.sk->ts == 2 ? 0.75 : 1.25 + 0.1 * (double)over;
+    return over > 0 && pl.rk &&
+           (double)over * pl.rest_cost + (steps > over ? 10000.0 : 0.0) < part * pl.sk->ts * pl.cost;
+}
+
 void fill_stats(const perks_stencil *st, const Plan *pl, long long steps, int variant,
                 perks_run_stats *o) {
     std::memset(o, 0, sizeof(*o));
@@ -912,7 +937,8 @@ void fill_stats(const perks_stencil *st, const Plan *pl, long long steps, int va
         o->planes_per_sync = pl->sk->ts;  // steps per sweep
         o->halo_cells_per_step = pl->halo_cells;
         // the field is read and written once per sweep of ts steps
-        const double sweeps = (double)((steps + pl->sk->ts - 1) / pl->sk->ts);
+        const double sweeps = strip_rest_alone(st, *pl, steps) ? (double)(steps / pl->sk->ts + steps % pl->sk->ts)
+                                                               : (double)((steps + pl->sk->ts - 1) / pl->sk->ts);
         o->algorithmic_bytes = S * (2.0 * sweeps * (double)st->cells + (double)steps * pl->halo_cells);
     } else if (variant == PERKS_PERSISTENT && pl && pl->resident) {
         o->kernel = PERKS_KERNEL_RESIDENT;
@@ -1019,32 +1045,43 @@ perks_status run_resident(perks_stencil *st, long long steps, cudaStream_t s, co
     return PERKS_OK;
 }
 
-// One cooperative launch of the column-strip kernel, sk->ts steps per sweep.
+// The column-strip kernel: sk->ts steps per sweep, all sweeps in one
+// cooperative launch, and the steps left over (fewer than ts) as a last sweep
+// or in a launch of their own (strip_rest_alone).
 perks_status run_strip(perks_stencil *st, long long steps, cudaStream_t s, const Plan &pl) {
     perks_context *ctx = st->ctx;
     const perks_status rc = ensure_sync(st);
     if (rc) return rc;
+    const long long over = steps % pl.sk->ts;
+    const bool own = strip_rest_alone(st, pl, steps);
     StripKArgs a;
     std::memset(&a, 0, sizeof(a));
     a.X = st->X; a.Z = st->Z;
-    a.nsx = pl.ntx; a.nch = pl.ntz;
     a.sms = ctx->sm_count;
-    a.steps = steps;
     a.boundary = st->desc.boundary;
     a.boundary_f = (float)st->desc.boundary;
     for (int i = 0; i < 25; ++i) { a.w[i] = st->kw[i]; a.wf[i] = (float)st->kw[i]; }
-    a.field[0] = st->field[st->cur];
-    a.field[1] = st->field[st->cur ^ 1];
     a.bar = st->bar;
     a.err = st->err;
     a.timeout_ns = ctx->timeout_ns;
-    PERKS_CUDA(ctx, cudaMemsetAsync(st->bar, 0, sizeof(unsigned long long), s));
     PERKS_CUDA(ctx, cudaMemsetAsync(st->err, 0, sizeof(DevError), s));
-    void *args[] = {&a};
-    PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)pl.sk->fn, dim3(pl.blocks), dim3(pl.sk->nt), args,
-                                                0, s));
-    if (((steps + pl.sk->ts - 1) / pl.sk->ts) & 1) st->cur ^= 1;
-    return PERKS_OK;
+    auto launch = [&](const StripKEntry &e, int nsx, int nch, int blocks, long long n) -> perks_status {
+        a.nsx = nsx; a.nch = nch;
+        a.steps = n;
+        a.field[0] = st->field[st->cur];
+        a.field[1] = st->field[st->cur ^ 1];
+        PERKS_CUDA(ctx, cudaMemsetAsync(st->bar, 0, sizeof(unsigned long long), s));
+        void *args[] = {&a};
+        PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)e.fn, dim3(blocks), dim3(e.nt), args, 0, s));
+        if (((n + e.ts - 1) / e.ts) & 1) st->cur ^= 1;
+        return PERKS_OK;
+    };
+    if (!own) return launch(*pl.sk, pl.ntx, pl.ntz, pl.blocks, steps);
+    if (steps > over) {
+        const perks_status r = launch(*pl.sk, pl.ntx, pl.ntz, pl.blocks, steps - over);
+        if (r) return r;
+    }
+    return launch(*pl.rk, pl.rest_x, pl.rest_z, pl.rest_blocks, over);
 }
 
 // One cooperative launch of the patch kernel.

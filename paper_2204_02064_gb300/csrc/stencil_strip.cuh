@@ -57,6 +57,7 @@ struct StripKEntry {
     int nt;               // threads per block, two blocks per SM
     int hl;               // overlap lanes on each side
     bool aligned;         // rows start on V-cell boundaries (X % V == 0)
+    bool rest;            // for the steps left over from whole sweeps only
     StripKFn fn;
 };
 
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(NT, 2) perks_strip_kernel(const __grid_constan
     }
 }
 
-template <typename T, class SH, int TS, bool AL, int NT> StripKEntry strip_entry(int dtype, int shape) {
+template <typename T, class SH, int TS, bool AL, int NT> StripKEntry strip_entry(int dtype, int shape, bool rest) {
     StripKEntry e;
     e.dtype = dtype;
     e.shape = shape;
@@ -308,13 +309,16 @@ template <typename T, class SH, int TS, bool AL, int NT> StripKEntry strip_entry
     e.hl = strip_hl<T, SH, TS>();
     e.aligned = AL;
     e.nt = NT;
+    e.rest = rest;
     e.fn = perks_strip_kernel<T, SH, TS, AL, NT>;
     return e;
 }
 
-template <typename T, class SH, int TS, int NT = 256> void strip_entries(std::vector<StripKEntry> &out, int dtype, int shape) {
-    out.push_back(strip_entry<T, SH, TS, true, NT>(dtype, shape));
-    if constexpr (!std::is_same<T, __nv_bfloat16>::value) out.push_back(strip_entry<T, SH, TS, false, NT>(dtype, shape));
+template <typename T, class SH, int TS, int NT = 256>
+void strip_entries(std::vector<StripKEntry> &out, int dtype, int shape, bool rest = false) {
+    out.push_back(strip_entry<T, SH, TS, true, NT>(dtype, shape, rest));
+    if constexpr (!std::is_same<T, __nv_bfloat16>::value)
+        out.push_back(strip_entry<T, SH, TS, false, NT>(dtype, shape, rest));
 }
 
 }  // namespace perks

@@ -10,6 +10,11 @@ void register_strip_f32(std::vector<StripKEntry> &out) {
     strip_entries<float, S2ds9, 2>(out, PERKS_F32, SH_2DS9);
     strip_entries<float, S2ds9, 4, 192>(out, PERKS_F32, SH_2DS9);
     strip_entries<float, S2d25, 2, 192>(out, PERKS_F32, SH_2D25);
+    // steps left over from whole sweeps
+    strip_entries<float, S2d5, 1>(out, PERKS_F32, SH_2D5, true);
+    strip_entries<float, S2d9, 1>(out, PERKS_F32, SH_2D9, true);
+    strip_entries<float, S2ds9, 1>(out, PERKS_F32, SH_2DS9, true);
+    strip_entries<float, S2d25, 1, 192>(out, PERKS_F32, SH_2D25, true);
 }
 
 }  // namespace perks

@@ -94,3 +94,43 @@ def test_strip_barrier_timeout_and_trace(ctx, oracle):
     out = torch.empty_like(src)
     st.get_field(out)
     assert rel_err(out.cpu().numpy(), oracle.stencil_run(f, offs, w, 6)) <= 1e-12
+
+
+#: Steps per sweep the strips are compiled for.
+COMPILED = {"f64": {"2d5pt": (1, 2), "2d9pt": (1, 2), "2ds9pt": (1, 2), "2d25pt": (1,)},
+            "f32": {"2d5pt": (4,), "2d9pt": (4,), "2ds9pt": (2, 4), "2d25pt": (2,)}}
+COMPILED["bf16"] = COMPILED["f32"]
+
+
+@pytest.mark.parametrize("name", ["2d5pt", "2ds9pt", "2d9pt", "2d25pt"])
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("nx", [120, 257])
+@pytest.mark.parametrize("ts", [1, 2, 4])
+def test_every_number_of_steps_per_sweep(ctx, oracle, name, dtype, nx, ts):
+    """Each compiled number of steps per sweep, for runs of one to nine steps (whole sweeps, and every remainder), is
+    what runs; the others are refused."""
+    from paper_2204_02064_gb300 import api
+    shape = (301, nx // 8 * 8 if dtype == "bf16" else nx)
+    offs, w = inputs.shape_offsets(name), inputs.workload_weights(name, seed=5)
+    st = api.Stencil(ctx, shape, offs, w, dtype=dtype, boundary=0.375)
+    src = torch.from_numpy(inputs.stencil_field(shape, 49)).to(TT[dtype]).cuda()
+    st.set_plan(kernel=api.KERNEL_STRIP, planes_per_barrier=ts, tiles=(0, 0, 7))
+    if ts not in COMPILED[dtype][name]:
+        with pytest.raises(api.PerksError) as ei:
+            st.run(1)
+        assert ei.value.name == "UNSUPPORTED"
+        return
+    for steps in range(1, 10):
+        st.set_field(src)
+        stats = st.run(steps, stats=True)
+        assert (stats["kernel"], stats["planes_per_sync"], stats["tiles_z"]) == (api.KERNEL_STRIP, ts, 7)
+        out = torch.empty_like(src)
+        st.get_field(out)
+        torch.cuda.synchronize()
+        if dtype == "f64":
+            ref = oracle.stencil_run(src.cpu().numpy(), offs, w, steps, boundary=0.375)
+            assert rel_err(out.cpu().numpy(), ref) <= 1e-12
+        else:
+            ref = oracle.stencil_run_lowp(src.float().cpu().numpy(), offs, w, steps, dtype, boundary=0.375)
+            assert np.array_equal(out.float().cpu().numpy(), ref)
+    st.close()
