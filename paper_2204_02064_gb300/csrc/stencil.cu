@@ -562,7 +562,9 @@ perks_status make_slab_plan(perks_stencil *st, Plan &pl, int want_x = 0, int wan
     return PERKS_OK;
 }
 
-perks_status make_base_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
+// cache_free = false leaves out the search for the cache-free plan that a
+// domain without a plan takes when the caches do not hold it.
+perks_status make_base_plan(perks_stencil *st, Plan &pl, bool per_step = false, bool cache_free = true) {
     perks_context *ctx = st->ctx;
     // The resident-tile kernel when it is asked for, or by default (no plan)
     // when every tile of the domain fits in shared memory.
@@ -730,7 +732,7 @@ perks_status make_base_plan(perks_stencil *st, Plan &pl, bool per_step = false) 
     }
     bp.cached_cells = cached;
     bp.halo_cells = halo;
-    if (!st->has_plan && !per_step && cached < st->cells) {
+    if (!st->has_plan && !per_step && cache_free && cached < st->cells) {
         // Default plan when the caches cannot hold the whole domain: the
         // cache-free body for all steps in one launch.  Measured on GB300,
         // caching a part of a domain (3-D 384^3 in fp64/fp32/bf16, 2-D 4096^2)
@@ -807,7 +809,7 @@ bool slab_beats(const perks_stencil *st, const Plan &base, const Plan &slab) {
 // with 256 threads (two blocks per SM, one's FP64 work under the other's
 // barriers) in balanced shares: 384^3 838 -> 746 us per step, 256^3 265 ->
 // 228, 192^3 108 -> 101.
-void choose_f64_3d7(perks_stencil *st, Plan &pl) {
+bool choose_f64_3d7(perks_stencil *st, Plan &pl) {
     const std::string saved_msg = st->ctx->last_error;
     const perks_stencil_plan saved = st->plan;
     Plan alt;
@@ -816,10 +818,12 @@ void choose_f64_3d7(perks_stencil *st, Plan &pl) {
     st->plan.reserved[3] = 256;
     st->plan.balanced = 1;
     st->has_plan = true;
-    if (make_base_plan(st, alt, false) == PERKS_OK) pl = alt;
+    const bool ok = make_base_plan(st, alt, false) == PERKS_OK;
+    if (ok) pl = alt;
     st->has_plan = false;
     st->plan = saved;
     st->ctx->last_error = saved_msg;
+    return ok;
 }
 
 // The plan a run uses.  A domain without a plan takes, where the other kernels
@@ -841,8 +845,11 @@ perks_status search_plan(perks_stencil *st, Plan &pl, bool per_step) {
         return rt;
     }
     if (!asked && !open) return make_base_plan(st, pl, per_step);
+    // (a first run waits for this: the plans that another one replaces are not searched for)
+    const bool f64_3d7 = open && st->shape_id == SH_3D7 && st->desc.dtype == PERKS_F64 && st->X % 2 == 0 &&
+                         st->cells >= (1 << 22);
     st->has_plan = false;
-    perks_status rc = make_base_plan(st, pl, false);
+    perks_status rc = make_base_plan(st, pl, false, !f64_3d7 && !asked);
     st->has_plan = asked;
     if (rc) return rc;
     const perks_stencil_plan &want = st->plan;
@@ -852,19 +859,19 @@ perks_status search_plan(perks_stencil *st, Plan &pl, bool per_step) {
     if (kind == PERKS_KERNEL_PATCH) return make_patch_plan(st, pl, want.reserved[1], want.tiles_x, want.tiles_z);
     if (kind == PERKS_KERNEL_SLAB) return make_slab_plan(st, pl, want.tiles_x, want.tiles_y, want.tiles_z);
     const std::string saved_msg = st->ctx->last_error;
-    Plan sp, qp;
+    Plan alt;
     if (st->desc.ndim == 2) {
-        const bool strip = make_strip_plan(st, sp) == PERKS_OK;
-        const bool patch = make_patch_plan(st, qp) == PERKS_OK;
-        if (patch && (!strip || patch_beats(st))) pl = qp;
-        else if (strip) pl = sp;
-    } else {
-        if (make_slab_plan(st, sp) == PERKS_OK && slab_beats(st, pl, sp)) pl = sp;
-        else if (st->shape_id == SH_3D7 && st->desc.dtype == PERKS_F64 && st->X % 2 == 0 && st->cells >= (1 << 22))
-            choose_f64_3d7(st, pl);
+        const bool patch = patch_beats(st);
+        if (patch && make_patch_plan(st, alt) == PERKS_OK) pl = alt;
+        else if (make_strip_plan(st, alt) == PERKS_OK) pl = alt;
+        else if (!patch && make_patch_plan(st, alt) == PERKS_OK) pl = alt;
+    } else if (make_slab_plan(st, alt) == PERKS_OK && slab_beats(st, pl, alt)) {
+        pl = alt;
+    } else if (f64_3d7 && !choose_f64_3d7(st, pl)) {
+        rc = make_base_plan(st, pl, false);
     }
     st->ctx->last_error = saved_msg;
-    return PERKS_OK;
+    return rc;
 }
 
 perks_status make_plan(perks_stencil *st, Plan &pl, bool per_step = false) {
