@@ -622,15 +622,15 @@ struct perks_poisson {
     int *gprob = nullptr;
     double *gpart = nullptr;
     double *slots = nullptr;  // [2 x SMs][3]: every group's rounds of exchange_sum
-    double *halo = nullptr;   // [2 x SMs][2][nx]
+    double *halo = nullptr;   // [blocks of the automatic groups][2][nx]; none where a problem is one block's
+    void *small = nullptr;    // the allocation of all of these but halo, and of the counters and results above
     DevError *err = nullptr;
     int max_groups = 0;
 };
 
 namespace {
 void free_poisson(perks_poisson *P) {
-    void *ptrs[] = {P->fx, P->fy, P->dg, P->b, P->x, P->r, P->p, P->q, P->queue, P->iters, P->status, P->true_rel,
-                    P->gbar, P->gprob, P->gpart, P->slots, P->halo, P->err};
+    void *ptrs[] = {P->fx, P->fy, P->dg, P->b, P->x, P->r, P->p, P->q, P->small, P->halo};
     for (void *v : ptrs) if (v) cudaFree(v);
 }
 
@@ -724,20 +724,43 @@ extern "C" perks_status perks_poisson_create(perks_context *ctx, int32_t nx, int
     for (void **bp : bufs) if (e == cudaSuccess) e = cudaMalloc(bp, vb);
     if (e == cudaSuccess) e = cudaMalloc(&P->fx, fxb);
     if (e == cudaSuccess) e = cudaMalloc(&P->fy, fyb);
-    if (e == cudaSuccess) e = cudaMalloc(&P->queue, sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&P->iters, sizeof(int) * nprob);
-    if (e == cudaSuccess) e = cudaMalloc(&P->status, sizeof(int) * nprob);
-    if (e == cudaSuccess) e = cudaMalloc(&P->true_rel, sizeof(double) * nprob);
-    P->max_groups = 2 * ctx->sm_count;  // at most two blocks per SM
-    if (e == cudaSuccess) e = cudaMalloc(&P->gbar, sizeof(unsigned long long) * P->max_groups);
-    if (e == cudaSuccess) e = cudaMalloc(&P->gprob, sizeof(int) * P->max_groups);
-    if (e == cudaSuccess) e = cudaMalloc(&P->gpart, sizeof(double) * 2 * kPoiMaxGroup * P->max_groups);
-    if (e == cudaSuccess) e = cudaMalloc(&P->slots, sizeof(double) * 3 * P->max_groups);
-    if (e == cudaSuccess) e = cudaMalloc(&P->halo, sizeof(double) * 2 * nx * P->max_groups);
-    if (e == cudaSuccess) e = cudaMalloc(&P->err, sizeof(DevError));
     if (e == cudaSuccess && !on_device) {
         e = cudaMalloc(&kd, vb);
         if (e == cudaSuccess) e = cudaMemcpy(kd, k, vb, cudaMemcpyHostToDevice);
+    }
+    // One allocation for counters, results and sums
+    P->max_groups = 2 * ctx->sm_count;  // at most two blocks per SM
+    const size_t mg = P->max_groups, np = nprob;
+    size_t total = 0;
+    auto part = [&](size_t bytes) {
+        const size_t at = total;
+        total += (bytes + 511) & ~size_t(511);
+        return at;
+    };
+    const size_t queue = part(sizeof(int)), iters = part(sizeof(int) * np), status = part(sizeof(int) * np),
+                 rel = part(sizeof(double) * np), gbar = part(sizeof(unsigned long long) * mg),
+                 gprob = part(sizeof(int) * mg), gpart = part(sizeof(double) * 2 * kPoiMaxGroup * mg),
+                 slots = part(sizeof(double) * 3 * mg), err = part(sizeof(DevError));
+    if (e == cudaSuccess) e = cudaMalloc(&P->small, total);
+    if (e == cudaSuccess) {
+        char *at = static_cast<char *>(P->small);
+        P->queue = reinterpret_cast<int *>(at + queue);
+        P->iters = reinterpret_cast<int *>(at + iters);
+        P->status = reinterpret_cast<int *>(at + status);
+        P->true_rel = reinterpret_cast<double *>(at + rel);
+        P->gbar = reinterpret_cast<unsigned long long *>(at + gbar);
+        P->gprob = reinterpret_cast<int *>(at + gprob);
+        P->gpart = reinterpret_cast<double *>(at + gpart);
+        P->slots = reinterpret_cast<double *>(at + slots);
+        P->err = reinterpret_cast<DevError *>(at + err);
+        // halo rows of the blocks that run_group puts to work (two per block: at most two vectors' worth where every block
+        // has a row; two rows for each of 2 x SMs blocks took 10 GB for one problem of 1 x 2^21).  A batch that leaves no
+        // room for them is solved by the kernel without them.
+        const int C = P->n < (1LL << 30) ? run_group(P) : 1;
+        if (C > 1 && cudaMalloc(&P->halo, sizeof(double) * 2 * nx * std::min(nprob, P->max_groups / C) * C) != cudaSuccess) {
+            P->halo = nullptr;
+            (void)cudaGetLastError();
+        }
     }
     if (e != cudaSuccess) {
         if (kd) cudaFree(kd);
@@ -802,8 +825,9 @@ extern "C" perks_status perks_poisson_solve(perks_poisson *P, const double *b, d
     a.max_iter = max_iter;
     a.max_restarts = 8;
     // group size and rows per pass by default: the run kernel
-    const bool run = P->group == 0 && P->rows_per_pass == 1 && P->n < (1LL << 30);
-    const int C = run ? run_group(P) : effective_group(P);
+    const int own_group = run_group(P);
+    const bool run = P->group == 0 && P->rows_per_pass == 1 && P->n < (1LL << 30) && (own_group == 1 || P->halo);
+    const int C = run ? own_group : effective_group(P);
     const bool grouped = C > 1;
     const void *kern;
     size_t smem = 0;

@@ -235,3 +235,27 @@ def test_automatic_groups_match_oracle(ctx, oracle, nprob, ny, nx):
         ref = oracle.cg(rp, c, val, f[i].ravel(), rtol=1e-8, max_iter=20000)
         assert np.linalg.norm(xs[i].ravel() - ref["x"]) <= 1e-6 * np.linalg.norm(ref["x"])
     P.close()
+
+
+@pytest.mark.parametrize("nprob,ny,nx", [(1, 1, 1 << 21), (1, 3, 1 << 20), (300, 1, 20000), (2, 70, 3000)])
+def test_memory_is_a_few_vectors(ctx, nprob, ny, nx):
+    """An object holds its eight vectors (two of face coefficients) and at most two more for the rows its blocks
+    exchange, however long a row is (64 MB for the rest); and its solver works."""
+    from paper_2204_02064_gb300 import api
+    k = torch.from_numpy(_k(nprob, ny, nx, 23)).cuda()
+    f = torch.ones_like(k)
+    torch.cuda.synchronize()
+    api.Poisson(ctx, k[:, :, :8].contiguous()).close()    # the kernels are loaded
+    free = torch.cuda.mem_get_info()[0]
+    P = api.Poisson(ctx, k)
+    used = free - torch.cuda.mem_get_info()[0]
+    assert used <= 8 * nprob * (10 * ny * nx + ny + nx) + (64 << 20)
+    # five iterations against the kernel a set group runs: ten sums of up to 3.1 M terms, each within 3.1 M x 2^-53
+    xs = []
+    for group in (0, 1):
+        P.set_group(group)
+        x = torch.zeros_like(k)
+        P.solve(f, x, rtol=1e-30, max_iter=5, stats=False)
+        xs.append(x)
+    assert float((xs[0] - xs[1]).norm()) <= 1e-8 * float(xs[1].norm()) and float(xs[1].norm()) > 0.0
+    P.close()
