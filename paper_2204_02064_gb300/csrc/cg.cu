@@ -344,7 +344,7 @@ void free_op(perks_op *op) {
 // nonzero (8 in fp32) and 4 per row.
 size_t slice_smem(const perks_op *op, int mode) {
     const size_t nnz = ((size_t)op->max_nnz2 + 3) & ~size_t(3);
-    return kCgRowvecSmem + ((nnz * (mode == CGK_FP32_IR ? 4 : 8) + 15) & ~size_t(15)) + nnz * 4 +
+    return kCgShortSmem + ((nnz * (mode == CGK_FP32_IR ? 4 : 8) + 15) & ~size_t(15)) + nnz * 4 +
            ((size_t)op->max_rows2 + 4) * 4;
 }
 
@@ -471,7 +471,7 @@ perks_status launch_persistent(perks_op *op, const CgArgs &a, cudaStream_t s) {
     // keep kind 0, whose L1 is not cut by shared memory.
     if (op->spmv_kind == PERKS_SPMV_ROWVEC && a.vcache == 0 && (a.slice || a.short_rows))
         PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)perks_cg_kernel<3>, dim3(op->G2), dim3(kCgThreads),
-                                                    args, a.slice ? slice_smem(op, a.mode) : kCgRowvecSmem, s));
+                                                    args, a.slice ? slice_smem(op, a.mode) : kCgShortSmem, s));
     else if (op->spmv_kind == PERKS_SPMV_ROWVEC)
         PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)perks_cg_kernel<0>, dim3(op->G2),
                                                     dim3(kCgThreads), args, rowvec_smem(op, a.vcache), s));

@@ -228,6 +228,30 @@ template <int NT> __device__ __forceinline__ double reduce4(double *s, int n) {
     return threadIdx.x == 0 ? (part[0] + part[1]) + (part[2] + part[3]) : 0.0;
 }
 
+// The same sum of the threads' v, added in the same order, in 1 KB of scratch
+// (128 doubles) for five more block barriers: for kernels that keep their
+// data in shared memory up to its limit.
+constexpr size_t kSmallReduceBytes = 128 * sizeof(double);
+
+template <int NT> __device__ __forceinline__ double reduce4_small(double v, double *s) {
+    static_assert(NT == 512, "four quarters of 128 values");
+    const int quarter = threadIdx.x >> 7, i = threadIdx.x & 127;
+    __syncthreads();  // the last sum's result has been read
+    if (quarter == 1) s[i] = v;
+    __syncthreads();
+    if (quarter == 0) v += s[i];
+    __syncthreads();
+    if (quarter == 3) s[i] = v;
+    __syncthreads();
+    if (quarter == 2) s[i] += v;
+    __syncthreads();
+    if (quarter == 0) v = warp_sum(v + s[i]);
+    __syncthreads();
+    if (quarter == 0 && (i & 31) == 0) s[i >> 5] = v;
+    __syncthreads();
+    return threadIdx.x == 0 ? (s[0] + s[1]) + (s[2] + s[3]) : 0.0;
+}
+
 // What every thread of a block needs from a sum: the sum, a ratio formed from
 // it and a decision.  Thread 0 forms them and hands them out: an fp64 division
 // is some 15 operations of the FP64 pipe, and 32 warps forming the same one
@@ -237,24 +261,30 @@ struct SumResult {
     int flag;
 };
 
-// Sum of s[0..n) with post(total, ratio, flag) applied by thread 0, in every
-// thread.  s[] is complete (a block barrier lies behind its last store).
-template <int NT, class POST>
-__device__ __forceinline__ void finish_sum(double *s, int n, SumResult &out, POST &&post) {
-    const double total = reduce4<NT>(s, n);
-    int *flag = reinterpret_cast<int *>(s + NT + 10);
+// `total` of thread 0, with post(total, ratio, flag) applied by it, in every
+// thread, by way of at[0..2].
+template <class POST>
+__device__ __forceinline__ void hand_out(double total, double *at, SumResult &out, POST &&post) {
+    int *flag = reinterpret_cast<int *>(at + 2);
     if (threadIdx.x == 0) {
         double ratio = 0.0;
         int f = 0;
         post(total, ratio, f);
-        s[NT + 8] = total;
-        s[NT + 9] = ratio;
+        at[0] = total;
+        at[1] = ratio;
         *flag = f;
     }
     __syncthreads();
-    out.total = s[NT + 8];
-    out.ratio = s[NT + 9];
+    out.total = at[0];
+    out.ratio = at[1];
     out.flag = *flag;
+}
+
+// Sum of s[0..n) with post(total, ratio, flag) applied by thread 0, in every
+// thread.  s[] is complete (a block barrier lies behind its last store).
+template <int NT, class POST>
+__device__ __forceinline__ void finish_sum(double *s, int n, SumResult &out, POST &&post) {
+    hand_out(reduce4<NT>(s, n), s + NT + 8, out, post);
 }
 
 // Sum of v over the threads of one block.
@@ -270,22 +300,32 @@ __device__ __forceinline__ void block_sum4(double v, double *s, SumResult &out, 
 // of them in the same order.  (Spinning on the slots themselves saves a trip
 // for a few blocks -- exchange_sum -- but with 304 blocks the polls of 304
 // words by 304 blocks queue at the L2: 9.5 us a sum.)
-template <int NT, class POST>
+// SMALL: s holds kSmallReduceBytes (G at most NT), otherwise reduce_scratch.
+template <int NT, bool SMALL, class POST>
 __device__ __forceinline__ bool grid_sum4(double *slots, int G, unsigned long long *bar, unsigned long long &epoch,
                                           DevError *err, long long timeout_ns, unsigned &round, double v, double *s,
                                           SumResult &out, POST &&post) {
     double *row = slots + (size_t)(round & 1) * G;
     ++round;
-    s[threadIdx.x] = v;
-    __syncthreads();
-    const double sum = reduce4<NT>(s, NT);
+    double sum;
+    if constexpr (SMALL) {
+        sum = reduce4_small<NT>(v, s);
+    } else {
+        s[threadIdx.x] = v;
+        __syncthreads();
+        sum = reduce4<NT>(s, NT);
+    }
     if (threadIdx.x == 0) __stcg(row + blockIdx.x, sum);
     if (!grid_barrier(bar, G, epoch, err, timeout_ns)) return false;
     double mine = 0.0;
     for (int i = threadIdx.x; i < G; i += NT) mine = i < NT ? __ldcg(row + i) : mine + __ldcg(row + i);
-    s[threadIdx.x] = mine;
-    __syncthreads();
-    finish_sum<NT>(s, G < NT ? G : NT, out, post);
+    if constexpr (SMALL) {
+        hand_out(reduce4_small<NT>(mine, s), s + 8, out, post);
+    } else {
+        s[threadIdx.x] = mine;
+        __syncthreads();
+        finish_sum<NT>(s, G < NT ? G : NT, out, post);
+    }
     return true;
 }
 

@@ -390,3 +390,27 @@ def test_vector_cache_levels_identical_short_rows(ctx, mode):
         out.append(x)
     assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
     op.close()
+
+
+@pytest.mark.parametrize("level", [1, 2])
+@pytest.mark.parametrize("mode", [0, 1], ids=["fp64", "fp32_ir"])
+def test_vector_cache_at_the_limit_of_shared_memory(ctx, level, mode):
+    """As many rows as two blocks per SM hold x, r and q of beside 1 KB of scratch (24 bytes a row, half an SM less the
+    1 KB a block reserves): the cache is on, and gives the bits of a solve without it."""
+    from paper_2204_02064_gb300 import api
+    sms = ctx.info()["sm_count"]
+    per_sm = torch.cuda.get_device_properties(0).shared_memory_per_multiprocessor
+    rows = (per_sm // 2 - 1024 - 1024 - 64) // 24 - 2      # the partition gives a block a row more or less
+    n = 2 * sms * rows
+    rp, c, v = _banded_spd(n, 1, 95)
+    b = torch.from_numpy(inputs.cg_rhs(n, 96)).cuda()
+    op = api.CsrOperator(ctx, torch.from_numpy(rp).cuda(), torch.from_numpy(c).cuda(), torch.from_numpy(v).cuda())
+    out = []
+    for lv in (0, level):
+        op.set_vector_cache(lv)
+        assert op.vector_cache_active == lv
+        x = torch.zeros(n, dtype=torch.float64, device="cuda")
+        op.solve(b, x, rtol=1e-10, mode=mode)
+        out.append(x)
+    assert torch.equal(out[0], out[1])
+    op.close()
