@@ -177,6 +177,14 @@ __global__ void __launch_bounds__(kCgThreads) cg_multi_restart(const __grid_cons
 
 __global__ void cg_multi_clear_done(MultiState *ms) { ms->done = 0; }
 
+__global__ void longest_row(const int *__restrict__ rowptr, int n, int *longest) {
+    int m = 0;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        m = max(m, rowptr[i + 1] - rowptr[i]);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(longest, m);
+}
+
 __global__ void check_columns(const int *__restrict__ col, long long nnz, int n, int *bad) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nnz; i += (long long)gridDim.x * blockDim.x)
         if (col[i] < 0 || col[i] >= n) { atomicExch(bad, 1); return; }
@@ -730,13 +738,14 @@ extern "C" perks_status perks_csr_create(perks_context *ctx, int32_t n, int64_t 
     OPCHK(dalloc(ctx, &op->part_row2, (size_t)G2 + 1));
     OPCHK(dalloc(ctx, &op->part_ntiles2, (size_t)G2));
     OPCHK(dalloc(ctx, &op->part_tiles2, (size_t)G2 * (kCgMaxTiles + 1)));
-    int *overflow = nullptr;
-    OPCHK(dalloc(ctx, &overflow, 1));
-    OPCUDA(cudaMemset(overflow, 0, sizeof(int)));
+    int *overflow = nullptr;  // and the longest row, which a walk over the host copy takes 0.6 ms for per million rows
+    OPCHK(dalloc(ctx, &overflow, 2));
+    OPCUDA(cudaMemset(overflow, 0, 2 * sizeof(int)));
     cg_partition_kernel<<<G, 256>>>(op->rowptr, n, nnz, G, op->part_row, op->part_ntiles, op->part_tiles,
                                     overflow);
     cg_partition_kernel<<<G2, 256>>>(op->rowptr, n, nnz, G2, op->part_row2, op->part_ntiles2, op->part_tiles2,
                                      overflow);
+    longest_row<<<std::min(n / 256 + 1, 4 * G), 256>>>(op->rowptr, n, overflow + 1);
     OPCUDA(cudaGetLastError());
     {
         std::vector<int> pr((size_t)G2 + 1);
@@ -745,12 +754,12 @@ extern "C" perks_status perks_csr_create(perks_context *ctx, int32_t n, int64_t 
             op->max_rows2 = std::max(op->max_rows2, pr[g + 1] - pr[g]);
             op->max_nnz2 = std::max(op->max_nnz2, rp[pr[g + 1]] - rp[pr[g]]);
         }
-        for (int i = 0; i < n; ++i) op->max_row = std::max(op->max_row, rp[i + 1] - rp[i]);
     }
-    int ov = 0;
-    OPCUDA(cudaMemcpy(&ov, overflow, sizeof(int), cudaMemcpyDeviceToHost));
+    int ov[2] = {0, 0};
+    OPCUDA(cudaMemcpy(ov, overflow, sizeof(ov), cudaMemcpyDeviceToHost));
     cudaFree(overflow);
-    if (ov) {
+    op->max_row = ov[1];
+    if (ov[0]) {
         free_op(op); delete op;
         return fail(ctx, PERKS_ERR_UNSUPPORTED, "csr_create: matrix too large (more than %d tiles per block)",
                     kCgMaxTiles);
