@@ -185,6 +185,17 @@ __global__ void longest_row(const int *__restrict__ rowptr, int n, int *longest)
     if ((threadIdx.x & 31) == 0) atomicMax(longest, m);
 }
 
+// Rows whose middle nonzero lies at most 8 columns from the next row's.
+__global__ void near_rows(const int *__restrict__ rowptr, const int *__restrict__ col, int n, int *near) {
+    int m = 0;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i + 1 < n; i += (long long)gridDim.x * blockDim.x) {
+        const int a = rowptr[i], b = rowptr[i + 1], c = rowptr[i + 2];
+        if (a < b && b < c) m += abs(col[(a + b) / 2] - col[(b + c) / 2]) <= 8;
+    }
+    m = __reduce_add_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m > 0) atomicAdd(near, m);
+}
+
 __global__ void check_columns(const int *__restrict__ col, long long nnz, int n, int *bad) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nnz; i += (long long)gridDim.x * blockDim.x)
         if (col[i] < 0 || col[i] >= n) { atomicExch(bad, 1); return; }
@@ -314,7 +325,8 @@ struct perks_op {
     double *b = nullptr, *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr;
     float *r32 = nullptr, *p32 = nullptr, *q32 = nullptr, *d32 = nullptr;
     double *part = nullptr;
-    int max_nnz2 = 0, max_row = 0;                      // nonzeros of the largest block (of G2), of the longest row
+    int max_nnz2 = 0;                                   // nonzeros of the largest block (of G2)
+    bool short_rows = false, short_spmv = false;        // one lane per row, in a solve and in a product by itself
     int dyn3 = 0;                                       // kind 3: dynamic shared memory a block may take
     double *trace = nullptr;
     int trace_cap = 0;
@@ -390,7 +402,7 @@ CgArgs make_args(perks_op *op, double rtol, int max_iter, int mode, double inner
         a.slice_nnz = (op->max_nnz2 + 3) & ~3;
         a.slice = mode != CGK_SPMV && slice_smem(op, mode) <= (size_t)op->dyn3;
     }
-    a.short_rows = rv && op->max_row <= kShortRow;  // at every vector cache level: the same sums
+    a.short_rows = rv && (mode == CGK_SPMV ? op->short_spmv : op->short_rows);  // at every vector cache level: the same sums
     a.seg.nseg = op->nseg;
     a.seg.val = op->sval;
     a.seg.val32 = op->sval32;
@@ -757,8 +769,17 @@ extern "C" perks_status perks_csr_create(perks_context *ctx, int32_t n, int64_t 
     }
     int ov[2] = {0, 0};
     OPCUDA(cudaMemcpy(ov, overflow, sizeof(ov), cudaMemcpyDeviceToHost));
+    // One lane per row or eight (spmv_rows_short): rows of 16 nonzeros at most, 15.5 on average; a product by itself 12.5,
+    // or 15.5 where neighbouring rows have neighbouring columns.
+    op->short_rows = op->short_spmv = ov[1] <= kShortRow && (double)nnz <= 15.5 * n;
+    if (op->short_rows && (double)nnz > 12.5 * n) {
+        OPCUDA(cudaMemset(overflow + 1, 0, sizeof(int)));
+        near_rows<<<std::min(n / 256 + 1, 4 * G), 256>>>(op->rowptr, op->col, n, overflow + 1);
+        OPCUDA(cudaGetLastError());
+        OPCUDA(cudaMemcpy(ov + 1, overflow + 1, sizeof(int), cudaMemcpyDeviceToHost));
+        op->short_spmv = 2LL * ov[1] > n;
+    }
     cudaFree(overflow);
-    op->max_row = ov[1];
     if (ov[0]) {
         free_op(op); delete op;
         return fail(ctx, PERKS_ERR_UNSUPPORTED, "csr_create: matrix too large (more than %d tiles per block)",

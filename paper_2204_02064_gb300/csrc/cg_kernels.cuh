@@ -486,15 +486,22 @@ __device__ double spmv_block_vec(const CgArgs &a, const CgSlice &sl, const V *__
     return block_sum(spmv_rows_vec<V>(a, sl, a.col, gval, vin, vout, dotv, vout_s), red);
 }
 
-// Short rows (at most kShortRow nonzeros): one lane per row, the gathers of
-// kShortStep of its nonzeros in flight.  A warp instruction of the FP64 pipe
+// Short rows (at most kShortRow nonzeros; csr_create chooses): one lane per
+// row, the gathers of kShortStep of its nonzeros in flight.  A warp instruction of the FP64 pipe
 // costs the same with one lane active or 32, so eight lanes per row spend
 // eight times the issue of a 5-entry row on padding and another three
 // additions on the exchange.  Rows are summed in order.  The thread that
 // computes a row also updates its vector entries.  Returns this thread's
 // share of the dot product.  An iteration of a 5-point matrix of 430 K rows:
 // 44.5 -> 23.6 us (fp64), 37.7 -> 18.5 us (fp32 inner), with the sums of
-// grid_sum4 and, in fp32, the nonzeros on chip.
+// grid_sum4 and, in fp32, the nonzeros on chip.  A lane's columns and values
+// are a run of their own, so a warp's loads of them touch up to 32 lines each.
+// At 16 nonzeros (all lanes' values 128 bytes apart) that costs more than the
+// padding wherever the columns lie, from 13 on in a product by itself whose
+// gathers too touch a line per lane.  3 M rows, one lane / eight, us: a product
+// with near columns of 9 nonzeros 101 / 162, 13 110 / 163, 15 130 / 163, 16 253 /
+// 162; scattered, 8 118 / 139, 12 176 / 181, 13 194 / 187, 15 227 / 215, 16 327 /
+// 229; ten fp64 iterations, scattered, 14 3167 / 3315, 16 4498 / 3623.
 constexpr int kShortRow = 16;
 constexpr int kShortStep = 8;
 template <typename V>

@@ -414,3 +414,45 @@ def test_vector_cache_at_the_limit_of_shared_memory(ctx, level, mode):
         out.append(x)
     assert torch.equal(out[0], out[1])
     op.close()
+
+
+@pytest.mark.parametrize("near", [True, False], ids=["near", "scattered"])
+@pytest.mark.parametrize("m", [12, 13, 14, 15, 16, 17])
+def test_rows_around_the_one_lane_limit(ctx, oracle, m, near):
+    """Every row holds m nonzeros, in columns beside the diagonal or anywhere: products and solves on either side of
+    the line between one lane per row and eight."""
+    from paper_2204_02064_gb300 import api
+    n = 40000
+    at, rows, cols = np.arange(n), [], []
+    rng = np.random.default_rng(m)
+    for h in range((m - 1) // 2):                  # cycles through all rows: two entries each
+        p = at if near else rng.permutation(n)
+        q = (at + h + 1) % n if near else np.roll(p, 1)
+        rows += [p, q]
+        cols += [q, p]
+    if (m - 1) % 2:                                # and pairs: one
+        p = at if near else rng.permutation(n)
+        rows += [p[:n // 2], p[n // 2:]]
+        cols += [p[n // 2:], p[:n // 2]]
+    r, c = np.concatenate(rows), np.concatenate(cols)
+    key = np.unique(r * n + c)                     # a few scattered pairs coincide
+    r, c = key // n, key % n
+    v = -1.0 - ((r * c) % 7) / 8.0
+    diag = 1.05 * np.bincount(r, weights=-v, minlength=n)
+    r, c, v = np.concatenate([r, at]), np.concatenate([c, at]), np.concatenate([v, diag])
+    o = np.lexsort((c, r))
+    c, v = c[o].astype(np.int32), v[o]
+    rp = np.concatenate([[0], np.cumsum(np.bincount(r, minlength=n))]).astype(np.int32)
+    b = inputs.cg_rhs(n, 97)
+    op = _op(ctx, rp, c, v)
+    y = torch.zeros(n, dtype=torch.float64, device="cuda")
+    op.spmv(_dev(b), y)
+    torch.cuda.synchronize()
+    # rows of up to 17 terms, 62 in all, in another order on either side
+    assert np.max(np.abs(y.cpu().numpy() - oracle.spmv(rp, c, v, b))) <= 17 * 2.0 ** -52 * 62.0
+    ref = oracle.cg(rp, c, v, b, rtol=1e-10)
+    for mode in (api.CG_FP64, api.CG_FP32_IR):
+        x = torch.zeros(n, dtype=torch.float64, device="cuda")
+        assert op.solve(_dev(b), x, rtol=1e-10, mode=mode)["true_rel_residual"] <= 1e-10
+        assert np.linalg.norm(x.cpu().numpy() - ref["x"]) <= 1e-8 * np.linalg.norm(ref["x"])
+    op.close()
