@@ -592,6 +592,11 @@ struct LogProd {
         m <<= n;
         e -= n;
     }
+    // no value had a logarithm of its own and the product is within 2^-20 of 1, and not 1; m normalised
+    __device__ __forceinline__ bool near_one() const {
+        if (__double_as_longlong(s) != 0) return false;
+        return e == 0 ? m >> 43 == 1ull << 20 && m != 1ull << 63 : e == -1 && m >> 43 == (1ull << 21) - 1;
+    }
     // sum of the logarithms; m normalised
     __device__ __forceinline__ double value() const {
         const double d = __ull2double_rn(m);  // in [2^63, 2^64]
@@ -599,6 +604,17 @@ struct LogProd {
         return fma((double)e, 0.69314718055994530942, log(x)) + s;
     }
 };
+
+// Sum of the logarithms of a coarse cell whose product is near 1: LogProd's
+// error, 2^-47 at most whatever the sum, would no longer be small beside it
+// (coefficients within 1e-9 of 1: 1e-7 of the mean at F = 2, 1e-12: 3e-3).
+// Rare, and out of line.
+__device__ __noinline__ double log_sum(const double *k, int nx, int F) {
+    double s = 0.0;
+    for (int dy = 0; dy < F; ++dy)
+        for (int dx = 0; dx < F; ++dx) s += log(k[(long long)dy * nx + dx]);
+    return s;
+}
 
 constexpr int kPoolThreads = 256;
 constexpr int kPoolJobs = 8;  // jobs per round, at most
@@ -701,7 +717,8 @@ __global__ void __launch_bounds__(kPoolThreads, 3) features_kernel(const double 
                         }
                     lp.normalise();
                 }
-                lk = lp.value();
+                if (lp.near_one()) lk = log_sum(k + (long long)row * F * nx + (long long)X * F, nx, F);
+                else lk = lp.value();
             }
             const long long img = row / H, p = (long long)(row % H) * W + X;
             x0[(img * 2 + 0) * plane + p] = st_f<S>((float)(lk * inv));

@@ -459,3 +459,28 @@ def test_pooling_rounds_of_jobs(ctx, F, ny, nx, nimg):
         torch.cuda.synchronize()
         assert torch.equal(one[0], u[i]), i
     net.close()
+
+
+@pytest.mark.parametrize("F", [1, 2, 3, 8, 32])
+@pytest.mark.parametrize("amp", [1e-5, 1e-7, 1e-9, 1e-12, 2e-16, 0.0])
+def test_log_of_coefficients_near_one(ctx, F, amp):
+    """Coefficients 1 + amp x [-1/4, 1]: the mean log keeps its digits however small it is, from the network of the
+    test above (fp32 rounding of a mean); a field of ones gives 0."""
+    from paper_2204_02064_gb300 import api
+    ny, nx = 4 * F, 8 * F
+    k = 1.0 + amp * (1.25 * inputs.uniform(91, ny * nx).reshape(1, ny, nx) - 0.25)
+    net = api.WarmNet(ctx, storage=api.F32, dilations=DIL, seed=1, pool=F)
+    p = _pass_through_params(0)
+    p[2 * 9 + 4] = -1.0
+    a1 = 32 * 2 * 9 + 32
+    p[a1 + (32 + 1) * 9 + 4] = 1.0
+    a2 = a1 + 32 * 32 * 9 + 32
+    p[a2 + (32 + 1) * 9 + 4] = 1.0
+    p[a2 + 32 * 32 * 9 + 32 + 9 + 4] = -1.0
+    net.params = p
+    net.scale = 1.0
+    u = torch.zeros((1, ny, nx), dtype=torch.float64, device="cuda")
+    net.predict(_dev(k), _dev(np.zeros_like(k)), u)
+    torch.cuda.synchronize()
+    ref = _bilinear(_pool(np.log(k), F), F)
+    assert np.max(np.abs(u.cpu().numpy() - ref)) <= 2.0 ** -22 * np.max(np.abs(ref))
