@@ -259,3 +259,27 @@ def test_memory_is_a_few_vectors(ctx, nprob, ny, nx):
         xs.append(x)
     assert float((xs[0] - xs[1]).norm()) <= 1e-8 * float(xs[1].norm()) and float(xs[1].norm()) > 0.0
     P.close()
+
+
+def test_automatic_group_wait_timeout_reported(ctx, oracle):
+    """A block of an automatic group that waits for the others' sums past the limit ends the solve with
+    BARRIER_TIMEOUT; the next solve starts from clean slots."""
+    from paper_2204_02064_gb300 import api
+    k = _k(4, 300, 300, 25)
+    f = 2.0 * inputs.uniform(26, k.size).reshape(k.shape) - 1.0
+    P = api.Poisson(ctx, torch.from_numpy(k).cuda())
+    b, x = torch.from_numpy(f).cuda(), torch.zeros(k.shape, dtype=torch.float64, device="cuda")
+    ctx.set_barrier_timeout(0)
+    try:
+        with pytest.raises(api.PerksError) as ei:
+            P.solve(b, x, rtol=1e-8)
+        assert ei.value.name == "BARRIER_TIMEOUT"
+    finally:
+        ctx.set_barrier_timeout(2_000_000_000)
+    x.zero_()
+    res = P.solve(b, x, rtol=1e-8)
+    assert res["grid_blocks"] > k.shape[0] and res["max_true_rel_residual"] <= 1e-8
+    rp, c, val = oracle.poisson_csr(k[0])
+    ref = oracle.cg(rp, c, val, f[0].ravel(), rtol=1e-8, max_iter=20000)
+    assert np.linalg.norm(x[0].cpu().numpy().ravel() - ref["x"]) <= 1e-6 * np.linalg.norm(ref["x"])
+    P.close()

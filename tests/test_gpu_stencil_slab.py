@@ -114,3 +114,34 @@ def test_plan_is_kept_until_the_request_changes(ctx):
     st.set_trace(0)
     assert st.describe(10) == first
     st.close()
+
+
+@pytest.mark.parametrize("name", ["3d7pt", "3d13pt", "3d27pt", "poisson"])
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("nx", [33, 40])
+@pytest.mark.parametrize("parts", [47, 9, 8, 7, 6, 5, 2, 1])
+def test_slab_parts_of_every_depth(ctx, oracle, name, dtype, nx, parts):
+    """A column of 47 planes cut into parts of 1, 5, 6, 7, 8, 9, 23 and 47: ring slots filled again, the planes in the
+    middle of a part without checks, for every remainder of the unrolled loops."""
+    from paper_2204_02064_gb300 import api
+    if dtype == "bf16":
+        nx = nx // 8 * 8
+    stats = _check(ctx, oracle, name, dtype, (47, 9, nx), 3, api.KERNEL_SLAB, tiles=(1, 1, parts))
+    assert stats["tiles_z"] == parts
+    # (fp64 without parts: the planner's own equal shares)
+    assert stats["grid_blocks"] == (47 if dtype == "f64" and parts == 1 else parts)
+
+
+@pytest.mark.parametrize("name", ["3d7pt", "3d13pt", "3d27pt", "poisson"])
+@pytest.mark.parametrize("dtype,nx", [("f64", 9), ("f64", 16), ("f32", 9), ("f32", 16), ("bf16", 16)])
+def test_slab_equal_shares_across_columns(ctx, oracle, name, dtype, nx):
+    """Equal shares of seven planes that run from one column into the next (two parts per column would leave a fifth of
+    the blocks idle): 61 columns of 35 planes, in fp64 one long column too."""
+    from paper_2204_02064_gb300 import api
+    rows = 32 * (4 if dtype == "f32" and name in ("3d27pt", "poisson") else 2)   # of a column of 8 lanes a row
+    shapes = [(35, 60 * rows + 5, nx)] + ([(2200, 9, nx)] if dtype == "f64" else [])
+    for shape in shapes:
+        stats = _check(ctx, oracle, name, dtype, shape, 2, api.KERNEL_SLAB)
+        columns = stats["tiles_x"] * stats["tiles_y"]
+        assert columns == (61 if shape[0] == 35 else 1) and stats["tiles_z"] == 1
+        assert stats["grid_blocks"] * 6 < columns * shape[0]

@@ -484,3 +484,79 @@ def test_log_of_coefficients_near_one(ctx, F, amp):
     torch.cuda.synchronize()
     ref = _bilinear(_pool(np.log(k), F), F)
     assert np.max(np.abs(u.cpu().numpy() - ref)) <= 2.0 ** -22 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("dil", [(16, 16, 16, 16), (3, 12, 5, 16), (1, 7, 13, 2)])
+def test_forward_bf16_other_dilations(ctx, oracle, dil):
+    """The tensor-core layers' staged halo, operand strides and shared memory follow the dilation, up to the largest
+    the ABI takes; tolerance as for the default dilations (a sum on a bf16 rounding boundary)."""
+    from paper_2204_02064_gb300 import api
+    nimg, ny, nx = 2, 53, 70
+    k, f = _case(nimg, ny, nx, 51)
+    net = api.WarmNet(ctx, storage=api.BF16, dilations=dil, seed=1)
+    p = _params(8)
+    net.params = p
+    net.scale = 1.0
+    u = torch.zeros((nimg, ny, nx), dtype=torch.float64, device="cuda")
+    net.predict(_dev(k), _dev(f), u)
+    torch.cuda.synchronize()
+    rb = oracle.bf16_round
+    x = _features(k, f, lambda a: rb(a.astype(np.float32)).astype(np.float64))
+    pd, ref = p.astype(np.float64), []
+    for i in range(nimg):
+        y, o = x[i], 0
+        for l, (co, ci) in enumerate([(C1, 2), (C1, C1), (C1, C1), (1, C1)]):
+            W, B = pd[o:o + co * ci * 9].reshape(co, ci, 3, 3), pd[o + co * ci * 9:o + co * ci * 9 + co]
+            o += co * ci * 9 + co
+            y = oracle.conv2d(y, W, B, dil[l])
+            if l < 3:
+                y = rb(np.maximum(y, 0).astype(np.float32)).astype(np.float64)
+        ref.append(y[0])
+    ref = np.stack(ref)
+    assert np.max(np.abs(u.cpu().numpy() - ref)) <= 1e-2 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("dil", [(16, 11, 3, 16), (5, 8, 11, 13)])
+def test_f32_other_dilations(ctx, oracle, dil):
+    """Forward and gradient in fp32 at dilations whose tiles are mostly halo (11: the widest the inner layers' forward
+    takes); tolerances of the default dilations."""
+    from paper_2204_02064_gb300 import api
+    nimg, ny, nx = 2, 37, 51
+    k, f = _case(nimg, ny, nx, 52)
+    u = inputs.uniform(53, nimg * ny * nx).reshape(nimg, ny, nx) * 3.0 - 1.0
+    net = api.WarmNet(ctx, storage=api.F32, dilations=dil, seed=1)
+    p = _params(9)
+    net.params = p
+    net.scale = 1.5
+    out = torch.zeros((nimg, ny, nx), dtype=torch.float64, device="cuda")
+    net.predict(_dev(k), _dev(f), out)
+    torch.cuda.synchronize()
+    x = _features(k, f, lambda a: a.astype(np.float32).astype(np.float64))
+    ref = np.stack([oracle.warmnet_forward(p.astype(np.float64), x[i], C1, dil) for i in range(nimg)]) * 1.5
+    assert np.max(np.abs(out.cpu().numpy() - ref)) <= 1e-4 * np.max(np.abs(ref))
+    loss, g = net.gradient(_dev(k), _dev(f), _dev(u))
+    ref_loss, ref_g = oracle.warmnet_grad(p.astype(np.float64), x, u / 1.5, C1, dil)
+    assert loss == pytest.approx(ref_loss, rel=1e-4)
+    assert np.max(np.abs(g - ref_g)) <= 1e-4 * np.max(np.abs(ref_g))
+
+
+def test_gradient_bf16_other_dilations(ctx, oracle):
+    """bf16 gradient at the widest dilation the inner layers' weight gradient takes (14); the next one is an error, and
+    leaves the context usable."""
+    from paper_2204_02064_gb300 import api
+    nimg, ny, nx = 2, 40, 44
+    k, f = _case(nimg, ny, nx, 54)
+    u = inputs.uniform(55, nimg * ny * nx).reshape(nimg, ny, nx) * 2.0 - 1.0
+    wide = api.WarmNet(ctx, storage=api.BF16, dilations=(1, 2, 15, 8), seed=1)
+    with pytest.raises(api.PerksError):
+        wide.gradient(_dev(k), _dev(f), _dev(u))
+    wide.close()
+    dil = (2, 14, 12, 16)
+    net = api.WarmNet(ctx, storage=api.BF16, dilations=dil, seed=1)
+    p = _params(10)
+    net.params = p
+    loss, g = net.gradient(_dev(k), _dev(f), _dev(u))
+    x = _features(k, f)
+    ref_loss, ref_g = oracle.warmnet_grad(p.astype(np.float64), x, u, C1, dil)
+    assert loss == pytest.approx(ref_loss, rel=5e-2)
+    assert np.linalg.norm(g - ref_g) <= 5e-2 * np.linalg.norm(ref_g)
