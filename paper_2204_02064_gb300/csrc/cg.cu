@@ -364,7 +364,7 @@ void free_op(perks_op *op) {
 // nonzero (8 in fp32) and 4 per row.
 size_t slice_smem(const perks_op *op, int mode) {
     const size_t nnz = ((size_t)op->max_nnz2 + 3) & ~size_t(3);
-    return kCgShortSmem + ((nnz * (mode == CGK_FP32_IR ? 4 : 8) + 15) & ~size_t(15)) + nnz * 4 +
+    return kCgRowvecSmem + ((nnz * (mode == CGK_FP32_IR ? 4 : 8) + 15) & ~size_t(15)) + nnz * 4 +
            ((size_t)op->max_rows2 + 4) * 4;
 }
 
@@ -439,7 +439,7 @@ perks_status configure(perks_op *op) {
     if (per_sm2 < 1 || per_sm2 * ctx->sm_count < op->G2)
         return fail(ctx, PERKS_ERR_LAUNCH_TOO_LARGE, "CG kernel of %d blocks is not co-resident", op->G2);
     // vector cache: on when the largest block's rows fit with all G2 blocks co-resident
-    op->smem_vc = kCgRowvecSmem + (((size_t)op->max_rows2 * kCgVcacheBytesPerRow + 15) & ~size_t(15));
+    op->smem_vc = kCgVcacheSmem + (((size_t)op->max_rows2 * kCgVcacheBytesPerRow + 15) & ~size_t(15));
     op->vcache_ok = false;
     // (the attribute is per function, shared by every operator: set to the
     // device limit less the kernel's static shared memory; each launch passes
@@ -479,7 +479,7 @@ perks_status configure(perks_op *op) {
 size_t rowvec_smem(const perks_op *op, int level) {
     if (level <= 0) return kCgRowvecSmem;
     const size_t per_row = level == 1 ? sizeof(double) : kCgVcacheBytesPerRow;
-    return kCgRowvecSmem + (((size_t)op->max_rows2 * per_row + 15) & ~size_t(15));
+    return kCgVcacheSmem + (((size_t)op->max_rows2 * per_row + 15) & ~size_t(15));
 }
 
 perks_status launch_persistent(perks_op *op, const CgArgs &a, cudaStream_t s) {
@@ -491,7 +491,7 @@ perks_status launch_persistent(perks_op *op, const CgArgs &a, cudaStream_t s) {
     // keep kind 0, whose L1 is not cut by shared memory.
     if (op->spmv_kind == PERKS_SPMV_ROWVEC && a.vcache == 0 && (a.slice || a.short_rows))
         PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)perks_cg_kernel<3>, dim3(op->G2), dim3(kCgThreads),
-                                                    args, a.slice ? slice_smem(op, a.mode) : kCgShortSmem, s));
+                                                    args, a.slice ? slice_smem(op, a.mode) : kCgRowvecSmem, s));
     else if (op->spmv_kind == PERKS_SPMV_ROWVEC)
         PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)perks_cg_kernel<0>, dim3(op->G2),
                                                     dim3(kCgThreads), args, rowvec_smem(op, a.vcache), s));

@@ -558,12 +558,13 @@ __device__ __forceinline__ bool cg_sync(const CgArgs &a, unsigned long long &epo
     return grid_barrier(a.bar, gridDim.x, epoch, a.err, a.timeout_ns);
 }
 
-// Shared memory of the row-vector kernel (kind 0): the reduction scratch, the
-// small one, followed (vector cache on) by kCgVcacheBytesPerRow bytes per row
-// of the largest block: x, r and q in fp64, or r32, d32 and q32 for the fp32
-// inner solves.  Kind 3: the scratch of reduce4, then a block's nonzeros.
-constexpr size_t kCgRowvecSmem = kSmallReduceBytes;
-constexpr size_t kCgShortSmem = (reduce_scratch<kCgThreads>() * sizeof(double) + 1023) / 1024 * 1024;
+// Shared memory of the row-vector kernels: the scratch of reduce4, in kind 3
+// followed by a block's nonzeros.  With the vector cache on (kind 0), the small
+// scratch, followed by kCgVcacheBytesPerRow bytes per row of the largest block:
+// x, r and q in fp64, or r32, d32 and q32 for the fp32 inner solves.  (Without
+// the cache the small scratch's extra barriers cost the n = 2^20 solve 2.7 %.)
+constexpr size_t kCgRowvecSmem = (reduce_scratch<kCgThreads>() * sizeof(double) + 1023) / 1024 * 1024;
+constexpr size_t kCgVcacheSmem = kSmallReduceBytes;
 constexpr size_t kCgVcacheBytesPerRow = 3 * sizeof(double);
 
 // Persistent CG (mode FP64 / FP32_IR) or a single SpMV (mode SPMV).
@@ -625,7 +626,7 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 || KIND == 3 ? 2 : 1) pe
     if constexpr (KIND == 3) {
         if (a.slice) {
             const bool single = a.mode == CGK_FP32_IR;
-            unsigned char *at = smem_raw + kCgShortSmem;
+            unsigned char *at = smem_raw + kCgRowvecSmem;
             double *sv = reinterpret_cast<double *>(at);
             float *sv32 = reinterpret_cast<float *>(at);
             at += ((size_t)a.slice_nnz * (single ? 4 : 8) + 15) & ~size_t(15);
@@ -683,8 +684,11 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 || KIND == 3 ? 2 : 1) pe
     // grid-wide sum of v over all threads, with post(total, ratio, flag) of it, and a grid barrier
     auto gsum = [&](double v, SumResult &out, auto &&post) -> bool {
         if constexpr (EXCHANGE) {
-            return grid_sum4<kCgThreads, KIND == 0>(a.part, gridDim.x, a.bar, epoch, a.err, a.timeout_ns, round, v,
-                                                    s.red, out, post);
+            if (KIND == 0 && a.vcache > 0)
+                return grid_sum4<kCgThreads, true>(a.part, gridDim.x, a.bar, epoch, a.err, a.timeout_ns, round, v, s.red,
+                                                   out, post);
+            return grid_sum4<kCgThreads, false>(a.part, gridDim.x, a.bar, epoch, a.err, a.timeout_ns, round, v, s.red,
+                                                out, post);
         } else {
             double *part = a.part + (size_t)(round++ & 1) * gridDim.x;
             v = block_sum(v, s.red);
@@ -731,9 +735,9 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 || KIND == 3 ? 2 : 1) pe
     const bool vr32 = KIND == 0 && a.vcache >= 1 && a.mode == CGK_FP32_IR;
     const bool vc32 = KIND == 0 && a.vcache >= 2 && a.mode == CGK_FP32_IR;
     const int cap = a.vcache_rows;
-    double *rs = reinterpret_cast<double *>(smem_raw + kCgRowvecSmem);
+    double *rs = reinterpret_cast<double *>(smem_raw + kCgVcacheSmem);
     double *xs = rs + cap, *qs = xs + cap;
-    float *r32s = reinterpret_cast<float *>(smem_raw + kCgRowvecSmem);
+    float *r32s = reinterpret_cast<float *>(smem_raw + kCgVcacheSmem);
     float *d32s = r32s + cap, *q32s = d32s + cap;
     const int r0 = sl.r0;
     auto X = [&](int i) -> double & { return vc64 ? xs[i - r0] : x[i]; };
