@@ -229,7 +229,7 @@ struct perks_stencil {
     int cur = 0;
     void *faces[2] = {nullptr, nullptr};
     size_t faces_bytes = 0;
-    unsigned long long *bar = nullptr;     // barrier counter, then the patch kernel's exchange counts, one per SM
+    unsigned long long *bar = nullptr;     // barrier counter, and kFlagsAt words on the patch kernel's exchange counts
     DevError *err = nullptr;
     int shape_id = -1;
     double kw[kMaxKernelPoints] = {};
@@ -985,9 +985,10 @@ void fill_stats(const perks_stencil *st, const Plan *pl, long long steps, int va
 // The counters and the error record of every persistent kernel: whichever runs
 // first allocates them for all, so that a later run under capture, where
 // nothing can be allocated, may take another one.
+constexpr int kFlagsAt = 32;  // 256 bytes: a memset of the flags starts on an allocation's boundary
 perks_status ensure_sync(perks_stencil *st) {
     perks_context *ctx = st->ctx;
-    if (!st->bar) PERKS_CUDA(ctx, cudaMalloc(&st->bar, sizeof(unsigned long long) * (1 + (size_t)ctx->sm_count)));
+    if (!st->bar) PERKS_CUDA(ctx, cudaMalloc(&st->bar, sizeof(unsigned long long) * (kFlagsAt + (size_t)ctx->sm_count)));
     if (!st->err) PERKS_CUDA(ctx, cudaMalloc(&st->err, sizeof(DevError)));
     return PERKS_OK;
 }
@@ -1107,10 +1108,10 @@ perks_status run_patch(perks_stencil *st, long long steps, cudaStream_t s, const
     for (int i = 0; i < 25; ++i) { a.w[i] = st->kw[i]; a.wf[i] = (float)st->kw[i]; }
     a.field[0] = st->field[st->cur];
     a.field[1] = st->field[st->cur ^ 1];
-    a.flags = st->bar + 1;
+    a.flags = st->bar + kFlagsAt;
     a.err = st->err;
     a.timeout_ns = ctx->timeout_ns;
-    PERKS_CUDA(ctx, cudaMemsetAsync(st->bar + 1, 0, sizeof(unsigned long long) * ctx->sm_count, s));
+    PERKS_CUDA(ctx, cudaMemsetAsync(st->bar + kFlagsAt, 0, sizeof(unsigned long long) * ctx->sm_count, s));
     PERKS_CUDA(ctx, cudaMemsetAsync(st->err, 0, sizeof(DevError), s));
     void *args[] = {&a};
     PERKS_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)pl.qk->fn, dim3(pl.blocks), dim3(kPatchThreads), args,
