@@ -701,16 +701,15 @@ perks_status plan_strips(perks_batch *b, int rows) {
     std::iota(order.begin(), order.end(), 0);
     if (items.size() <= (size_t)nwarps) {
         // A warp per item at most: neighbouring items, one shape's after the other's, to the warps of a block, the same
-        // number in every block, and neighbouring runs to the two blocks that share an SM.  An SM then runs one or two
-        // shapes' code, and not four's: 40 fp32 domains of 244 x 333, four shapes, 9.8 us a step, 14.9 with an SM's items
-        // from all over the batch.  (A heap of idle warps, as below, does much the same, at 60 ns an item: as long as
-        // several steps of a small batch.)
+        // number in every block.  An SM then runs two or three shapes' code, not four's (40 fp32 domains of 244 x 333, four
+        // shapes, 9.4 us a step, 14.9 with an SM's items from all over the batch), and its two blocks, half the batch apart,
+        // shapes that differ in what bounds them (the 64-domain workload 2.5 % faster than with one shape's).  (A heap of
+        // idle warps, as below, does much the same, at 60 ns an item: as long as several steps of a small batch.)
         std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->shape[items[x].dom] < b->shape[items[y].dom]; });
         const int wpb = k->threads / 32, n = (int)items.size();
         for (int r = 0; r < G; ++r) {
-            const int block = r / per_sm + r % per_sm * ctx->sm_count;
             const int q0 = (int)((long long)n * r / G), q1 = (int)((long long)n * (r + 1) / G);
-            for (int q = q0; q < q1; ++q) owner[order[q]] = block * wpb + q - q0;
+            for (int q = q0; q < q1; ++q) owner[order[q]] = r * wpb + q - q0;
         }
     } else {
         // LPT: the costliest item to the least loaded warp
