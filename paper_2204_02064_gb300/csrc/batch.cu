@@ -121,8 +121,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) perks_batch_kernel(const __g
 //
 // Column-strip streaming: the batch's work is cut into items (domain, strip
 // of 32 vectors = 32 V cells, or a little less where strips overlap, range of
-// rows) and a static longest-processing-time-first assignment gives every WARP
-// its items.  A
+// rows) and a static assignment (plan_strips) gives every WARP its items.  A
 // warp streams its item's input rows through a private ring of D row slots
 // in shared memory (16-byte cp.async per lane, plus two halo cells on each
 // side from the neighbouring strips), keeps the 2R + 1 rows the stencil
@@ -154,18 +153,16 @@ struct StripArgs {
 // fp64 (fp32 takes perks_batch_sweep_kernel)
 constexpr int kStripThreads = 256;
 constexpr int kStripDepth = 8;   // ring rows per warp (16 measured slower: longer ring fill per item)
-
-template <typename T, int V>
-__host__ __device__ constexpr int strip_row_cells() { return 32 * V + 2 * V; }  // V pad cells on each side
+constexpr int kStripCells = 2;   // cells per lane
+constexpr int kStripRow = 34 * kStripCells;  // cells of a ring row: a lane's worth of padding on each side
 
 // One item: output rows z0..z1-1 of the strip at x0.
-template <typename T, class SH, int V, int D>
-__device__ __forceinline__ void strip_item(const PersistentArgs &a, const StripItem it, int src, T *ring, int lane) {
-    using A = typename ScalarOps<T>::A;
+template <class SH>
+__device__ __forceinline__ void strip_item(const PersistentArgs &a, const StripItem it, int src, double *ring, int lane) {
+    using T = double;
+    constexpr int R = SH::R, W = 2 * R + 1;
+    constexpr int V = kStripCells, D = kStripDepth, ROW = kStripRow;
     using VT = VecOf<T, V>;
-    constexpr int R = SH::R;
-    constexpr int W = 2 * R + 1;
-    constexpr int ROW = strip_row_cells<T, V>();
     static_assert(R <= 2 && D > 2 * R, "strip ring depth");
     const T *in = static_cast<const T *>(a.field[src]);
     T *out = static_cast<T *>(a.field[src ^ 1]);
@@ -173,7 +170,7 @@ __device__ __forceinline__ void strip_item(const PersistentArgs &a, const StripI
     const int xl = it.x0 + lane * V;
     const bool own = xl < X;
     const T bnd = ScalarOps<T>::bnd(a);
-    A w[SH::NPTS];
+    T w[SH::NPTS];
 #pragma unroll
     for (int i = 0; i < SH::NPTS; ++i) w[i] = ScalarOps<T>::w(a, i);
     const int rfirst = it.z0 - R, rlast = it.z1 - 1 + R;
@@ -196,26 +193,26 @@ __device__ __forceinline__ void strip_item(const PersistentArgs &a, const StripI
         }
         cp_async_commit();
     };
-    // the lane's cells -2 .. V+1 of row r (from its ring slot), in the accumulator type
-    auto fetch = [&](int r, A (&row)[V + 4]) {
+    // the lane's cells -2 .. V+1 of row r (from its ring slot)
+    auto fetch = [&](int r, T (&row)[V + 4]) {
         cp_async_wait<D - 1>();
         __syncwarp();
         const T *p = ring + ((r - rfirst) % D) * ROW + V + lane * V;
         const VT c = *reinterpret_cast<const VT *>(p);
         const PairOf<T> l = *reinterpret_cast<const PairOf<T> *>(p - 2);
         const PairOf<T> h = *reinterpret_cast<const PairOf<T> *>(p + V);
-        row[0] = to_acc(l.v[0]);
-        row[1] = to_acc(l.v[1]);
+        row[0] = l.v[0];
+        row[1] = l.v[1];
 #pragma unroll
-        for (int j = 0; j < V; ++j) row[2 + j] = to_acc(c.v[j]);
-        row[V + 2] = to_acc(h.v[0]);
-        row[V + 3] = to_acc(h.v[1]);
+        for (int j = 0; j < V; ++j) row[2 + j] = c.v[j];
+        row[V + 2] = h.v[0];
+        row[V + 3] = h.v[1];
         __syncwarp();  // every lane has read the slot before it is refilled
         issue(r + D);
     };
 
     for (int j = 0; j < D; ++j) issue(rfirst + j);
-    A win[W][V + 4];
+    T win[W][V + 4];
     // the first 2R rows of the window: rows z0-R .. z0+R-1 in slots 0 .. 2R-1
     static_for<0, 2 * R>([&](auto JI) { fetch(rfirst + decltype(JI)::value, win[decltype(JI)::value]); });
     // output row z reads window slots (z - rfirst + k) % W, k = 0..2R; the loop
@@ -227,17 +224,14 @@ __device__ __forceinline__ void strip_item(const PersistentArgs &a, const StripI
             if (z < it.z1) {
                 fetch(z + R, win[(p + 2 * R) % W]);
                 VT o;
-                A acc[V];
 #pragma unroll
-                for (int q = 0; q < V; ++q) acc[q] = A(0);
+                for (int q = 0; q < V; ++q) o.v[q] = 0.0;
                 static_for<0, SH::NPTS>([&](auto II) {
                     constexpr int i = decltype(II)::value;
                     constexpr int slot = (p + R + SH::dz(i)) % W;
 #pragma unroll
-                    for (int q = 0; q < V; ++q) acc[q] = fma(w[i], win[slot][2 + q + SH::dx(i)], acc[q]);
+                    for (int q = 0; q < V; ++q) o.v[q] = fma(w[i], win[slot][2 + q + SH::dx(i)], o.v[q]);
                 });
-#pragma unroll
-                for (int q = 0; q < V; ++q) o.v[q] = from_acc<T>(acc[q]);
                 if (own) *reinterpret_cast<VT *>(out + (long long)z * X + xl) = o;
             }
         });
@@ -246,12 +240,10 @@ __device__ __forceinline__ void strip_item(const PersistentArgs &a, const StripI
     __syncwarp();
 }
 
-template <typename T, int V>
 __global__ void __launch_bounds__(kStripThreads, 1) perks_batch_strip_kernel(const __grid_constant__ StripArgs b) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int D = kStripDepth;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    T *ring = reinterpret_cast<T *>(smem_raw) + (long long)warp * D * strip_row_cells<T, V>();
+    double *ring = reinterpret_cast<double *>(smem_raw) + (long long)warp * kStripDepth * kStripRow;
     const int gw = blockIdx.x * (kStripThreads / 32) + warp;
     const int i0 = b.warp_first[gw], i1 = b.warp_first[gw + 1];
     unsigned long long epoch = 0;
@@ -261,10 +253,10 @@ __global__ void __launch_bounds__(kStripThreads, 1) perks_batch_strip_kernel(con
             const StripItem it = b.items[q];
             const PersistentArgs &a = b.doms[it.dom];
             switch (b.dom_shape[it.dom]) {
-            case SH_2D5: strip_item<T, S2d5, V, D>(a, it, src, ring, lane); break;
-            case SH_2D9: strip_item<T, S2d9, V, D>(a, it, src, ring, lane); break;
-            case SH_2D25: strip_item<T, S2d25, V, D>(a, it, src, ring, lane); break;
-            default: strip_item<T, S2ds9, V, D>(a, it, src, ring, lane); break;
+            case SH_2D5: strip_item<S2d5>(a, it, src, ring, lane); break;
+            case SH_2D9: strip_item<S2d9>(a, it, src, ring, lane); break;
+            case SH_2D25: strip_item<S2d25>(a, it, src, ring, lane); break;
+            default: strip_item<S2ds9>(a, it, src, ring, lane); break;
             }
         }
         if (k + 1 < b.steps) {
@@ -353,8 +345,8 @@ struct StripKernel {
 
 const StripKernel *strip_kernel(int dtype) {
     static const StripKernel f32 = {perks_batch_sweep_kernel<float>, kSweepThreads, 0, 30 * 4};
-    static const StripKernel f64 = {perks_batch_strip_kernel<double, 2>, kStripThreads,
-                                    (size_t)(kStripThreads / 32) * kStripDepth * strip_row_cells<double, 2>() * 8, 32 * 2};
+    static const StripKernel f64 = {perks_batch_strip_kernel, kStripThreads,
+                                    sizeof(double) * (kStripThreads / 32) * kStripDepth * kStripRow, 32 * kStripCells};
     return dtype == PERKS_F32 ? &f32 : dtype == PERKS_F64 ? &f64 : nullptr;
 }
 

@@ -398,7 +398,6 @@ CgArgs make_args(perks_op *op, double rtol, int max_iter, int mode, double inner
     a.vcache = rv && op->vcache_ok && mode != CGK_SPMV ? op->vcache_level : 0;
     a.vcache_rows = op->max_rows2;
     if (rv && a.vcache == 0) {
-        a.slice_rows = op->max_rows2;
         a.slice_nnz = (op->max_nnz2 + 3) & ~3;
         a.slice = mode != CGK_SPMV && slice_smem(op, mode) <= (size_t)op->dyn3;
     }

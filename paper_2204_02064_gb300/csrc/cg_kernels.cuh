@@ -34,8 +34,6 @@
 namespace perks {
 
 constexpr int kCgThreads = 512;
-// vector entries of a thread whose loads are in flight together (within 64 registers)
-constexpr int kCgRows64 = 1, kCgRows32 = 1;
 constexpr int kCgIpt = 4;
 constexpr int kCgTile = kCgThreads * kCgIpt;  // merge-path items per tile
 constexpr int kCgMaxTiles = 2048;              // tiles per block
@@ -80,7 +78,7 @@ struct CgArgs {
     int vcache_rows;         // rows of the largest block (capacity of each cached vector)
     int slice;               // kind 3: the blocks keep their nonzeros (of the solve's value type) in shared memory
     int short_rows;          // row-vector kinds: one lane per row (else eight)
-    int slice_rows, slice_nnz;  // rows and nonzeros of the largest block
+    int slice_nnz;           // nonzeros of the largest block
     const double *spmv_in;
     double *spmv_out;
     SegArgs seg;             // column-segmented layout (spmv_kind 2)
@@ -782,23 +780,13 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 || KIND == 3 ? 2 : 1) pe
                 if (sum.flag) { status = PERKS_ERR_BREAKDOWN; break; }
                 const double alpha = sum.ratio;
                 double rn_p = 0.0;
-                for (int i0 = sl.r0 + tid; i0 < sl.r1; i0 += kCgRows64 * kCgThreads) {
-                    double pv[kCgRows64], xv[kCgRows64], qv[kCgRows64], rv[kCgRows64];
-#pragma unroll
-                    for (int u = 0; u < kCgRows64; ++u) {
-                        const int i = i0 + u * kCgThreads;
-                        if (i < sl.r1) { pv[u] = p[i]; xv[u] = X(i); qv[u] = Q(i); rv[u] = R(i); }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kCgRows64; ++u) {
-                        const int i = i0 + u * kCgThreads;
-                        if (i < sl.r1) {
-                            X(i) = fma(alpha, pv[u], xv[u]);
-                            const double ri = fma(-alpha, qv[u], rv[u]);
-                            R(i) = ri;
-                            rn_p += ri * ri;
-                        }
-                    }
+                for (int i = sl.r0 + tid; i < sl.r1; i += kCgThreads) {
+                    // every load before the first store, which the compiler cannot move them across
+                    const double pv = p[i], xv = X(i), qv = Q(i), rv = R(i);
+                    X(i) = fma(alpha, pv, xv);
+                    const double ri = fma(-alpha, qv, rv);
+                    R(i) = ri;
+                    rn_p += ri * ri;
                 }
                 // C: beta; p = r + beta p
                 if (!gsum(rn_p, sum, [&](double t, double &ratio, int &flag) { ratio = t / rr; flag = t <= tol2; }))
@@ -810,19 +798,7 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 || KIND == 3 ? 2 : 1) pe
                     a.trace[3 * it + 1] = beta;
                     a.trace[3 * it + 2] = rr_new;
                 }
-                for (int i0 = sl.r0 + tid; i0 < sl.r1; i0 += kCgRows64 * kCgThreads) {
-                    double pv[kCgRows64], rv[kCgRows64];
-#pragma unroll
-                    for (int u = 0; u < kCgRows64; ++u) {
-                        const int i = i0 + u * kCgThreads;
-                        if (i < sl.r1) { pv[u] = p[i]; rv[u] = R(i); }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kCgRows64; ++u) {
-                        const int i = i0 + u * kCgThreads;
-                        if (i < sl.r1) p[i] = fma(beta, pv[u], rv[u]);
-                    }
-                }
+                for (int i = sl.r0 + tid; i < sl.r1; i += kCgThreads) p[i] = fma(beta, p[i], R(i));
                 rr = rr_new;
                 ++it;
                 if (!cg_sync(a, epoch)) return;
@@ -877,43 +853,20 @@ __global__ void __launch_bounds__(kCgThreads, KIND == 0 || KIND == 3 ? 2 : 1) pe
                 if (sum.flag) { status = PERKS_ERR_BREAKDOWN; break; }
                 const float alpha = (float)sum.ratio;
                 double rn_p = 0.0;
-                for (int i0 = sl.r0 + tid; i0 < sl.r1; i0 += kCgRows32 * kCgThreads) {
-                    float pv[kCgRows32], dv[kCgRows32], qv[kCgRows32], rv[kCgRows32];
-#pragma unroll
-                    for (int u = 0; u < kCgRows32; ++u) {
-                        const int i = i0 + u * kCgThreads;
-                        if (i < sl.r1) { pv[u] = p32[i]; dv[u] = D32(i); qv[u] = Q32(i); rv[u] = R32(i); }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kCgRows32; ++u) {
-                        const int i = i0 + u * kCgThreads;
-                        if (i < sl.r1) {
-                            D32(i) = fmaf(alpha, pv[u], dv[u]);
-                            const float ri = fmaf(-alpha, qv[u], rv[u]);
-                            R32(i) = ri;
-                            const double rd = (double)ri;
-                            rn_p = fma(rd, rd, rn_p);
-                        }
-                    }
+                for (int i = sl.r0 + tid; i < sl.r1; i += kCgThreads) {
+                    const float pv = p32[i], dv = D32(i), qv = Q32(i), rv = R32(i);
+                    D32(i) = fmaf(alpha, pv, dv);
+                    const float ri = fmaf(-alpha, qv, rv);
+                    R32(i) = ri;
+                    const double rd = (double)ri;
+                    rn_p = fma(rd, rd, rn_p);
                 }
                 if (!gsum(rn_p, sum, [&](double t, double &ratio, int &flag) { ratio = t / irr; flag = t <= itol2; }))
                     return;
                 const double rr_new = sum.total;
                 const float beta = (float)sum.ratio;
                 const bool inner_done = sum.flag != 0;
-                for (int i0 = sl.r0 + tid; i0 < sl.r1; i0 += kCgRows32 * kCgThreads) {
-                    float pv[kCgRows32], rv[kCgRows32];
-#pragma unroll
-                    for (int u = 0; u < kCgRows32; ++u) {
-                        const int i = i0 + u * kCgThreads;
-                        if (i < sl.r1) { pv[u] = p32[i]; rv[u] = R32(i); }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kCgRows32; ++u) {
-                        const int i = i0 + u * kCgThreads;
-                        if (i < sl.r1) p32[i] = fmaf(beta, pv[u], rv[u]);
-                    }
-                }
+                for (int i = sl.r0 + tid; i < sl.r1; i += kCgThreads) p32[i] = fmaf(beta, p32[i], R32(i));
                 irr = rr_new;
                 ++it;
                 if (!cg_sync(a, epoch)) return;
