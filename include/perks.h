@@ -156,13 +156,19 @@ typedef struct {
                                            the 16-byte-vector kernel; reserved[1] = planes per
                                            block barrier of the vector kernel (2 or 4, 0 =
                                            automatic); STRIP: time steps per sweep (1, 2 or 4
-                                           where compiled, 0 = automatic), tiles_z the runs of
-                                           rows (0 = automatic); reserved[2] = kernel body
+                                           where compiled, 0 = automatic); PATCH: steps per
+                                           exchange (4 for radius 1, 2 for radius 2, 0 =
+                                           automatic); reserved[2] = kernel body
                                            (PERKS_KERNEL_AUTO / _RESIDENT / _STREAMING / _STRIP /
-                                           _SLAB / _PATCH;
-                                           AUTO in a plan means STREAMING, AUTO with no plan
-                                           picks the resident tile when every tile fits in shared
-                                           memory, the column strips for other 2-D domains);
+                                           _SLAB / _PATCH).  AUTO in a plan means STREAMING; for
+                                           no plan see below.  Tiles of STRIP: tiles_x strips
+                                           across (their number follows from the steps per
+                                           sweep), tiles_z runs of rows; PATCH: tiles_x x tiles_z
+                                           patches; SLAB: tiles_x x tiles_y columns, of 32, 16 or
+                                           8 lanes per row, tiles_z parts of each (1 where the
+                                           planner cuts the columns into equal shares).  What the
+                                           kernel cannot take is UNSUPPORTED.  A traced run and a
+                                           per-step run leave such a plan aside;
                                            reserved[3] = threads per block (0 = automatic):
                                            256 or 512 for the resident tile kernel; 256 picks the
                                            plane-streaming kernel's two-blocks-per-SM
@@ -178,6 +184,15 @@ typedef struct {
                                            next); tiles_z is ignored.  0 = one tile per block */
 } perks_stencil_plan;
 
+/* The persistent kernel without a plan: 2d5pt, 2ds9pt, 2d9pt and 2d25pt run
+ * patches up to sizes measured per type and shape, column strips beyond; 3d7pt,
+ * 3d13pt, 3d27pt and poisson run slabs where those were measured to be faster
+ * (fp32 and bf16 that do not fit on chip: always), otherwise the resident tile
+ * (3d7pt whose tiles fit in shared memory) or plane streaming, fp64 3d7pt of
+ * 4 M cells and more with 256 threads in balanced shares; everything else plane
+ * streaming.  A domain that neither the resident tile nor plane streaming can
+ * host is UNSUPPORTED. */
+
 /* What a run did; filled by perks_stencil_run when asked. */
 typedef struct {
     int64_t steps;
@@ -192,8 +207,10 @@ typedef struct {
     int64_t halo_cells_per_step;        /* halo cells written + read per step (H) */
     double algorithmic_bytes;           /* S (2 N D_uncache + 2 D_cache) + S N H for the whole run */
     int32_t kernel;                     /* PERKS_KERNEL_*: which kernel body runs */
-    int32_t planes_per_sync;            /* column strips: time steps per sweep; resident tile: planes a thread computes between two block
-                                           barriers; plane streaming: planes per block barrier */
+    int32_t planes_per_sync;            /* column strips: time steps per sweep; patches: steps per
+                                           exchange; resident tile: planes a thread computes
+                                           between two block barriers; plane streaming: planes
+                                           per block barrier */
 } perks_run_stats;
 
 /* Kernel bodies of a stencil run (perks_run_stats.kernel, perks_stencil_plan.reserved[2]). */
@@ -207,7 +224,8 @@ enum {
     PERKS_KERNEL_PER_STEP = 3,   /* one launch per step (PERKS_PER_STEP) */
     PERKS_KERNEL_STRIP = 4,      /* column strips (2-D: 2d5pt, 2ds9pt, 2d9pt, 2d25pt): every warp streams a strip of
                                     rows through register windows, several time steps per sweep; a sweep, not a
-                                    step, ends at the grid barrier.  Not used while a step trace is on */
+                                    step, ends at the grid barrier.  Steps left over from whole sweeps may run
+                                    as one-step sweeps of a second launch.  Not used while a step trace is on */
     PERKS_KERNEL_SLAB = 5,       /* slab streaming (3-D: 3d7pt, 3d13pt, 3d27pt, poisson; any row length): rows of
                                     neighbouring lanes, several rows per thread, planes through a shared-memory
                                     ring, no caches.  Not used while a step trace is on */
@@ -241,8 +259,8 @@ perks_status perks_stencil_get_trace(perks_stencil *st, uint64_t *host, int64_t 
  * `probe_steps` (>= 2) and 3 `probe_steps` steps, so that the per-run launch,
  * prologue and epilogue cancel -- the resident-tile kernel with 256 and 512
  * threads and 1 and 2 rows per thread where the domain fits, the column strips
- * with each compiled number of steps per sweep (2-D), and the model's
- * own tiling and up to six tilings ranked by tz * (1 + halo fraction), each
+ * with each compiled number of steps per sweep and the patches (2-D) or the
+ * slabs (3-D) unless a step trace is on, and the model's own tiling and up to six tilings ranked by tz * (1 + halo fraction), each
  * with registers + shared memory, shared memory only, no cache, or no cache
  * in balanced shares (perks_stencil_plan.balanced), and with 2 or 4 planes
  * per block barrier -- restores the field, installs the fastest plan (as

@@ -371,9 +371,11 @@ class Stencil:
         resident-tile kernel (``tiles`` and ``threads`` 256/512 apply to
         it, 0 = automatic), KERNEL_STRIP the column-strip kernel of 2-D
         domains (``planes_per_barrier`` = time steps per sweep, ``tiles[2]``
-        = runs of rows), KERNEL_SLAB the slab-streaming kernel of 3-D domains,
-        KERNEL_PATCH the patch kernel of small 2-D domains
-        (``planes_per_barrier`` = steps per exchange),
+        = runs of rows), KERNEL_SLAB the slab-streaming kernel of 3-D domains
+        (``tiles`` = columns across x and y, parts of each), KERNEL_PATCH the
+        patch kernel of small 2-D domains (``planes_per_barrier`` = steps per
+        exchange, ``tiles[0]`` x ``tiles[2]`` patches); a traced or per-step
+        run leaves these three aside,
         KERNEL_STREAMING / KERNEL_AUTO the plane-streaming
         kernel; ``rows`` (1 or 2, 0 = automatic) is the resident kernel's
         rows per thread; ``balanced`` (cache-free plane streaming only) cuts
@@ -664,12 +666,12 @@ class Poisson:
         self.ctx.check(self._lib.perks_poisson_scale_guess(self.handle, bp, xp, _stream(stream)))
 
     def set_block_threads(self, threads: int):
-        """512 (one block per SM, default) or 256 threads per problem's block."""
+        """512 (default) or 256 threads per block, for several rows per pass."""
         self.ctx.check(self._lib.perks_poisson_set_block_threads(self.handle, int(threads)))
 
     def set_rows_per_pass(self, rows: int):
-        """4 (default: 128 registers, one 512-thread block per SM) or 1 (64
-        registers, two blocks per SM)."""
+        """1 (default: 64 registers, two blocks per SM) or 4 (128 registers, one
+        512-thread block per SM)."""
         self.ctx.check(self._lib.perks_poisson_set_rows_per_pass(self.handle, int(rows)))
 
     def set_group(self, blocks: int):

@@ -694,7 +694,7 @@ perks_status plan_strips(perks_batch *b, int rows) {
     if (items.size() <= (size_t)nwarps) {
         // A warp per item at most: neighbouring items, one shape's after the other's, to the warps of a block, the same
         // number in every block.  An SM then runs two or three shapes' code, not four's (40 fp32 domains of 244 x 333, four
-        // shapes, 9.4 us a step, 14.9 with an SM's items from all over the batch), and its two blocks, half the batch apart,
+        // shapes, 9.1 us a step, 14.9 with an SM's items from all over the batch), and its two blocks, half the batch apart,
         // shapes that differ in what bounds them (the 64-domain workload 2.5 % faster than with one shape's).  (A heap of
         // idle warps, as below, does much the same, at 60 ns an item: as long as several steps of a small batch.)
         std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->shape[items[x].dom] < b->shape[items[y].dom]; });

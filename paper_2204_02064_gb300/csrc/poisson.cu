@@ -379,11 +379,11 @@ __global__ void __launch_bounds__(NT, MINB) perks_poisson_cg_kernel(const __grid
 //     barriers: p of the two rows next to a block's own is updated by the
 //     block itself, from the neighbours' r of those rows, which travels with
 //     the <r, r> exchange.
-//   * r stays in shared memory where a block's share fits, and the automatic
-//     group size (effective_group) makes it fit.
-// 64 problems of 512^2, 24 iterations: 11.8 ms with the kernel above, 10.5
+//   * r stays in shared memory where a block's share fits; run_group prefers
+//     group sizes that make it fit.
+// 64 problems of 512^2, 24 iterations: 11.8 ms with the kernel above, 10.4
 // here (the FP64 pipe's time is 6.7 ms); 16 problems of 83 x 368, 2.0 -> 0.5
-// ms; 202 problems of 64 x 81 to 1e-10, 61 -> 27 ms.
+// ms; 202 problems of 64 x 81 to 1e-8, 61 -> 28 ms.
 template <int NT, bool GROUP>
 __global__ void __launch_bounds__(NT, 2) perks_poisson_run_kernel(const __grid_constant__ PoissonArgs a) {
     extern __shared__ __align__(16) double poi_smem[];

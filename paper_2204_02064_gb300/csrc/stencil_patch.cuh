@@ -11,14 +11,17 @@
 // is overwritten in exchange e + 2, and a block gets there only after its
 // neighbours have raised flag e + 1, which they do after reading rim e.
 //
-// Why: a small domain's step is the exchange, not the arithmetic -- 2d5pt
-// fp64 256^2 spends 0.5 us of the FP64 pipe per step of 3.9 us in the
-// resident-tile kernel, which exchanges halos after every step through a
-// grid-wide barrier; here it takes 2.4 us (fp32 64^2: 1.0, 0.98 M cells of fp64
-// 12).  K = 4 for radius 1, 2 for radius 2: half of that was slower or equal
-// at every size (256^2 fp64 2d5pt K = 2 3.4 us; 2d25pt K = 1 7.5 against 6.7).
-// Bound: the exchange (a write, a flag and a read through L2, about 2.5 us)
-// for small tiles, the FP64 pipe and the recomputed rim for large fp64 ones.
+// Why: in the resident-tile kernel, which exchanges halos after every step
+// through a grid-wide barrier, a small domain's step is mostly that exchange:
+// 2d5pt fp64 256^2 spends 0.5 us of the FP64 pipe per step of 3.9 us.  Here one
+// exchange (a write, a flag and a read through L2, about 2.5 us) serves four
+// steps, and a step takes 2.4 us (fp32 64^2: 1.0, 0.98 M cells of fp64 12): a
+// quarter of it the exchange, a third the FP64 work with the recomputed rim,
+// the rest short passes (some 780 cells for 512 threads) and a block barrier
+// per step.  K = 4 for radius 1, 2 for radius 2: half of that was slower or
+// equal at every size (256^2 fp64 2d5pt K = 2 3.4 us; 2d25pt K = 1 7.5 against
+// 6.7).  Bound: latency for small tiles, the FP64 pipe and the recomputed rim
+// for large fp64 ones.
 //
 // Cells add their terms in table order with one fma chain from 0 and are
 // rounded to the storage type after every step (fp32 / bf16: the same bits as

@@ -36,7 +36,8 @@
 // walk running pointers: 3d27pt 251 x 246 x 233 took 42 us, 3d13pt bf16 384^3
 // 90 (now 56), with a branch per row and the addresses formed anew.
 // Bound: HBM (8 B per cell and step in fp32) for stars of large domains, the
-// issue slots for boxes (60 %, FMA pipe 43 %), the FP64 pipe for fp64.
+// latency of shared loads and block barriers for boxes (issue slots 52 %, FMA
+// pipe 38 %), the FP64 pipe for fp64.
 #pragma once
 
 #include "stencil_vec.cuh"

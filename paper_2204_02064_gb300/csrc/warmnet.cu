@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(kWgThreads, 2) wgrad_mid_kernel(const S *__res
     }
     // the two streams' sums, through shared memory, into the block's row
     float *row = part + (long long)blockIdx.x * nparams;
-    float *s_o = smem;                              // 96 threads x 105 sums
+    float *s_o = smem;                              // 96 threads x 104 sums
     __syncthreads();
     if (stream == 1) {
         float *o = s_o + (warp - 3) * 32 + lane;
