@@ -187,7 +187,7 @@ typedef struct {
 /* The persistent kernel without a plan: 2d5pt, 2ds9pt, 2d9pt and 2d25pt run
  * patches up to sizes measured per type and shape, column strips beyond; 3d7pt,
  * 3d13pt, 3d27pt and poisson run slabs where those were measured to be faster
- * (fp32 and bf16 that do not fit on chip: always), otherwise the resident tile
+ * (fp32 and bf16 always where there is no resident tile), otherwise the resident tile
  * (3d7pt whose tiles fit in shared memory) or plane streaming, fp64 3d7pt of
  * 4 M cells and more with 256 threads in balanced shares; everything else plane
  * streaming.  A domain that neither the resident tile nor plane streaming can

@@ -190,7 +190,7 @@ __global__ void near_rows(const int *__restrict__ rowptr, const int *__restrict_
     int m = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i + 1 < n; i += (long long)gridDim.x * blockDim.x) {
         const int a = rowptr[i], b = rowptr[i + 1], c = rowptr[i + 2];
-        if (a < b && b < c) m += abs(col[(a + b) / 2] - col[(b + c) / 2]) <= 8;
+        if (a < b && b < c) m += abs(col[a + (b - a) / 2] - col[b + (c - b) / 2]) <= 8;
     }
     m = __reduce_add_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0 && m > 0) atomicAdd(near, m);
@@ -768,6 +768,12 @@ extern "C" perks_status perks_csr_create(perks_context *ctx, int32_t n, int64_t 
     }
     int ov[2] = {0, 0};
     OPCUDA(cudaMemcpy(ov, overflow, sizeof(ov), cudaMemcpyDeviceToHost));
+    if (ov[0]) {
+        cudaFree(overflow);
+        free_op(op); delete op;
+        return fail(ctx, PERKS_ERR_UNSUPPORTED, "csr_create: matrix too large (more than %d tiles per block)",
+                    kCgMaxTiles);
+    }
     // One lane per row or eight (spmv_rows_short): rows of 16 nonzeros at most, 15.5 on average; a product by itself 12.5,
     // or 15.5 where neighbouring rows have neighbouring columns.
     op->short_rows = op->short_spmv = ov[1] <= kShortRow && (double)nnz <= 15.5 * n;
@@ -779,11 +785,6 @@ extern "C" perks_status perks_csr_create(perks_context *ctx, int32_t n, int64_t 
         op->short_spmv = 2LL * ov[1] > n;
     }
     cudaFree(overflow);
-    if (ov[0]) {
-        free_op(op); delete op;
-        return fail(ctx, PERKS_ERR_UNSUPPORTED, "csr_create: matrix too large (more than %d tiles per block)",
-                    kCgMaxTiles);
-    }
     OPCHK(dalloc(ctx, &op->b, (size_t)n));
     OPCHK(dalloc(ctx, &op->x, (size_t)n));
     OPCHK(dalloc(ctx, &op->r, (size_t)n));
